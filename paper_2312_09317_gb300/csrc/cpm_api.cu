@@ -26,6 +26,7 @@ struct cpm_handle {
     uint32_t s = 1, C = 1, sd = 1, k = 1, per_mcs = 1, per_sub_mcs = 1;
     uint32_t nbx = 1, nby = 1, nbz = 1, n_active = 0;
     bool perim = false, act = false;
+    uint32_t uni = 0;  // the type of every cell when they all share one, else 0
     // device state
     int32_t *lat = nullptr;        // lattice words: ids, with the Act stamps in the high byte when act
     int32_t *stage = nullptr;      // staging for host reads and loads of packed words (lazily allocated)
@@ -90,6 +91,8 @@ int fail(cpm_handle *h, int code, const char *fmt, ...)
             return fail((h), e_ == cudaErrorMemoryAllocation ? CPM_E_NOMEM : CPM_E_CUDA, "%s: %s", \
                         #expr, cudaGetErrorString(e_));                                          \
     } while (0)
+
+constexpr uint64_t kL2LatticeBytes = 80u << 20;
 
 uint32_t ipow(uint32_t b, int e)
 {
@@ -254,19 +257,14 @@ int pers_step(cpm_handle *h)
     return CPM_OK;
 }
 
-int run_subpass(cpm_handle *h)
+// What all rounds of a lattice share, and its buffers.
+RoundArgs round_args(const cpm_handle *h)
 {
-    if (h->act && h->sp == 0 && h->t % 64 == 0) {
-        CUDA_TRY(h, launch_clamp_stamps(h->lat, h->n_sites, (uint32_t)h->t, h->stream));
-        h->launches += 1;
-    }
-    const uint32_t col = colour_of(h, h->t, h->sp);
     RoundArgs a;
     memset(&a, 0, sizeof a);
-    a.lat = h->lat;
     a.packed = h->act ? 1u : 0u;
-    a.stream_loads = h->act && h->cfg.a >= 8 ? 1u : 0u;
-    a.pdl = 1;  // each round overlaps its set-up with the previous round's tail
+    // (a lattice that fits L2 beside its tallies must stay there, not be the first to go)
+    a.stream_loads = h->act && h->cfg.a >= 8 && 4 * h->n_sites > kL2LatticeBytes ? 1u : 0u;
     a.cell_type = h->cell_type;
     a.thr = h->thr;
     a.ln_tab = h->ln_tab;
@@ -276,37 +274,68 @@ int run_subpass(cpm_handle *h)
     a.nx = h->cfg.nx; a.ny = h->cfg.ny; a.nz = h->cfg.nz;
     a.s = h->s; a.c = h->cfg.c; a.sd = h->sd;
     a.nbx = h->nbx; a.nby = h->nby;
-    a.nax = h->nbx / h->cfg.c; a.nay = h->nby / h->cfg.c;
+    a.nax = h->nbx / h->cfg.c; a.nay = h->nby / h->cfg.c; a.naz = h->dim == 3 ? h->nbz / h->cfg.c : 1;
     a.n_active = h->n_active;
-    a.cx = col % h->cfg.c;
-    a.cy = (col / h->cfg.c) % h->cfg.c;
-    a.cz = col / (h->cfg.c * h->cfg.c);
-    a.t = (uint32_t)h->t;
-    a.sp = (uint32_t)h->sp;
     a.key0 = (uint32_t)h->cfg.seed;
     a.key1 = (uint32_t)(h->cfg.seed >> 32);
-    a.tp = h->tp;
     a.chem = h->chem;
     a.pers_dir = h->pers ? h->pers_dir : nullptr;
-    pick_bricks(h->dim, a.nax, a.nay, a);
-    for (uint32_t r = 0; r < h->k; r++) {
-        const int cur = (int)(h->g & 1);
-        a.r = r;
-        a.Vc = V_buf(h, cur);
-        a.Ac = A_buf(h, cur);
-        a.Vn = V_buf(h, cur ^ 1);
-        a.An = A_buf(h, cur ^ 1);
-        a.pend_prev = h->pend + (size_t)(cur ^ 1) * h->n_active;
-        a.pend_cur = h->pend + (size_t)cur * h->n_active;
-        a.flag_prev = h->flags + (size_t)(cur ^ 1) * h->n_active;
-        a.flag_cur = h->flags + (size_t)cur * h->n_active;
+    a.uni = h->uni;
+    a.tp = h->tp;
+    fill_round_constants(a, h->cfg.temperature);
+    return a;
+}
+
+LatticeBufs lattice_bufs(cpm_handle *h)
+{
+    LatticeBufs l{};
+    l.lat = h->lat;
+    for (int p = 0; p < 2; p++) {
+        l.V[p] = V_buf(h, p);
+        l.A[p] = A_buf(h, p);
+        l.pend[p] = h->pend + (size_t)p * h->n_active;
+        l.flag[p] = h->flags + (size_t)p * h->n_active;
         if (h->csum) {
-            a.Sc = S_buf(h, cur);
-            a.Sn = S_buf(h, cur ^ 1);
-            a.tpend_prev = h->tpend + (size_t)(cur ^ 1) * h->n_active;
-            a.tpend_cur = h->tpend + (size_t)cur * h->n_active;
+            l.S[p] = S_buf(h, p);
+            l.tpend[p] = h->tpend + (size_t)p * h->n_active;
         }
-        CUDA_TRY(h, launch_round(h->dim, h->perim, h->act, a, h->stream));
+    }
+    return l;
+}
+
+// What follows the last round of an MCS (h->t already counts it).
+int end_of_mcs(cpm_handle *h)
+{
+    if (h->csum) {
+        // every centroid back into [0, n): the same shift in both buffers
+        const int cur = (int)(h->g & 1);
+        CUDA_TRY(h, launch_track_rewrap(h->dim, h->cfg.nx, h->cfg.ny, h->cfg.nz, h->n_cells, V_buf(h, cur),
+                                        S_buf(h, cur), S_buf(h, cur ^ 1), h->stream));
+        h->launches += 1;
+    }
+    return h->pers ? pers_step(h) : CPM_OK;
+}
+
+int run_subpass(cpm_handle *h)
+{
+    if (h->act && h->sp == 0 && h->t % 64 == 0) {
+        CUDA_TRY(h, launch_clamp_stamps(h->lat, h->n_sites, (uint32_t)h->t, h->stream));
+        h->launches += 1;
+    }
+    RoundArgs a = round_args(h);
+    a.pdl = 1;  // each round overlaps its set-up with the previous round's tail
+    pick_bricks(h->dim, a);
+    const LatticeBufs bufs = lattice_bufs(h);
+    const uint32_t col = colour_of(h, h->t, h->sp);
+    RoundPos pos{};
+    pos.cx = col % h->cfg.c;
+    pos.cy = (col / h->cfg.c) % h->cfg.c;
+    pos.cz = col / (h->cfg.c * h->cfg.c);
+    pos.t = (uint32_t)h->t;
+    pos.sp = (uint32_t)h->sp;
+    for (uint32_t r = 0; r < h->k; r++) {
+        pos.r = r;
+        CUDA_TRY(h, launch_round(h->dim, h->perim, h->act, a, round_bufs(bufs, (uint32_t)(h->g & 1)), pos, h->stream));
         h->launches += 1;
         h->g += 1;
         h->attempts += h->n_active;
@@ -314,14 +343,7 @@ int run_subpass(cpm_handle *h)
     if (++h->sp == (int32_t)h->per_mcs) {
         h->sp = 0;
         h->t += 1;
-        if (h->csum) {
-            // every centroid back into [0, n): the same shift in both buffers
-            const int cur = (int)(h->g & 1);
-            CUDA_TRY(h, launch_track_rewrap(h->dim, h->cfg.nx, h->cfg.ny, h->cfg.nz, h->n_cells, V_buf(h, cur),
-                                            S_buf(h, cur), S_buf(h, cur ^ 1), h->stream));
-            h->launches += 1;
-        }
-        if (h->pers) return pers_step(h);
+        return end_of_mcs(h);
     }
     return CPM_OK;
 }
@@ -591,6 +613,9 @@ int create_impl(cpm_handle *h, const cpm_config *c, TableCache *cache = nullptr)
     h->sp = 0;
     h->g = 0;
     if (c->n_cells >= 1) {
+        h->uni = c->cell_type[1];
+        for (int32_t i = 2; i <= c->n_cells && h->uni; i++)
+            if (c->cell_type[i] != h->uni) h->uni = 0;
         h->v_ref = c->v_target[c->cell_type[1]];
         h->a_ref = c->a_target[c->cell_type[1]];
     }
@@ -633,10 +658,7 @@ int create_impl(cpm_handle *h, const cpm_config *c, TableCache *cache = nullptr)
     {
         std::vector<int32_t> ln, ex;
         ln_expq_tables(ln, ex);
-        for (int a = 0; a < CPM_MAX_TYPES; a++) {
-            const int m = c->max_act[a] < 0 ? 0 : (c->max_act[a] > 127 ? 127 : c->max_act[a]);
-            h->tp.gm_max[a] = m > 0 ? ex[ln[m] >> 6] : 0;
-        }
+        fill_act_bounds(h->tp, ln.data(), ex.data());
     }
     rc = reset_tallies(h);
     if (rc) return rc;
@@ -975,13 +997,14 @@ struct cpm_batch {
     uint32_t n_clamp_items = 0;
     uint32_t brick[3] = {8, 4, 4};       // active blocks per CTA (x, y, z)
     BatchLattice *d_lats = nullptr;
-    int2 *d_items = nullptr;
+    int4 *d_items = nullptr;              // round items: member, brick x y z
     int2 *d_clamp = nullptr;
     ObserveItem *d_obs = nullptr;        // observation items, built on first use
     TableCache *tables = nullptr;        // LN / EXPQ / THR shared by the members
     int64_t obs_max_sites = 0;
     int64_t obs_rows = 0;
     int32_t obs_max_cells = 0;
+    uint8_t *d_colours = nullptr;        // BatchLattice::colours of every member
     double *traj = nullptr;              // centroid tracks of cpm_batch_summarize
     size_t traj_cap = 0;
     cudaGraphExec_t graph = nullptr;     // one MCS of every member
@@ -1024,6 +1047,7 @@ void batch_free(cpm_batch *b)
     delete b->tables;
     b->tables = nullptr;
     cudaFree(b->d_lats);
+    cudaFree(b->d_colours);
     cudaFree(b->d_items);
     cudaFree(b->d_clamp);
     cudaFree(b->d_obs);
@@ -1041,20 +1065,24 @@ uint32_t batch_threads(const cpm_batch *b) { return b->brick[0] * b->brick[1] * 
 // rounds per MCS (descending), and the Act clamp items (member, 65,536 sites)
 int batch_build_items(cpm_batch *b)
 {
-    std::vector<int2> items;
+    std::vector<int4> items;
     b->items_upto.assign(1, 0);
-    const uint32_t bz = b->dim == 3 ? b->brick[2] : 1;
+    const auto log2 = [](uint32_t n) {
+        uint32_t l = 0;
+        while ((1u << l) < n) l++;
+        return l;
+    };
+    const uint32_t lx = log2(b->brick[0]), ly = log2(b->brick[1]), lz = b->dim == 3 ? log2(b->brick[2]) : 0;
     for (uint32_t l : b->order) {
-        const cpm_handle *h = b->hs[l];
-        const uint32_t nax = h->nbx / h->cfg.c, nay = h->nby / h->cfg.c;
-        const uint32_t naz = h->n_active / (nax * nay);
-        const uint32_t nb = ((nax + b->brick[0] - 1) / b->brick[0]) * ((nay + b->brick[1] - 1) / b->brick[1]) *
-                            ((naz + bz - 1) / bz);
-        for (uint32_t c = 0; c < nb; c++) items.push_back(make_int2((int)l, (int)c));
+        RoundArgs &a = b->lats[l].base;
+        a.brick_lx = lx;
+        a.brick_ly = ly;
+        a.brick_lz = lz;
+        for (uint32_t z = 0; z < a.naz; z += 1u << lz)
+            for (uint32_t y = 0; y < a.nay; y += 1u << ly)
+                for (uint32_t x = 0; x < a.nax; x += 1u << lx)
+                    items.push_back(make_int4((int)l, (int)(x >> lx), (int)(y >> ly), (int)(z >> lz)));
         b->items_upto.push_back((uint32_t)items.size());
-        b->lats[l].base.brick_x = b->brick[0];
-        b->lats[l].base.brick_y = b->brick[1];
-        b->lats[l].base.brick_z = bz;
     }
     std::vector<int2> clamp;
     for (size_t l = 0; l < b->hs.size(); l++) {
@@ -1081,10 +1109,10 @@ int batch_build_items(cpm_batch *b)
     cudaError_t e = cudaMalloc(&b->d_upto_q, sizeof(uint32_t) * std::max<size_t>(upto_q.size(), 1));
     if (e == cudaSuccess)
         e = cudaMemcpy(b->d_upto_q, upto_q.data(), sizeof(uint32_t) * upto_q.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int2) * std::max<size_t>(items.size(), 1));
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int4) * std::max<size_t>(items.size(), 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->d_clamp, sizeof(int2) * std::max<size_t>(clamp.size(), 1));
     if (e == cudaSuccess)
-        e = cudaMemcpy(b->d_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(b->d_items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !clamp.empty())
         e = cudaMemcpy(b->d_clamp, clamp.data(), sizeof(int2) * clamp.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
@@ -1101,8 +1129,9 @@ int batch_build_graph(cpm_batch *b)
     batch_drop_graph(b);
     cudaError_t e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
-    int64_t n = 0;
-    if (b->act) {
+    int64_t n = 1;
+    e = launch_batch_colours(b->d_lats, (uint32_t)b->lats.size(), b->capture_stream);
+    if (b->act && e == cudaSuccess) {
         e = launch_batch_clamp(b->d_lats, b->d_clamp, b->n_clamp_items, b->capture_stream);
         n++;
     }
@@ -1111,7 +1140,7 @@ int batch_build_graph(cpm_batch *b)
     for (uint32_t q = 0; q < r_max && e == cudaSuccess; q++) {
         while (active > 0 && b->lats[b->order[active - 1]].R <= q) active--;
         e = launch_batch_round(b->dim, b->perim, b->act, b->track, b->d_lats, b->d_items, b->items_upto[active], q,
-                               batch_threads(b), b->capture_stream);
+                               batch_threads(b), q > 0, b->capture_stream);
         n++;
     }
     if (e == cudaSuccess) {
@@ -1204,31 +1233,8 @@ int cpm_batch_create(const cpm_config *cfgs, int32_t n, void *cuda_stream, cpm_b
     for (cpm_handle *h : b->hs) {
         BatchLattice L;
         memset(&L, 0, sizeof L);
-        RoundArgs &a = L.base;
-        a.lat = h->lat;
-        a.packed = h->act ? 1u : 0u;
-        a.stream_loads = h->act && h->cfg.a >= 8 ? 1u : 0u;
-        a.cell_type = h->cell_type;
-        a.thr = h->thr;
-        a.ln_tab = h->ln_tab;
-        a.expq = h->expq;
-        a.accepts = h->counters;
-        a.L = h->L;
-        a.nx = h->cfg.nx; a.ny = h->cfg.ny; a.nz = h->cfg.nz;
-        a.s = h->s; a.c = h->cfg.c; a.sd = h->sd;
-        a.nbx = h->nbx; a.nby = h->nby;
-        a.nax = h->nbx / h->cfg.c; a.nay = h->nby / h->cfg.c;
-        a.n_active = h->n_active;
-        a.key0 = (uint32_t)h->cfg.seed;
-        a.key1 = (uint32_t)(h->cfg.seed >> 32);
-        a.tp = h->tp;
-        a.chem = h->chem;
-        for (int p = 0; p < 2; p++) {
-            L.V[p] = V_buf(h, p);
-            L.A[p] = A_buf(h, p);
-            L.pend[p] = h->pend + (size_t)p * h->n_active;
-            L.flag[p] = h->flags + (size_t)p * h->n_active;
-        }
+        L.base = round_args(h);
+        L.bufs = lattice_bufs(h);
         L.k = h->k;
         L.C = h->C;
         L.R = h->per_sub_mcs * h->k;
@@ -1239,12 +1245,20 @@ int cpm_batch_create(const cpm_config *cfgs, int32_t n, void *cuda_stream, cpm_b
     for (int32_t i = 0; i < n; i++) b->order[i] = (uint32_t)i;
     std::stable_sort(b->order.begin(), b->order.end(),
                      [&](uint32_t x, uint32_t y) { return b->lats[x].R > b->lats[y].R; });
+    size_t n_colours = 0;
+    for (const BatchLattice &L : b->lats) n_colours += L.R / L.k;
     cudaError_t e = cudaMalloc(&b->d_lats, sizeof(BatchLattice) * b->lats.size());
+    if (e == cudaSuccess) e = cudaMalloc(&b->d_colours, n_colours);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
         batch_free(b);
         delete b;
         return bfail(nullptr, e == cudaErrorMemoryAllocation ? CPM_E_NOMEM : CPM_E_CUDA, cudaGetErrorString(e));
+    }
+    n_colours = 0;
+    for (BatchLattice &L : b->lats) {
+        L.colours = b->d_colours + n_colours;
+        n_colours += L.R / L.k;
     }
     int rc = batch_build_items(b);
     if (rc) {
@@ -1361,10 +1375,7 @@ int cpm_batch_track_centroids(cpm_batch *b, int32_t on)
         cpm_handle *h = b->hs[l];
         if (int rc = cpm_track_centroids(h, on))
             return bfail(b, rc, "lattice " + std::to_string(l) + ": " + cpm_last_error(h));
-        for (int p = 0; p < 2; p++) {
-            b->lats[l].S[p] = on ? S_buf(h, p) : nullptr;
-            b->lats[l].tpend[p] = on ? h->tpend + (size_t)p * h->n_active : nullptr;
-        }
+        b->lats[l].bufs = lattice_bufs(h);
     }
     b->track = on != 0;
     b->descriptors_dirty = true;

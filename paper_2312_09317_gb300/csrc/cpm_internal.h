@@ -74,6 +74,10 @@ __host__ __device__ __forceinline__ int32_t pack_word(int32_t id, uint32_t stamp
 __host__ __device__ __forceinline__ int64_t track_image_shift(int64_t x, int64_t S, int64_t V, int64_t n)
 {
     const int64_t num = 2 * (S - x * V) + n * V, den = 2 * n * V;
+    // a cell within one lattice length of its site, the usual case, needs no 64-bit division
+    if (num >= 0 && num < den) return 0;
+    if (num >= den && num - den < den) return 1;
+    if (num < 0 && num + den >= 0) return -1;
     int64_t q = num / den;
     if (num % den != 0 && num < 0) q -= 1;
     return q;
@@ -89,21 +93,38 @@ struct TypeParams {
     int32_t lambda_chem[kMaxTypes], lambda_pers[kMaxTypes];  // motility weights, scaled
     double inv_len[4];                                        // 1 / sqrt(k), k = |d|^2 of a copy direction
     int32_t gm_max[kMaxTypes];  // EXPQ[LN[Max_act] >> 6]: the largest Act geometric mean a type's site can have
+    // bounds of the Act term: act_lo[i] = floor(-lambda_i Gmax_i / (4096 Max_i)) where a cell of type i moves,
+    // act_hi[m][j] = floor(lambda_m Gmax_j / (4096 Max_m)) where a cell of type m moves and type j is the target
+    int64_t act_lo[kMaxTypes], act_hi[kMaxTypes][kMaxTypes];
 };
+// gm_max and the Act bounds from the weights and the LN / EXPQ tables (0 where Max_act is 0)
+inline void fill_act_bounds(TypeParams &tp, const int32_t *ln, const int32_t *expq)
+{
+    const auto floor_div = [](int64_t num, int64_t den) {
+        const int64_t q = num / den;
+        return num % den != 0 && num < 0 ? q - 1 : q;
+    };
+    for (int a = 0; a < kMaxTypes; a++) {
+        const int m = tp.max_act[a] < 0 ? 0 : (tp.max_act[a] > 127 ? 127 : tp.max_act[a]);
+        tp.gm_max[a] = m > 0 ? expq[ln[m] >> 6] : 0;
+    }
+    for (int a = 0; a < kMaxTypes; a++) {
+        const int64_t lam = tp.lambda_act[a], den = (int64_t)tp.max_act[a] * 4096;
+        tp.act_lo[a] = den > 0 ? floor_div(-lam * tp.gm_max[a], den) : 0;
+        for (int b = 0; b < kMaxTypes; b++) tp.act_hi[a][b] = den > 0 ? floor_div(lam * tp.gm_max[b], den) : 0;
+    }
+}
 
-// Everything one round of the sweep needs.
-struct RoundArgs {
+// The state a round reads and writes.  Pointers are generic: a kernel that runs many rounds of a
+// small lattice keeps some of it in shared memory.
+struct RoundBufs {
     int32_t *lat;              // lattice words (see cell_id), x fastest
-    uint32_t packed;           // 1: the words carry Act stamps (Act on for this lattice)
-    uint32_t stream_loads;     // 1: lattice words through the streaming cache path (Act, area edge >= 8)
-    uint32_t pdl;              // 1: launched as a programmatic dependent of the previous round
-    const uint8_t *cell_type;  // per cell id
     const int32_t *Vc, *Ac;    // tallies as of the start of this round
     int32_t *Vn, *An;          // tallies being built for the next round
     const int4 *pend_prev;     // accepted change of the previous round, per active index (valid where flagged)
     int4 *pend_cur;            // accepted change of this round, per active index (written on accept only)
-    const uint8_t *flag_prev;  // 1 where the previous round accepted a copy, per active index
-    uint8_t *flag_cur;         // this round's flags (every active index written)
+    uint8_t *flag_prev;        // 1 where the previous round accepted a copy, per active index; cleared as it is read
+    uint8_t *flag_cur;         // this round's flags: all 0 as the round begins, set on accept
     // composite variable tracking (Eq. 11); null when off.  Coordinate sums of every cell,
     // [n_cells + 1][3], as of the start of this round and being built for the next round, and
     // per active index the site and image shifts of an accepted change (valid where flagged).
@@ -111,6 +132,20 @@ struct RoundArgs {
     long long *Sn;
     const int2 *tpend_prev;
     int2 *tpend_cur;
+};
+
+// Where a round stands.
+struct RoundPos {
+    uint32_t cx, cy, cz;       // active colour, per axis
+    uint32_t t, sp, r;         // MCS (low 32 bits), sub-pass, round
+};
+
+// What all rounds of a lattice share.
+struct RoundArgs {
+    uint32_t packed;           // 1: the words carry Act stamps (Act on for this lattice)
+    uint32_t stream_loads;     // 1: lattice words through the streaming cache path (Act, area edge >= 8)
+    uint32_t pdl;              // 1: launched as a programmatic dependent of the previous round
+    const uint8_t *cell_type;  // per cell id
     const uint32_t *thr;       // acceptance thresholds, L entries
     const int32_t *ln_tab;     // LN[0..128]
     const int32_t *expq;       // EXPQ[m]
@@ -118,37 +153,66 @@ struct RoundArgs {
     int32_t L;
     uint32_t nx, ny, nz;
     uint32_t s, c, sd;         // block edge, divisions, sites per block
+    uint32_t s_log2;           // log2 of s, or 32 where s is not a power of two
     uint32_t nbx, nby;         // blocks per axis
-    uint32_t nax, nay;         // active blocks per axis (nbx / c, nby / c)
+    uint32_t nax, nay, naz;    // active blocks per axis (nbx / c, nby / c, nbz / c)
     uint32_t n_active;
-    uint32_t cx, cy, cz;       // active colour, per axis
-    uint32_t t, sp, r;         // MCS (low 32 bits), sub-pass, round
     uint32_t key0, key1;
-    uint32_t brick_x, brick_y, brick_z;  // active blocks per CTA along each axis (product <= 256)
+    uint32_t brick_lx, brick_ly, brick_lz;  // log2 of the active blocks per CTA along each axis
+    uint32_t nbr_x, nbr_y;     // bricks along x and y where the grid is linear, else 0
+    uint32_t uni;              // the type of every cell when they all share one, else 0
+    float h_scale, h_eps;      // the test's logarithm: 16 T ln 2, and the margin within which the table decides
     const int16_t *chem;       // chemotaxis field, dim int16 per site (Q14), or null
     const double *pers_dir;    // persistence directions, 3 per cell id, or null
     TypeParams tp;
 };
 
-// Batched ensembles: one lattice of the batch.  base carries its buffers and
-// constants (per-round fields are filled in by the kernel); the round of
-// lattice l at batch step q is round g_start + q of that lattice, in MCS
-// t_start + q / R.
-constexpr uint32_t kBatchMaxThreads = 256;
-struct BatchLattice {
-    RoundArgs base;
+// The buffers of one lattice, both parities of the round index, and the round's view of them.
+struct LatticeBufs {
+    int32_t *lat;
     int32_t *V[2], *A[2];
     int4 *pend[2];
     uint8_t *flag[2];
-    long long *S[2];     // tracked centroid sums, when the batch tracks them (else null)
+    long long *S[2];     // tracked centroid sums, when tracking is on (else null)
     int2 *tpend[2];
+};
+__host__ __device__ __forceinline__ RoundBufs round_bufs(const LatticeBufs &l, uint32_t par)
+{
+    RoundBufs b;
+    b.lat = l.lat;
+    b.Vc = l.V[par];
+    b.Ac = l.A[par];
+    b.Vn = l.V[par ^ 1u];
+    b.An = l.A[par ^ 1u];
+    b.pend_prev = l.pend[par ^ 1u];
+    b.pend_cur = l.pend[par];
+    b.flag_prev = l.flag[par ^ 1u];
+    b.flag_cur = l.flag[par];
+    b.Sc = l.S[par];
+    b.Sn = l.S[par ^ 1u];
+    b.tpend_prev = l.tpend[par ^ 1u];
+    b.tpend_cur = l.tpend[par];
+    return b;
+}
+
+// Batched ensembles: one lattice of the batch; the round of lattice l at batch step q is round
+// g_start + q of that lattice, in MCS t_start.
+constexpr uint32_t kBatchMaxThreads = 256;
+struct BatchLattice {
+    RoundArgs base;
+    LatticeBufs bufs;
     uint32_t R, k, C;
     int32_t n_cells;
     int64_t t_start;
     uint64_t g_start;
+    uint8_t *colours;    // colour of every sub-pass of the current MCS (R / k entries, see launch_batch_colours)
 };
+// after_round: the kernel before it on the stream is a round of the same MCS (programmatic dependent launch)
 cudaError_t launch_batch_round(int dim, bool perim, bool act, bool track, const BatchLattice *lats,
-                               const int2 *items, uint32_t n_items, uint32_t q, uint32_t threads, cudaStream_t st);
+                               const int4 *items, uint32_t n_items, uint32_t q, uint32_t threads, bool after_round,
+                               cudaStream_t st);
+// the colours of every member's sub-passes of its current MCS
+cudaError_t launch_batch_colours(const BatchLattice *lats, uint32_t n, cudaStream_t st);
 // every tracking member's centroids into [0, n) after its MCS (csrc/cpm_track.cu)
 cudaError_t launch_batch_track_rewrap(int dim, const BatchLattice *lats, uint32_t n, cudaStream_t st);
 cudaError_t launch_batch_clamp(const BatchLattice *lats, const int2 *items, uint32_t n_items, cudaStream_t st);
@@ -157,7 +221,7 @@ cudaError_t launch_batch_advance(BatchLattice *lats, uint32_t n, cudaStream_t st
 struct BatchLoopArgs {
     BatchLattice *lats;
     uint32_t n_lats;
-    const int2 *items;        // round items, members by rounds per MCS (descending)
+    const int4 *items;        // round items (member, brick x y z), members by rounds per MCS (descending)
     const uint32_t *upto_q;   // items of round q: the first upto_q[q]
     uint32_t r_max;           // rounds per MCS of the longest member
     const int2 *clamp;        // Act clamp items
@@ -234,30 +298,42 @@ struct TileArgs {
 size_t tile_dyn_smem(int dim, bool act, uint32_t T, uint32_t cap, uint32_t a, uint32_t thr_smem);
 cudaError_t launch_tile_epoch(int dim, bool perim, bool act, const TileArgs &a, uint32_t n_tiles, cudaStream_t st);
 
-// CTA brick of active blocks for the round kernel, measured on GB300 against
-// other shapes and row-major mapping.  3D: 8x4x4 (128 threads) when active
-// blocks are less than 16 sites apart (areas of edge < 16), where the
-// stencils of neighbouring threads share lines; 16x8x2 (256 threads) when
-// they are 16 or more apart and a row has at least 16 of them: no lines are
-// shared, and a warp's loads then fall on 16 consecutive 64-byte granules of
-// a row (1024^3 tissue with 16^3 areas: 193.5 against 201.6 ms per MCS).
-// 2D: 16x16.
-inline void pick_bricks(int dim, uint32_t nax, uint32_t nay, RoundArgs &a)
+// Brick of active blocks per CTA (2^lx x 2^ly x 2^lz, a thread each): 256 of them, fewer where that leaves SMs
+// without a CTA.  3D: 8 along x when active blocks are less than 16 sites apart, where the stencils of
+// neighbouring threads share lines; 16 when they are 16 or more apart and a row has as many: no lines are
+// shared, and a warp's loads then fall on 16 consecutive 64-byte granules of a row.
+inline void pick_bricks(int dim, RoundArgs &a)
 {
-    if (dim == 3) {
-        if (a.s * a.c >= 16 && nax >= 16) {
-            a.brick_x = 16; a.brick_y = 8; a.brick_z = 2;
-        } else {
-            a.brick_x = 8; a.brick_y = 4; a.brick_z = 4;
-        }
+    uint32_t log2 = 8;
+    while (log2 > 5 && a.n_active < (152u * 2) << log2) log2--;
+    if (dim == 2) {
+        a.brick_lx = (log2 + 1) / 2;
+        a.brick_ly = log2 - a.brick_lx;
+        a.brick_lz = 0;
+    } else if (a.s * a.c >= 16 && a.nax >= 16) {
+        a.brick_lx = 4;
+        a.brick_ly = log2 - 4 < 3 ? log2 - 4 : 3;
+        a.brick_lz = log2 - 4 - a.brick_ly;
     } else {
-        a.brick_x = 16; a.brick_y = 16; a.brick_z = 1;
+        a.brick_lx = 3;
+        a.brick_ly = 2;
+        a.brick_lz = log2 - 5;
     }
-    (void)nay;
+}
+
+// The fields of RoundArgs that follow from the schedule and the temperature alone.
+inline void fill_round_constants(RoundArgs &a, double temperature)
+{
+    a.s_log2 = 32;
+    for (uint32_t k = 0; k < 31; k++)
+        if (a.s == (1u << k)) a.s_log2 = k;
+    a.h_scale = (float)(16.0 * 0.69314718055994531 * temperature);
+    a.h_eps = (float)(1.0 + 1e-3 * temperature);
 }
 
 // Launchers (defined in the per-dimension translation units).
-cudaError_t launch_round(int dim, bool perim, bool act, const RoundArgs &a, cudaStream_t st);
+cudaError_t launch_round(int dim, bool perim, bool act, const RoundArgs &a, const RoundBufs &b, const RoundPos &p,
+                         cudaStream_t st);
 cudaError_t launch_recount(int dim, const int32_t *lat, const uint8_t *cell_type, int32_t *V, int32_t *A,
                            uint32_t nx, uint32_t ny, uint32_t nz, cudaStream_t st);
 cudaError_t launch_compare(const int32_t *V, const int32_t *A, const int32_t *V2, const int32_t *A2, int32_t n,

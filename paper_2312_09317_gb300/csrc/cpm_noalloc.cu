@@ -183,7 +183,6 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
 
     RoundArgs a;
     memset(&a, 0, sizeof a);
-    a.lat = lattice;
     a.packed = 0;  // no Act term here: the words are plain ids
     a.pdl = 1;     // each round overlaps its set-up with the previous round's tail
     a.cell_type = cell_type;
@@ -195,11 +194,12 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
     a.nx = (uint32_t)c.nx; a.ny = (uint32_t)c.ny; a.nz = (uint32_t)c.nz;
     a.s = s; a.c = (uint32_t)c.c; a.sd = sd;
     a.nbx = nbx; a.nby = nby;
-    a.nax = nbx / (uint32_t)c.c; a.nay = nby / (uint32_t)c.c;
+    a.nax = nbx / (uint32_t)c.c; a.nay = nby / (uint32_t)c.c; a.naz = c.dim == 3 ? nbz / (uint32_t)c.c : 1;
     a.n_active = (uint32_t)n_active;
     a.key0 = (uint32_t)c.seed;
     a.key1 = (uint32_t)(c.seed >> 32);
-    pick_bricks(c.dim, a.nax, a.nay, a);
+    fill_round_constants(a, c.temperature);
+    pick_bricks(c.dim, a);
     memcpy(a.tp.J, c.J, sizeof a.tp.J);
     memcpy(a.tp.lambda_v, c.lambda_v, sizeof a.tp.lambda_v);
     memcpy(a.tp.v_target, c.v_target, sizeof a.tp.v_target);
@@ -212,7 +212,17 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
     for (int k = 0; k < CPM_MAX_TYPES; k++)
         if (c.lambda_p[k]) perim = true;
 
-    int32_t *Vb[2] = {V, V1}, *Ab[2] = {A, A1};
+    LatticeBufs bufs{};
+    bufs.lat = lattice;
+    bufs.V[0] = V;
+    bufs.V[1] = V1;
+    bufs.A[0] = A;
+    bufs.A[1] = A1;
+    for (int p = 0; p < 2; p++) {
+        bufs.pend[p] = pend + (size_t)p * n_active;
+        bufs.flag[p] = flags + (size_t)p * n_active;
+    }
+    RoundPos pos{};
     const uint32_t k_rounds = sd / (uint32_t)c.P;
     const uint32_t per_mcs = C * (uint32_t)c.P;
     uint64_t g = 0;
@@ -228,23 +238,14 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
             perm[j] = tmp;
         }
         const uint32_t col = perm[(uint32_t)sp % C];
-        a.cx = col % (uint32_t)c.c;
-        a.cy = (col / (uint32_t)c.c) % (uint32_t)c.c;
-        a.cz = col / ((uint32_t)c.c * (uint32_t)c.c);
-        a.t = (uint32_t)t;
-        a.sp = (uint32_t)sp;
+        pos.cx = col % (uint32_t)c.c;
+        pos.cy = (col / (uint32_t)c.c) % (uint32_t)c.c;
+        pos.cz = col / ((uint32_t)c.c * (uint32_t)c.c);
+        pos.t = (uint32_t)t;
+        pos.sp = (uint32_t)sp;
         for (uint32_t r = 0; r < k_rounds; r++, g++) {
-            const int cur = (int)(g & 1);
-            a.r = r;
-            a.Vc = Vb[cur];
-            a.Ac = Ab[cur];
-            a.Vn = Vb[cur ^ 1];
-            a.An = Ab[cur ^ 1];
-            a.pend_prev = pend + (size_t)(cur ^ 1) * n_active;
-            a.pend_cur = pend + (size_t)cur * n_active;
-            a.flag_prev = flags + (size_t)(cur ^ 1) * n_active;
-            a.flag_cur = flags + (size_t)cur * n_active;
-            NA_TRY(launch_round(c.dim, perim, false, a, st));
+            pos.r = r;
+            NA_TRY(launch_round(c.dim, perim, false, a, round_bufs(bufs, (uint32_t)(g & 1)), pos, st));
         }
         if (++sp == (int32_t)per_mcs) {
             sp = 0;

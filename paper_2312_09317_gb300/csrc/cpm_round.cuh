@@ -1,0 +1,530 @@
+// One round of copy attempts, as a warp runs it: shared by the single-lattice and the batched
+// round kernels.
+//
+// The energy change follows the paper's Methods: Eq. 1 (adhesion over the Moore neighbourhood,
+// each pair counted once; volume term), Eq. 3 (perimeter term) and Eq. 8/Eq. 9 (Act term,
+// geometric mean), all in integers; Eq. 2 acceptance through the integer threshold table.
+#pragma once
+
+#include <cstdint>
+
+#include "cpm_internal.h"
+
+namespace cpmgb {
+namespace {
+
+struct SmemTables {
+    int32_t J[kMaxTypes * kMaxTypes];
+    int32_t lv[kMaxTypes], vt[kMaxTypes], lp[kMaxTypes], at[kMaxTypes], la[kMaxTypes], ma[kMaxTypes];
+    int32_t ln[kLnEntries];
+};
+
+__device__ __forceinline__ void load_tables(SmemTables &sm, const RoundArgs &a, bool with_ln)
+{
+    for (int k = threadIdx.x; k < kMaxTypes * kMaxTypes; k += blockDim.x) sm.J[k] = a.tp.J[k / kMaxTypes][k % kMaxTypes];
+    if (threadIdx.x < kMaxTypes) {
+        const int k = threadIdx.x;
+        sm.lv[k] = a.tp.lambda_v[k];
+        sm.vt[k] = a.tp.v_target[k];
+        sm.lp[k] = a.tp.lambda_p[k];
+        sm.at[k] = a.tp.a_target[k];
+        sm.la[k] = a.tp.lambda_act[k];
+        sm.ma[k] = a.tp.max_act[k];
+    }
+    if (with_ln)
+        for (int k = threadIdx.x; k < kLnEntries; k += blockDim.x) sm.ln[k] = a.ln_tab[k];
+}
+
+// Type of a lattice id.  When every cell has the same type (a.uni), it follows from the id alone,
+// which takes the type table's load out of the chain of dependent loads of an attempt.
+__device__ __forceinline__ int type_of(const RoundArgs &a, int32_t sigma)
+{
+    if (a.uni) return sigma > 0 ? (int)a.uni : (sigma < 0 ? a.tp.obstacle_type : 0);
+    return sigma < 0 ? a.tp.obstacle_type : (int)__ldg(a.cell_type + sigma);
+}
+
+// x + d (d in -1, 0, 1) on a periodic axis of extent n, for x in [0, n)
+__device__ __forceinline__ uint32_t wrap_step(uint32_t x, int d, uint32_t n)
+{
+    return d < 0 ? (x == 0 ? n - 1 : x - 1) : (d > 0 ? (x + 1 == n ? 0 : x + 1) : x);
+}
+
+// A lattice word of the round kernels.  With Act and areas of edge 8 or
+// more, through the streaming cache path (ld.global.cs, evict first): the
+// active blocks of a round are then 8 sites apart, a round touches each
+// line of its stencils about once, and the tallies and type tables it also
+// reads stay in L2 longer (4% faster on the 1024^3 tissue with a = 8).  With
+// smaller areas the stencils of neighbouring blocks share lines and plain
+// loads are faster (6% on the same tissue with a = 4).
+template <bool ACT>
+__device__ __forceinline__ int32_t lat_word(const RoundArgs &a, const RoundBufs &b, uint32_t site)
+{
+    return ACT && a.stream_loads ? __ldcs(b.lat + site) : b.lat[site];
+}
+
+// Act value of a site from its stamp: Max - age, clipped at 0.
+__device__ __forceinline__ int act_value(uint32_t stamp, uint32_t t8, int max_act)
+{
+    const int age = (int)((t8 - stamp) & 255u);
+    const int v = max_act - age;
+    return v > 0 ? v : 0;
+}
+
+__device__ __noinline__ int64_t floor_div_pos(int64_t num, int64_t den)
+{
+    int64_t q = num / den;
+    if (num % den != 0 && num < 0) q -= 1;
+    return q;
+}
+
+// floor(num / (4096 mx)) for 1 <= mx <= 127: floor(floor(num / 4096) / mx), the second division in
+// 32 bits where the first quotient fits (any Act weight below 2^19 scaled), which keeps the 64-bit
+// division, some hundred instructions, off the usual path.
+__device__ __forceinline__ int64_t act_quotient(int64_t num, int32_t mx)
+{
+    const int64_t q = num >> 12;
+    const int32_t q32 = (int32_t)q;
+    if (q != (int64_t)q32) return floor_div_pos(q, mx);
+    const int32_t s = q32 >> 31;  // floor for negative values: ~((~q) / mx)
+    return (int64_t)((int32_t)((uint32_t)(q32 ^ s) / (uint32_t)mx) ^ s);
+}
+
+// Motility terms (Eq. 4, Eq. 5) of the copy from the source (stencil index
+// ox, oy, oz around the target) into the target, in 1/16 energy units: the
+// moving cell is si (sj when si is the medium), d = target - source, and
+// each term is floor(e) with e formed by the same rounded double operations,
+// in the same order, as the replay: chemotaxis
+// e = ((double)(-16 lambda (d . C_q)) / 16384) * (1/|d|), persistence
+// e = ((d_x p_x + d_y p_y + d_z p_z) * (double)(-16 lambda)) * (1/|d|).
+// Kept out of line: the round kernels call it only when a field or a
+// persistence direction is set, and inlining its FP64 code into every round
+// kernel enlarges them (instruction-fetch stalls).
+template <int DIM>
+__device__ __noinline__ int64_t motility_q(const RoundArgs &a, int32_t si, int32_t sj, int ti, int tj, int ox,
+                                              int oy, int oz, uint32_t isite)
+{
+    const int32_t m = si > 0 ? si : sj;
+    const int tp = si > 0 ? ti : tj;
+    const int dx = 1 - ox, dy = 1 - oy, dz = DIM == 3 ? 1 - oz : 0;
+    const double il = a.tp.inv_len[dx * dx + dy * dy + dz * dz];
+    int64_t dh = 0;
+    if (a.chem && a.tp.lambda_chem[tp] != 0) {
+        const int16_t *c = a.chem + (size_t)isite * DIM;
+        int64_t dc = (int64_t)dx * c[0] + (int64_t)dy * c[1];
+        if (DIM == 3) dc += (int64_t)dz * c[2];
+        const double e = __dmul_rn((double)(-16 * (int64_t)a.tp.lambda_chem[tp] * dc) / 16384.0, il);
+        dh += (int64_t)floor(e);
+    }
+    if (a.pers_dir && a.tp.lambda_pers[tp] != 0 && m > 0) {
+        const double *ph = a.pers_dir + 3 * (size_t)m;
+        double sd = __dmul_rn((double)dx, ph[0]);
+        sd = __dadd_rn(sd, __dmul_rn((double)dy, ph[1]));
+        sd = __dadd_rn(sd, __dmul_rn((double)dz, ph[2]));
+        const double e = __dmul_rn(__dmul_rn(sd, (double)(-16 * (int64_t)a.tp.lambda_pers[tp])), il);
+        dh += (int64_t)floor(e);
+    }
+    return dh;
+}
+
+// Composite variable tracking (Eq. 11).  A copy into site j adds j to sigma_i and
+// removes it from sigma_j, each at its periodic image nearest that cell's centroid
+// as the round began (Sc / Vc); the image shifts (-3..3 per axis, 3 bits each:
+// sigma_i's in bits 0..8, sigma_j's in bits 9..17) travel with the pending change,
+// so that the next round adds the same amounts to the other buffer.
+template <int DIM>
+__device__ __noinline__ int2 track_accept(const RoundArgs &a, const RoundBufs &b, int32_t si, int32_t sj, uint32_t j, uint32_t jx,
+                                          uint32_t jy, uint32_t jz)
+{
+    uint32_t bits = 0;
+    const int64_t Vi = si > 0 ? b.Vc[si] : 0, Vj = sj > 0 ? b.Vc[sj] : 0;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const int64_t x = d == 0 ? jx : (d == 1 ? jy : jz);
+        const int64_t n = d == 0 ? a.nx : (d == 1 ? a.ny : a.nz);
+        if (si > 0) {
+            const int64_t k = track_image_shift(x, b.Sc[3 * si + d], Vi, n);
+            atomicAdd((unsigned long long *)(b.Sn + 3 * si + d), (unsigned long long)(x + n * k));
+            bits |= (uint32_t)(k + 3) << (3 * d);
+        }
+        if (sj > 0) {
+            const int64_t k = track_image_shift(x, b.Sc[3 * sj + d], Vj, n);
+            atomicAdd((unsigned long long *)(b.Sn + 3 * sj + d), (unsigned long long)(-(x + n * k)));
+            bits |= (uint32_t)(k + 3) << (9 + 3 * d);
+        }
+    }
+    return make_int2((int32_t)j, (int32_t)bits);
+}
+
+// the previous round's tracked change (see track_accept) into the other buffer
+template <int DIM>
+__device__ __noinline__ void track_carry(const RoundArgs &a, const RoundBufs &b, int32_t si, int32_t sj, int2 e)
+{
+    const uint32_t j = (uint32_t)e.x, bits = (uint32_t)e.y;
+    const uint32_t jx = j % a.nx, jy = (j / a.nx) % a.ny, jz = j / (a.nx * a.ny);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const int64_t x = d == 0 ? jx : (d == 1 ? jy : jz);
+        const int64_t n = d == 0 ? a.nx : (d == 1 ? a.ny : a.nz);
+        if (si > 0) {
+            const int64_t k = (int64_t)((bits >> (3 * d)) & 7u) - 3;
+            atomicAdd((unsigned long long *)(b.Sn + 3 * si + d), (unsigned long long)(x + n * k));
+        }
+        if (sj > 0) {
+            const int64_t k = (int64_t)((bits >> (9 + 3 * d)) & 7u) - 3;
+            atomicAdd((unsigned long long *)(b.Sn + 3 * sj + d), (unsigned long long)(-(x + n * k)));
+        }
+    }
+}
+
+// An attempt that survived the early reject, handed from the lane that drew it to the group of four
+// lanes that evaluates it.
+struct __align__(16) Survivor {
+    uint32_t i_dir;  // active index, and the stencil index (0..26) of the source above bit kDirShift
+    uint32_t off;    // storage offset of the target
+    uint32_t x, y, z;
+    uint32_t w2;     // acceptance draw
+    int32_t wi, wj;  // lattice words of source and target
+};
+constexpr uint32_t kRoundThreads = 256;  // most threads of a CTA, one attempt each
+struct Survivors {
+    Survivor at[kRoundThreads];
+    uint32_t n[2];   // survivors so far; a loop over rounds clears one count while the other is in use
+};
+// n_active <= 2^31 / 27 in 3D and 2^31 / 9 in 2D, so the index and the direction share a word
+template <int DIM>
+constexpr int kDirShift = DIM == 3 ? 27 : 28;
+
+// Storage offset of a site, and the step in it from coordinate v to v + d (d in -1, 0, 1) on an axis.
+__device__ __forceinline__ uint32_t site_off(const RoundArgs &a, uint32_t x, uint32_t y, uint32_t z)
+{
+    return x + a.nx * (y + a.ny * z);
+}
+template <int AXIS>
+__device__ __forceinline__ uint32_t axis_step(const RoundArgs &a, uint32_t v, int d)
+{
+    const uint32_t to = wrap_step(v, d, AXIS == 0 ? a.nx : (AXIS == 1 ? a.ny : a.nz));
+    return (to - v) * (AXIS == 0 ? 1u : (AXIS == 1 ? a.nx : a.nx * a.ny));
+}
+
+// The share of one lane (sub, of G = 4 or 8) in the 3^d window around a site without its centre:
+// the eight columns (dx, dy) != (0, 0) are dealt out 8 / G to a lane, and in 3D lanes 0 and 1 also
+// take the sites below and above the centre.  The columns are the lane's for good, so an offset is
+// one addition of a column's and a plane's step, with no division and no shuffle per neighbour.
+template <int DIM, int G>
+struct Window {
+    static constexpr int COLS = 8 / G, K = DIM == 3 ? 3 * COLS + 1 : COLS;
+    uint32_t col[COLS], below, above;  // steps of the columns and the planes
+    __device__ __forceinline__ Window(const RoundArgs &a, uint32_t sub, uint32_t x, uint32_t y, uint32_t z)
+    {
+#pragma unroll
+        for (int c = 0; c < COLS; ++c) {
+            const uint32_t m = sub + (uint32_t)(G * c), idx = m + (m >= 4 ? 1u : 0u);  // skip the centre column
+            const int dy = idx < 3 ? -1 : (idx < 6 ? 0 : 1), dx = (int)idx - 3 * dy - 4;
+            col[c] = axis_step<0>(a, x, dx) + axis_step<1>(a, y, dy);
+        }
+        below = DIM == 3 ? axis_step<2>(a, z, -1) : 0;
+        above = DIM == 3 ? axis_step<2>(a, z, 1) : 0;
+    }
+    // whether the lane has a k-th neighbour, and its offset from the centre
+    __device__ __forceinline__ static bool has(int k, uint32_t sub) { return DIM == 2 || k < 3 * COLS || sub < 2; }
+    __device__ __forceinline__ uint32_t step(int k, uint32_t sub) const
+    {
+        if (DIM == 2) return col[k];
+        if (k == 3 * COLS) return sub == 0 ? below : above;
+        return col[k / 3] + (k % 3 == 0 ? below : (k % 3 == 2 ? above : 0u));
+    }
+};
+
+// sum over the G lanes of a group
+template <int G>
+__device__ __forceinline__ int32_t group_sum(int32_t v)
+{
+#pragma unroll
+    for (int d = 1; d < G; d *= 2) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// The draws of one attempt: active block (ix, iy, iz), active index i, in the round p.
+// Depends on the launch arguments only.
+struct Draw {
+    uint32_t i_dir, off, src, x, y, z, w2;
+};
+template <int DIM>
+__device__ __forceinline__ Draw round_draw(const RoundArgs &a, const RoundPos &p, uint32_t ix, uint32_t iy, uint32_t iz,
+                                           uint32_t i)
+{
+    constexpr uint32_t NB = DIM == 3 ? 26 : 8;
+    Draw d;
+    const uint32_t bx = ix * a.c + p.cx, by = iy * a.c + p.cy, bz = DIM == 3 ? iz * a.c + p.cz : 0;
+    const Philox4 w = philox4x32_10(bx + a.nbx * (by + a.nby * bz), p.r, p.t, p.sp, a.key0, a.key1);
+    const uint32_t jl = draw_below(w.v[0], a.sd);
+    if (a.s_log2 < 32) {
+        d.x = (bx << a.s_log2) + (jl & (a.s - 1));
+        d.y = (by << a.s_log2) + ((jl >> a.s_log2) & (a.s - 1));
+        d.z = DIM == 3 ? (bz << a.s_log2) + (jl >> (2 * a.s_log2)) : 0;
+    } else {
+        d.x = bx * a.s + jl % a.s;
+        d.y = by * a.s + (jl / a.s) % a.s;
+        d.z = DIM == 3 ? bz * a.s + jl / (a.s * a.s) : 0;
+    }
+    const uint32_t n = draw_below(w.v[1], NB);
+    const uint32_t idx = n + (n >= NB / 2 ? 1u : 0u);  // skip the centre of the 3^d stencil
+    const int ox = (int)(idx % 3), oy = (int)((idx / 3) % 3), oz = DIM == 3 ? (int)(idx / 9) : 1;
+    d.i_dir = i | (idx << kDirShift<DIM>);
+    d.off = site_off(a, d.x, d.y, d.z);
+    d.src = d.off + axis_step<0>(a, d.x, ox - 1) + axis_step<1>(a, d.y, oy - 1) +
+            (DIM == 3 ? axis_step<2>(a, d.z, oz - 1) : 0u);
+    d.w2 = w.v[2];
+    return d;
+}
+
+// One round's attempts of a CTA, one per thread with `valid` set.  Every thread of the CTA calls
+// it; n_queue, a count in shared memory (one of q.n), is 0 on entry.
+//
+// Phase 1, one lane per attempt: the target's and source's words, the carry of the previous
+// round's change, the early reject.  About a fifth of the attempts on a tissue survive.
+// Phase 2, G lanes per survivor, 32 / G survivors per warp, dealt out over the warps of the CTA.
+// With G = 4 a lane holds two of a window's eight columns, so that its loads (two in 2D, seven in
+// 3D) are issued together, a survivor's sums are two shuffles, and the scalar part of the energy is
+// paid once for eight survivors; G = 8 makes the chain of one survivor shorter where a CTA has
+// warps to spare.  With one lane per attempt throughout, the window's loads wait for one
+// another (registers), and a warp's instructions run for the fifth of its lanes that survived:
+// 82 warp instructions per attempt on the 3D tissue, 10 of 32 lanes active.
+// Measured against that (ms per MCS): 256^3 cube cells 0.911 -> 0.597, 1024^3 fibre tissue
+// 189.2 -> 143.3, 64 uneven lattices of a sweep 5.00 -> 2.90.  Eight lanes per survivor and a queue
+// per warp: 0.976 and 180.7; two attempts per lane (half the warps): 1.46 and 336.
+template <int DIM, bool PERIM, bool ACT, bool TRACK, int G>
+__device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b, uint32_t t, const SmemTables &sm,
+                                          Survivors &q, uint32_t &n_queue, bool valid, const Draw &d,
+                                          uint32_t first_warp = 0)
+{
+    using Win = Window<DIM, G>;
+    static_assert(G == 4 || G == 8, "the four tallies take four lanes");
+    constexpr int NB = DIM == 3 ? 26 : 8, K = Win::K;
+    constexpr uint32_t kIndexMask = (1u << kDirShift<DIM>) - 1u;
+    const uint32_t lane = threadIdx.x & 31u;
+    // the warps take the survivors in turn, from first_warp on
+    const uint32_t warp = (threadIdx.x >> 5) + (threadIdx.x >> 5 >= first_warp ? 0u : blockDim.x >> 5) - first_warp;
+    const uint32_t t8 = t & 255u;
+
+    // the lattice, flags and tallies read from here on are the previous round's output, so a round
+    // launched as a programmatic dependent of the previous one waits for it here
+    if (a.pdl) asm volatile("griddepcontrol.wait;" ::: "memory");
+    {
+        int32_t wj = 0, wi = 0;
+        bool alive = false;
+        if (valid) {
+            const uint32_t i = d.i_dir & kIndexMask;
+            const uint8_t flag = b.flag_prev[i];
+            wj = lat_word<ACT>(a, b, d.off);
+            wi = lat_word<ACT>(a, b, d.src);
+            // the previous round's accepted change goes into the next tallies; its flag is cleared here, so that
+            // the buffer is all 0 when the next round sets its own (most flags are never written)
+            if (flag) {
+                b.flag_prev[i] = 0;
+                const int4 e = b.pend_prev[i];
+                if (e.x > 0) { atomicAdd(b.Vn + e.x, 1); atomicAdd(b.An + e.x, e.z); }
+                if (e.y > 0) { atomicAdd(b.Vn + e.y, -1); atomicAdd(b.An + e.y, e.w); }
+                if (TRACK) track_carry<DIM>(a, b, e.x, e.y, b.tpend_prev[i]);
+            }
+            const int32_t sj = cell_id(wj), si = cell_id(wi);
+            alive = si != sj && si >= 0 && sj >= 0;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, alive);
+        uint32_t first = 0;
+        if (lane == 0 && m) first = atomicAdd(&n_queue, (uint32_t)__popc(m));
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (alive) {
+            Survivor &s = q.at[first + (uint32_t)__popc(m & ((1u << lane) - 1u))];
+            s.i_dir = d.i_dir;
+            s.off = d.off;
+            s.x = d.x;
+            s.y = d.y;
+            s.z = d.z;
+            s.w2 = d.w2;
+            s.wi = wi;
+            s.wj = wj;
+        }
+    }
+    __syncthreads();
+
+    const uint32_t cnt = n_queue, sub = lane & (G - 1u);
+    uint32_t accepted = 0;
+    for (uint32_t base = (32 / G) * warp; base < cnt; base += blockDim.x / G) {
+        const uint32_t e = base + lane / G;
+        const bool on = e < cnt;
+        const Survivor s = q.at[on ? e : base];  // a group without a survivor repeats a valid one, without effect
+        const int32_t si = cell_id(s.wi), sj = cell_id(s.wj);
+        // tallies of both cells: one load, a lane each
+        int32_t tal = 0;
+        if (sub < (PERIM ? 4u : 2u)) {
+            const int32_t cell = sub & 1u ? sj : si;
+            if (cell > 0) tal = (sub & 2u ? b.Ac : b.Vc)[cell];
+        }
+        const Win win(a, sub, s.x, s.y, s.z);
+        int32_t wn[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) wn[k] = Win::has(k, sub) ? lat_word<ACT>(a, b, s.off + win.step(k, sub)) : 0;
+        const int ti = type_of(a, si), tj = type_of(a, sj);
+        // Counts of the neighbours in sigma_i, in sigma_j, in the medium and on obstacles, a byte each.
+        // Target's Act log-sum over its same-cell window: 24 bits (at most 26 x LN[127]), the number of
+        // zero Act values above them.
+        const int maxj = ACT && sj > 0 ? (int)sm.ma[tj] : 0;
+        int32_t counts = 0, lsj = 0;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int32_t sn = cell_id(wn[k]);
+            int32_t c = sn == si ? 1 : 0;
+            if (sn == sj) c += 1 << 8;
+            if (sn == 0) c += 1 << 16;
+            if (sn < 0) c += 1 << 24;
+            if (ACT && sn == sj && Win::has(k, sub)) {
+                const int av = act_value(word_stamp(wn[k]), t8, maxj);
+                lsj += av == 0 ? 1 << 24 : sm.ln[av];
+            }
+            counts += Win::has(k, sub) ? c : 0;
+        }
+        counts = group_sum<G>(counts);
+        const int mi = counts & 255, mj = (counts >> 8) & 255;
+        int32_t adhesion;
+        if (a.uni) {
+            // every cell has one type: the adhesion follows from the counts
+            const int n0 = (counts >> 16) & 255, nf = (counts >> 24) & 255, nc = NB - n0 - nf;
+            const int32_t *Ji = sm.J + ti * kMaxTypes, *Jj = sm.J + tj * kMaxTypes;
+            adhesion = Ji[a.uni] * (nc - (si > 0 ? mi : 0)) + Ji[0] * (n0 - (si > 0 ? 0 : mi)) + Ji[a.tp.obstacle_type] * nf;
+            adhesion -= Jj[a.uni] * (nc - (sj > 0 ? mj : 0)) + Jj[0] * (n0 - (sj > 0 ? 0 : mj)) + Jj[a.tp.obstacle_type] * nf;
+        } else {
+            adhesion = 0;
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (Win::has(k, sub)) {
+                    const int32_t sn = cell_id(wn[k]);
+                    const int tn = type_of(a, sn);
+                    if (sn != si) adhesion += sm.J[ti * kMaxTypes + tn];
+                    if (sn != sj) adhesion -= sm.J[tj * kMaxTypes + tn];
+                }
+            adhesion = group_sum<G>(adhesion);
+        }
+        const int32_t Vi = __shfl_sync(0xffffffffu, tal, 0, G), Vj = __shfl_sync(0xffffffffu, tal, 1, G);
+        const int dAi = NB - 2 * mi, dAj = 2 * mj - NB;
+        int64_t dh = adhesion;
+        if (si > 0) dh += (int64_t)sm.lv[ti] * (2 * ((int64_t)Vi - sm.vt[ti]) + 1);
+        if (sj > 0) dh += (int64_t)sm.lv[tj] * (1 - 2 * ((int64_t)Vj - sm.vt[tj]));
+        if (PERIM) {
+            const int32_t Ai = __shfl_sync(0xffffffffu, tal, 2, G), Aj = __shfl_sync(0xffffffffu, tal, 3, G);
+            if (si > 0) dh += (int64_t)sm.lp[ti] * dAi * (2 * ((int64_t)Ai - sm.at[ti]) + dAi);
+            if (sj > 0) dh += (int64_t)sm.lp[tj] * dAj * (2 * ((int64_t)Aj - sm.at[tj]) + dAj);
+        }
+        int64_t dhq = 16 * dh;
+        const uint32_t dir = s.i_dir >> kDirShift<DIM>;
+        const int ox = (int)(dir % 3), oy = (int)((dir / 3) % 3), oz = DIM == 3 ? (int)(dir / 9) : 1;
+        if (a.chem || a.pers_dir) {
+            const uint32_t isite = wrap_step(s.x, ox - 1, a.nx) +
+                                   a.nx * (wrap_step(s.y, oy - 1, a.ny) +
+                                           a.ny * (DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0));
+            dhq += motility_q<DIM>(a, si, sj, ti, tj, ox, oy, oz, isite);
+        }
+        // the test of Eq. 2 at an energy h > 0 (w2 < THR[h]): THR[h] = floor(2^32 exp(-h / 16T)), so it
+        // holds exactly for h <= 16 T ln(2^32 / (w2 + 1)).  The logarithm in single precision decides all
+        // h but the few within a.h_eps (over ten times its error bound) of that value, for which the
+        // table is read; a test thus mostly ends without another dependent load.
+        const float hs = a.h_scale * (32.0f - __log2f((float)s.w2 + 1.0f));
+        const int64_t h_lo = (int64_t)(int32_t)floorf(hs - a.h_eps), h_hi = (int64_t)(int32_t)ceilf(hs + a.h_eps);
+        const auto below = [&](int64_t h) {
+            if (h <= h_lo) return true;
+            if (h > h_hi) return false;
+            return h < a.L && s.w2 < __ldg(a.thr + h);
+        };
+        // decided: 1 accept, 0 reject, -1 open
+        int decided = !on || (sj > 0 && Vj <= 1) ? 0 : -1;
+        if (ACT) {
+            lsj = group_sum<G>(lsj);
+            const int tp = si > 0 ? ti : tj;
+            const int64_t lam = sm.la[tp];
+            const int32_t mx = sm.ma[tp];
+            bool window = false;  // the source's window is needed
+            int64_t gj = 0;
+            if (decided < 0 && lam != 0 && mx != 0) {
+                // the Act term lies in [act_lo, act_hi] = [floor(-lam Gmax_i / (Max 4096)), floor(lam Gmax_j / (Max
+                // 4096))] (GM in [0, Gmax] per cell, lambda >= 0); when every value in that range gives the same
+                // outcome of the test below (THR is non-increasing), the geometric means are not needed
+                const int64_t lo = dhq + (si > 0 ? a.tp.act_lo[ti] : 0);
+                const int64_t hi = dhq + (sj > 0 ? a.tp.act_hi[tp][tj] : 0);
+                if (hi <= 0) decided = 1;
+                else if (lo > 0 && !below(lo)) decided = 0;
+                else if (below(hi)) decided = 1;
+                else {
+                    // target: the log-sum gathered above (the centre and the mj same-cell neighbours; 0 when any of
+                    // their Act values is 0)
+                    if (sj > 0) {
+                        const int cv = act_value(word_stamp(s.wj), t8, maxj);
+                        if (cv != 0 && lsj < 1 << 24)
+                            gj = (int64_t)__ldg(a.expq + ((uint32_t)(lsj + sm.ln[cv]) / (uint32_t)(mj + 1) >> 6));
+                    }
+                    // the same with the target's mean known: [floor(lam (G_j - Gmax_i) / ..), floor(lam G_j / ..)]
+                    const int64_t hi1 = dhq + act_quotient(lam * gj, mx);
+                    const int64_t lo1 = dhq + act_quotient(lam * (gj - (si > 0 ? a.tp.gm_max[ti] : 0)), mx);
+                    if (hi1 <= 0 || below(hi1)) decided = 1;
+                    else if (lo1 > 0 && !below(lo1)) decided = 0;
+                    else window = true;  // si > 0: otherwise lo1 = hi1, and one of the two holds
+                }
+            }
+            if (__any_sync(0xffffffffu, window)) {
+                const uint32_t xi = wrap_step(s.x, ox - 1, a.nx), yi = wrap_step(s.y, oy - 1, a.ny);
+                const uint32_t zi = DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0;
+                const uint32_t src = site_off(a, xi, yi, zi);
+                const Win win_i(a, sub, xi, yi, zi);
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    wn[k] = window && Win::has(k, sub) ? lat_word<ACT>(a, b, src + win_i.step(k, sub)) : 0;
+                const int maxi = sm.ma[ti];
+                int32_t ci = 0, lsi = 0;
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (Win::has(k, sub) && cell_id(wn[k]) == si) {
+                        const int av = act_value(word_stamp(wn[k]), t8, maxi);
+                        ci += 1;
+                        lsi += av == 0 ? 1 << 24 : sm.ln[av];
+                    }
+                ci = group_sum<G>(ci);
+                lsi = group_sum<G>(lsi);
+                if (window) {
+                    int64_t gi = 0;
+                    const int cv = act_value(word_stamp(s.wi), t8, maxi);
+                    if (cv != 0 && lsi < 1 << 24)
+                        gi = (int64_t)__ldg(a.expq + ((uint32_t)(lsi + sm.ln[cv]) / (uint32_t)(ci + 1) >> 6));
+                    dhq += act_quotient(lam * (gj - gi), mx);
+                }
+            }
+        }
+        const bool ok = decided >= 0 ? decided == 1 : (dhq <= 0 || below(dhq));
+        const bool leader = sub == 0 && ok;
+        if (leader) {
+            const uint32_t i = s.i_dir & kIndexMask;
+            // a copy stamps the site with this MCS (a medium copy: age 128, no activity)
+            b.lat[s.off] = ACT && a.packed ? pack_word(si, si > 0 ? t8 : ((t - 128u) & 255u)) : si;
+            if (si > 0) { atomicAdd(b.Vn + si, 1); atomicAdd(b.An + si, dAi); }
+            if (sj > 0) { atomicAdd(b.Vn + sj, -1); atomicAdd(b.An + sj, dAj); }
+            b.pend_cur[i] = make_int4(si, sj, dAi, dAj);
+            b.flag_cur[i] = 1;
+            if (TRACK)
+                b.tpend_cur[i] = track_accept<DIM>(a, b, si, sj, s.x + a.nx * (s.y + a.ny * s.z), s.x, s.y, s.z);
+        }
+        accepted += (uint32_t)__popc(__ballot_sync(0xffffffffu, leader));
+    }
+    if (lane == 0 && accepted != 0) atomicAdd(a.accepts, (unsigned long long)accepted);
+}
+
+// Stamps whose age is 128 or more are reset to age exactly 128, so that ages
+// stay below 256 until the next clamp (run every 64 MCS).  Obstacle words are
+// left as they are (their stamp is never read).
+__device__ __forceinline__ void clamp_word(int32_t *p, uint32_t t8)
+{
+    const int32_t w = *p;
+    if (cell_id(w) < 0) return;
+    const uint32_t age = (t8 - word_stamp(w)) & 255u;
+    if (age >= 128u) *p = pack_word(cell_id(w), (t8 - 128u) & 255u);
+}
+
+}  // namespace
+}  // namespace cpmgb

@@ -81,10 +81,11 @@ __global__ void track_rewrap_kernel(int dim, uint32_t nx, uint32_t ny, uint32_t 
 __global__ void batch_track_rewrap_kernel(int dim, const BatchLattice *lats)
 {
     const BatchLattice &L = lats[blockIdx.x];
-    if (!L.S[0]) return;
+    if (!L.bufs.S[0]) return;
     const uint32_t par = (uint32_t)(L.g_start & 1u);
     for (int32_t c = (int32_t)threadIdx.x + 1; c <= L.n_cells; c += (int32_t)blockDim.x)
-        rewrap_cell(dim, L.base.nx, L.base.ny, L.base.nz, c, L.V[par], L.S[par], L.S[par ^ 1u]);
+        rewrap_cell(dim, L.base.nx, L.base.ny, L.base.nz, c, L.bufs.V[par], L.bufs.S[par],
+                    L.bufs.S[par ^ 1u]);
 }
 
 unsigned grid_of(uint64_t n)
