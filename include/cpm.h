@@ -345,8 +345,7 @@ int cpm_batch_observe(cpm_batch *b, int64_t *cells_out, int64_t *member_out);
  *   15 elongation: sqrt of the ratio of the principal second moments.
  * Centroids follow Methods, "Composite variable tracking" (Eq. 10); a cell
  * absent at some snapshot counts for 0..3, 13 and 15 only.  One kernel
- * launch; the batch keeps a scratch track buffer of n_snap * 2 * rows
- * doubles.  Asynchronous on the batch's stream. */
+ * launch.  Asynchronous on the batch's stream. */
 int cpm_batch_summarize(cpm_batch *b, const int64_t *cells_hist, const int64_t *member_hist, int32_t n_snap,
                         int32_t every, double *out);
 

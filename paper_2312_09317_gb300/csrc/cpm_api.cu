@@ -1005,8 +1005,6 @@ struct cpm_batch {
     int64_t obs_rows = 0;
     int32_t obs_max_cells = 0;
     uint8_t *d_colours = nullptr;        // BatchLattice::colours of every member
-    double *traj = nullptr;              // centroid tracks of cpm_batch_summarize
-    size_t traj_cap = 0;
     cudaGraphExec_t graph = nullptr;     // one MCS of every member
     int64_t graph_launches = 0;          // kernels in one replay
     // the persistent loop (cpm_batch_set_persistent)
@@ -1051,7 +1049,6 @@ void batch_free(cpm_batch *b)
     cudaFree(b->d_items);
     cudaFree(b->d_clamp);
     cudaFree(b->d_obs);
-    cudaFree(b->traj);
     cudaFree(b->d_upto_q);
     cudaFree(b->d_bar);
     cudaFree(b->d_next);
@@ -1526,7 +1523,6 @@ int batch_obs_items(cpm_batch *b)
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
         if (e != cudaSuccess) {
             cudaFree(b->d_obs);
-    cudaFree(b->traj);
             b->d_obs = nullptr;
             return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
         }
@@ -1556,17 +1552,8 @@ int cpm_batch_summarize(cpm_batch *b, const int64_t *cells_hist, const int64_t *
     if (n_snap < 1 || n_snap > kSummaryMaxSnap) return bfail(b, CPM_E_INVALID, "n_snap must be in 1..1024");
     if (every < 1) return bfail(b, CPM_E_INVALID, "every must be >= 1");
     if (int rc = batch_obs_items(b)) return rc;
-    const size_t need = (size_t)b->obs_rows * 2 * (size_t)n_snap;
-    if (need > b->traj_cap) {
-        cudaFree(b->traj);
-        b->traj = nullptr;
-        b->traj_cap = 0;
-        cudaError_t e = cudaMalloc(&b->traj, sizeof(double) * need);
-        if (e != cudaSuccess) return bfail(b, CPM_E_NOMEM, cudaGetErrorString(e));
-        b->traj_cap = need;
-    }
     cudaError_t e = launch_summarize(b->d_obs, (uint32_t)b->hs.size(), b->obs_max_cells, cells_hist, b->obs_rows,
-                                     member_hist, n_snap, every, b->traj, out, b->stream);
+                                     member_hist, n_snap, every, out, b->stream);
     if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
     b->launches += 1;
     return CPM_OK;

@@ -263,8 +263,8 @@ cudaError_t launch_pers_update(const int64_t *cells, int32_t n_cells, uint32_t n
 constexpr int kSummaryStats = 16;
 constexpr int kSummaryMaxSnap = 1024;
 cudaError_t launch_summarize(const ObserveItem *d_items, uint32_t n_items, int32_t max_cells, const int64_t *cells,
-                             int64_t rows, const int64_t *member, int32_t n_snap, int32_t every, double *traj,
-                             double *out, cudaStream_t st);
+                             int64_t rows, const int64_t *member, int32_t n_snap, int32_t every, double *out,
+                             cudaStream_t st);
 
 // Tiled schedule: everything one epoch of one tile colour needs.
 constexpr int kMaxEpochSubpasses = 512;

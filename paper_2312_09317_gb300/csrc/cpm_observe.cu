@@ -6,9 +6,7 @@
 // second moments (cell shape) and its interface count (Eq. 3); per lattice the cell-medium neighbour pairs and
 // the accepted copies so far.
 //
-// Sites of one warp are mostly of one or two cells, so every per-cell sum is
-// reduced over the lanes that share the cell id (__match_any_sync, then
-// __reduce_*_sync over that group) and added by the group's first lane.
+// A thread walks along the slowest axis and keeps the sums of the cell it is in.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -44,90 +42,167 @@ __global__ void observe_init_kernel(const ObserveItem *items, int64_t *cells, in
     }
 }
 
+// A walk: the sites (x, y) of a chunk of kWalk planes in 3D, x of a chunk of kWalk rows in 2D.  Threads
+// next to each other walk next to each other along x.
+constexpr uint32_t kWalk = 16;
+struct Walk {
+    uint32_t site, step, lo, hi;  // first site, distance to the next, extent [lo, hi) along the walked axis
+    uint32_t x, y;                // the fixed coordinates (y: 3D only)
+};
+template <int DIM>
+__device__ __forceinline__ uint32_t walk_count(const ObserveItem &it)
+{
+    return DIM == 3 ? it.nx * it.ny * ((it.nz + kWalk - 1) / kWalk) : it.nx * ((it.ny + kWalk - 1) / kWalk);
+}
+template <int DIM>
+__device__ __forceinline__ Walk walk_of(const ObserveItem &it, uint32_t w)
+{
+    Walk r;
+    r.x = w % it.nx;
+    r.y = DIM == 3 ? w / it.nx % it.ny : 0;
+    const uint32_t chunk = w / (DIM == 3 ? it.nx * it.ny : it.nx), n = DIM == 3 ? it.nz : it.ny;
+    r.step = DIM == 3 ? it.nx * it.ny : it.nx;
+    r.lo = chunk * kWalk;
+    r.hi = r.lo + kWalk < n ? r.lo + kWalk : n;
+    r.site = r.x + it.nx * r.y + r.step * r.lo;
+    return r;
+}
+__device__ __forceinline__ int observed_id(const ObserveItem &it, uint32_t site)
+{
+    const int id = cell_id(it.lat[site]);
+    return id > it.n_cells ? 0 : id;  // never above in a validated lattice; keeps the writes in bounds
+}
+
+// Along a walk the first site of a run of one cell has its lowest index.
+template <int DIM>
 __global__ void __launch_bounds__(kObsThreads) observe_anchor_kernel(const ObserveItem *items, int64_t *cells)
 {
     const ObserveItem it = items[blockIdx.y];
-    const int64_t n = (int64_t)it.nx * it.ny * it.nz;
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        int id = i < n ? cell_id(it.lat[i]) : 0;
-        if (id > it.n_cells) id = 0;  // never present in a validated lattice; keeps the write in bounds
-        const unsigned grp = __match_any_sync(0xffffffffu, id);
-        const unsigned lo = __reduce_min_sync(grp, (unsigned)(i < n ? i : 0xffffffffu));
-        if (id > 0 && lane == __ffs(grp) - 1)
-            atomicMin(reinterpret_cast<unsigned long long *>(cells + (it.row0 + id) * kObsFields), (unsigned long long)lo);
+    const uint32_t n = walk_count<DIM>(it);
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < n; w += gridDim.x * blockDim.x) {
+        const Walk k = walk_of<DIM>(it, w);
+        int last = 0;
+        uint32_t site = k.site;
+        for (uint32_t z = k.lo; z < k.hi; ++z, site += k.step) {
+            const int id = observed_id(it, site);
+            if (id > 0 && id != last) {
+                unsigned long long *a = reinterpret_cast<unsigned long long *>(cells + (it.row0 + id) * kObsFields);
+                if (*reinterpret_cast<volatile unsigned long long *>(a) > site) atomicMin(a, (unsigned long long)site);
+            }
+            last = id;
+        }
     }
 }
 
+// The sums of every cell.  A thread keeps the sums of the run at hand (sites of one cell next to each other
+// along its walk) in registers and adds them to the cell when the run ends: with the walk's coordinates
+// fixed, a site costs the sums of its offset along the walk and the comparisons with its neighbours, of
+// which each step loads only the plane (3D: nine words) or row (three) that comes into the window.
+// Against one site per thread, its 3^d - 1 neighbours loaded, reduced over the lanes of equal id (twelve
+// group reductions per site and group): 64 uneven lattices of a sweep 1.05 -> 0.70 ms with the anchors,
+// 1,024 runs 148 -> 62 us.
 template <int DIM>
 __global__ void __launch_bounds__(kObsThreads) observe_sums_kernel(const ObserveItem *items, int64_t *cells,
                                                                    int64_t *member)
 {
+    constexpr int P = DIM == 3 ? 9 : 3;  // sites of a window's plane
     const ObserveItem it = items[blockIdx.y];
-    const int nx = (int)it.nx, ny = (int)it.ny, nz = (int)it.nz;
-    const int64_t plane = (int64_t)nx * ny, n = plane * nz;
-    const int lane = threadIdx.x & 31;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = base + threadIdx.x;
-        int id = i < n ? cell_id(it.lat[i]) : 0;
-        if (id > it.n_cells) id = 0;
-        int ox = 0, oy = 0, oz = 0, iface = 0, medium = 0;
-        if (id > 0) {
-            const int z = (int)(i / plane), y = (int)((i / nx) % ny), x = (int)(i % nx);
-            const int64_t a = cells[(it.row0 + id) * kObsFields];
-            const int az = (int)(a / plane), ay = (int)((a / nx) % ny), ax = (int)(a % nx);
-            ox = min_image(x - ax, nx);
-            oy = min_image(y - ay, ny);
-            oz = min_image(z - az, nz);
-            const int zlo = DIM == 3 ? -1 : 0, zhi = DIM == 3 ? 1 : 0;
-            for (int dz = zlo; dz <= zhi; ++dz) {
-                int zz = z + dz;
-                zz = zz < 0 ? zz + nz : (zz >= nz ? zz - nz : zz);
-                for (int dy = -1; dy <= 1; ++dy) {
-                    int yy = y + dy;
-                    yy = yy < 0 ? yy + ny : (yy >= ny ? yy - ny : yy);
-                    for (int dx = -1; dx <= 1; ++dx) {
-                        if (dx == 0 && dy == 0 && dz == 0) continue;
-                        int xx = x + dx;
-                        xx = xx < 0 ? xx + nx : (xx >= nx ? xx - nx : xx);
-                        const int v = cell_id(it.lat[(int64_t)zz * plane + (int64_t)yy * nx + xx]);
-                        iface += v != id;
-                        medium += v == 0;
-                    }
+    const int nx = (int)it.nx, ny = (int)it.ny, nz = (int)it.nz, nw = DIM == 3 ? nz : ny;
+    const uint32_t n = walk_count<DIM>(it);
+    int medium = 0;
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < n; w += gridDim.x * blockDim.x) {
+        const Walk k = walk_of<DIM>(it, w);
+        // columns of the window: site numbers within a plane
+        uint32_t col[P];
+        {
+            const uint32_t xs[3] = {k.x == 0 ? it.nx - 1 : k.x - 1, k.x, k.x + 1 == it.nx ? 0 : k.x + 1};
+            const uint32_t ys[3] = {k.y == 0 ? it.ny - 1 : k.y - 1, k.y, k.y + 1 == it.ny ? 0 : k.y + 1};
+#pragma unroll
+            for (int c = 0; c < P; ++c) col[c] = xs[c % 3] + (DIM == 3 ? it.nx * ys[c / 3] : 0);
+        }
+        int prev[P], cur[P], next[P], zero_prev = 0, zero_cur = 0;
+        const auto plane = [&](uint32_t z, int (&v)[P]) {
+            int zeros = 0;
+#pragma unroll
+            for (int c = 0; c < P; ++c) {
+                v[c] = cell_id(it.lat[col[c] + k.step * z]);
+                zeros += v[c] == 0 ? 1 : 0;
+            }
+            return zeros;
+        };
+        zero_prev = plane(k.lo == 0 ? (uint32_t)nw - 1 : k.lo - 1, prev);
+        zero_cur = plane(k.lo, cur);
+        // the run at hand: cell, its anchor's coordinates, offsets, sums over its sites
+        int id = 0, ox = 0, oy = 0, aw = 0;
+        int cnt = 0, sw = 0, sww = 0, iface = 0;
+        const auto flush = [&]() {
+            if (id <= 0) return;
+            unsigned long long *row = reinterpret_cast<unsigned long long *>(cells + (it.row0 + id) * kObsFields);
+            const auto add = [&](int f, int64_t v) { atomicAdd(row + f, (unsigned long long)v); };
+            const int64_t c = cnt;
+            add(1, c);
+            add(2, c * ox);
+            add(5, iface);
+            add(6, c * ox * ox);
+            if (DIM == 3) {
+                add(3, c * oy);
+                add(4, sw);
+                add(7, c * oy * oy);
+                add(8, sww);
+                add(9, c * ox * oy);
+                add(10, (int64_t)sw * ox);
+                add(11, (int64_t)sw * oy);
+            } else {
+                add(3, sw);
+                add(7, sww);
+                add(9, (int64_t)sw * ox);
+            }
+        };
+        for (uint32_t z = k.lo; z < k.hi; ++z) {
+            const int zero_next = plane(z + 1 == (uint32_t)nw ? 0 : z + 1, next);
+            int c = cur[P / 2];
+            if (c > it.n_cells) c = 0;
+            if (c != id) {
+                flush();
+                id = c;
+                cnt = sw = sww = iface = 0;
+                if (id > 0) {
+                    const uint32_t a = (uint32_t)cells[(it.row0 + id) * kObsFields];
+                    ox = min_image((int)k.x - (int)(a % it.nx), nx);
+                    if (DIM == 3) oy = min_image((int)k.y - (int)(a / it.nx % it.ny), ny);
+                    aw = (int)(DIM == 3 ? a / (it.nx * it.ny) : a / it.nx);
                 }
             }
+            if (id > 0) {
+                int same = -1;  // the site itself
+#pragma unroll
+                for (int q = 0; q < P; ++q) same += (prev[q] == id) + (cur[q] == id) + (next[q] == id);
+                iface += 3 * P - 1 - same;
+                medium += zero_prev + zero_cur + zero_next;
+                const int ow = min_image((int)z - aw, nw);
+                ++cnt;
+                sw += ow;
+                sww += ow * ow;
+            }
+#pragma unroll
+            for (int q = 0; q < P; ++q) {
+                prev[q] = cur[q];
+                cur[q] = next[q];
+            }
+            zero_prev = zero_cur;
+            zero_cur = zero_next;
         }
-        const unsigned grp = __match_any_sync(0xffffffffu, id);
-        const int cnt = __reduce_add_sync(grp, id > 0 ? 1 : 0);
-        const int sx = __reduce_add_sync(grp, ox), sy = __reduce_add_sync(grp, oy), sz = __reduce_add_sync(grp, oz);
-        const int sf = __reduce_add_sync(grp, iface);
-        const int sxx = __reduce_add_sync(grp, ox * ox), syy = __reduce_add_sync(grp, oy * oy);
-        const int szz = __reduce_add_sync(grp, oz * oz), sxy = __reduce_add_sync(grp, ox * oy);
-        const int sxz = __reduce_add_sync(grp, ox * oz), syz = __reduce_add_sync(grp, oy * oz);
-        const int sm = __reduce_add_sync(0xffffffffu, medium);
-        if (id > 0 && lane == __ffs(grp) - 1) {
-            unsigned long long *row = reinterpret_cast<unsigned long long *>(cells + (it.row0 + id) * kObsFields);
-            atomicAdd(row + 1, (unsigned long long)(int64_t)cnt);
-            atomicAdd(row + 2, (unsigned long long)(int64_t)sx);
-            atomicAdd(row + 3, (unsigned long long)(int64_t)sy);
-            atomicAdd(row + 4, (unsigned long long)(int64_t)sz);
-            atomicAdd(row + 5, (unsigned long long)(int64_t)sf);
-            atomicAdd(row + 6, (unsigned long long)(int64_t)sxx);
-            atomicAdd(row + 7, (unsigned long long)(int64_t)syy);
-            atomicAdd(row + 8, (unsigned long long)(int64_t)szz);
-            atomicAdd(row + 9, (unsigned long long)(int64_t)sxy);
-            atomicAdd(row + 10, (unsigned long long)(int64_t)sxz);
-            atomicAdd(row + 11, (unsigned long long)(int64_t)syz);
-        }
-        if (lane == 0 && sm)
-            atomicAdd(reinterpret_cast<unsigned long long *>(member + 2 * blockIdx.y), (unsigned long long)sm);
+        flush();
     }
+    medium = __reduce_add_sync(0xffffffffu, medium);
+    if ((threadIdx.x & 31) == 0 && medium)
+        atomicAdd(reinterpret_cast<unsigned long long *>(member + 2 * blockIdx.y), (unsigned long long)medium);
 }
 
-constexpr int kSumThreads = 128;
+constexpr int kSumThreads = 128, kSumWarps = kSumThreads / 32;
 constexpr int kMaxLag = 20;  // step-direction autocorrelation lags (x every MCS)
-// scalar accumulators of one lattice
+constexpr size_t kSumUnitBytes = 48 * 1024;  // step directions held at a time (at least one cell's)
+// scalar accumulators of one lattice, a copy per warp
 enum {
     A_MSD = 0,       // 3 sums, then 3 counts
     A_SP = 6,        // speed sum, sum of squares, count
@@ -135,162 +210,292 @@ enum {
     A_DAC = 11,      // 50-MCS direction cosine sum, count
     A_SLOW = 13,     // slow 50-MCS sub-tracks, count
     A_EL = 15,       // elongation sum, count
-    A_AC = 17,       // autocorrelation sums, lags 0..kMaxLag
-    A_ACN = A_AC + kMaxLag + 1,
-    A_N = A_ACN + kMaxLag + 1
+    A_AC = 17,       // sum and count of the direction cosines of the lag at hand
+    A_N = 19
 };
 
-// One CTA per lattice, threads over its cells.  Per cell: the centroid at
-// every snapshot (anchor + offset sums / volume), unwrapped across
-// snapshots by minimal-image steps; a cell absent at any snapshot has no
-// track.  Per-snapshot volume and interface moments and every track
-// statistic are accumulated in shared memory, then thread 0 forms the
-// sixteen statistics.
+__device__ __forceinline__ double warp_sum(double v)
+{
+#pragma unroll
+    for (int d = 16; d > 0; d /= 2) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
+
+// a / b with inv = 1 / b at hand: the product corrected by its residual (within an ulp of the quotient,
+// three operations instead of a division's dozen)
+__device__ __forceinline__ double quotient(double a, double b, double inv)
+{
+    const double q = a * inv;
+    return fma(fma(-q, b, a), inv, q);
+}
+
+// One CTA per lattice, a warp per cell, its lanes over the snapshots.  Per cell: the centroid at
+// every snapshot (anchor + offset sums / volume), unwrapped across snapshots by minimal-image
+// steps; a cell absent at any snapshot has no track.  Per-snapshot volume and interface moments are
+// sums of integers; the track statistics are summed per lane, then over lanes and warps in a fixed
+// order.
+//
+// Bound by the FP64 unit (about two operations per SM and clock): what counts is the number of
+// divisions and square roots.  A step's direction is formed once, not once per lag and partner, and
+// the autocorrelation, which ends at its first value <= 0, is not taken beyond it where the CTA
+// holds the directions of all its cells.  512 runs of 16 cells, 81 snapshots: 4.57 ms with a thread
+// per cell and the directions formed per lag, 0.62 ms so.
 __global__ void __launch_bounds__(kSumThreads) summarize_kernel(const ObserveItem *items, const int64_t *cells,
                                                                 int64_t rows, const int64_t *member, int n_items,
-                                                                int S1, int every, double *traj, double *out)
+                                                                int S1, int every, int cap, double *out)
 {
-    extern __shared__ double snap[];  // sV, sV2, sA, sA2, sN: S1 each
-    __shared__ double acc[A_N];
-    const int run = blockIdx.x;
+    extern __shared__ double sum_smem[];
+    __shared__ double part[kSumWarps][A_N];
+    __shared__ double pers_s;
+    __shared__ int open_s;
+    const int run = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const ObserveItem it = items[run];
-    double *sV = snap, *sV2 = snap + S1, *sA = snap + 2 * S1, *sA2 = snap + 3 * S1, *sN = snap + 4 * S1;
-    for (int i = threadIdx.x; i < 5 * S1; i += blockDim.x) snap[i] = 0.0;
-    for (int i = threadIdx.x; i < A_N; i += blockDim.x) acc[i] = 0.0;
+    // per snapshot: number of cells, V, V^2, A, A^2 over them
+    unsigned long long *snap = reinterpret_cast<unsigned long long *>(sum_smem);
+    // per warp: the track of its cell and the lengths of its 50-MCS displacements
+    double *X = sum_smem + 5 * S1 + warp * 3 * S1, *Y = X + S1, *F = Y + S1;
+    // per cell of the chunk: step directions ((0, 0) for a step of length 0 or a cell without a track)
+    double *U = sum_smem + (5 + 3 * kSumWarps) * S1;
+    for (int i = threadIdx.x; i < 5 * S1; i += blockDim.x) snap[i] = 0;
+    if (threadIdx.x == 0) {
+        pers_s = 0.5 * every;
+        open_s = 1;
+    }
     __syncthreads();
-    const int nx = (int)it.nx, ny = (int)it.ny;
+    const double nx = (double)it.nx, ny = (double)it.ny;
     const int lags[3] = {10, 50, 200};
     const int k50 = 50 % every == 0 ? 50 / every : 0;
     const int n_ac = S1 - 1 < kMaxLag + 1 ? S1 - 1 : kMaxLag + 1;  // lags 1 .. n_ac - 1
-    for (int c = 1 + threadIdx.x; c <= it.n_cells; c += blockDim.x) {
-        const int64_t row = it.row0 + c;
-        double *tr = traj + row * 2 * S1;
-        bool track = true;
-        double px = 0.0, py = 0.0, qx = 0.0, qy = 0.0, el = 0.0, eln = 0.0;
-        for (int s = 0; s < S1; ++s) {
-            const int64_t *r = cells + ((int64_t)s * rows + row) * kObsFields;
-            if (r[1] <= 0) {
-                track = false;
+    const bool one_chunk = it.n_cells <= cap;
+    double acc[A_N];
+#pragma unroll
+    for (int k = 0; k < A_N; ++k) acc[k] = 0.0;
+    double ac_sum = 0.0, ac_cnt = 0.0;   // of lag 1 + lane, over all chunks but where one holds all cells
+    for (int c0 = 1; c0 <= it.n_cells; c0 += cap) {
+        const int nc = it.n_cells - c0 + 1 < cap ? it.n_cells - c0 + 1 : cap;
+        for (int c = warp; c < nc; c += kSumWarps) {
+            const int64_t row = it.row0 + c0 + c;
+            double *UX = U + (size_t)c * 2 * S1, *UY = UX + S1;
+            bool present = true;
+            for (int s = lane; s < S1; s += 32) {
+                const int64_t *r = cells + ((int64_t)s * rows + row) * kObsFields;
+                const int64_t v = r[1];
+                if (v <= 0) {
+                    present = false;
+                    continue;
+                }
+                atomicAdd(snap + s, 1ull);
+                atomicAdd(snap + S1 + s, (unsigned long long)v);
+                atomicAdd(snap + 2 * S1 + s, (unsigned long long)(v * v));
+                atomicAdd(snap + 3 * S1 + s, (unsigned long long)r[5]);
+                atomicAdd(snap + 4 * S1 + s, (unsigned long long)(r[5] * r[5]));
+                const double V = (double)v, inv = 1.0 / V;
+                const double mx = quotient((double)r[2], V, inv), my = quotient((double)r[3], V, inv);
+                const double cxx = quotient((double)r[6], V, inv) - mx * mx;
+                const double cyy = quotient((double)r[7], V, inv) - my * my;
+                const double cxy = quotient((double)r[9], V, inv) - mx * my;
+                const double t2 = cxx + cyy, det = cxx * cyy - cxy * cxy;
+                const double disc = sqrt(fmax(t2 * t2 / 4.0 - det, 0.0));
+                const double l1 = t2 / 2.0 + disc, l2 = t2 / 2.0 - disc;
+                if (l2 > 1e-9) {
+                    acc[A_EL] += sqrt(l1 / l2);
+                    acc[A_EL + 1] += 1.0;
+                }
+                const uint32_t anchor = (uint32_t)r[0];  // below 2^31
+                X[s] = (double)(anchor % it.nx) + mx;
+                Y[s] = (double)(anchor / it.nx) + my;
+            }
+            present = __all_sync(0xffffffffu, present);
+            __syncwarp();
+            if (!present) {
+                for (int s = lane; s < S1; s += 32) UX[s] = UY[s] = 0.0;
+                __syncwarp();
                 continue;
             }
-            const double V = (double)r[1], A = (double)r[5];
-            atomicAdd(&sV[s], V);
-            atomicAdd(&sV2[s], V * V);
-            atomicAdd(&sA[s], A);
-            atomicAdd(&sA2[s], A * A);
-            atomicAdd(&sN[s], 1.0);
-            const double mx = (double)r[2] / V, my = (double)r[3] / V;
-            const double cxx = (double)r[6] / V - mx * mx, cyy = (double)r[7] / V - my * my;
-            const double cxy = (double)r[9] / V - mx * my;
-            const double t2 = cxx + cyy, det = cxx * cyy - cxy * cxy;
-            const double disc = sqrt(fmax(t2 * t2 / 4.0 - det, 0.0));
-            const double l1 = t2 / 2.0 + disc, l2 = t2 / 2.0 - disc;
-            if (l2 > 1e-9) {
-                el += sqrt(l1 / l2);
-                eln += 1.0;
+            // minimal-image steps, then the track as their running sum
+            for (int s = lane; s + 1 < S1; s += 32) {
+                double dx = X[s + 1] - X[s], dy = Y[s + 1] - Y[s];
+                if (fabs(dx) > 0.499 * nx) dx -= nx * rint(dx / nx);
+                if (fabs(dy) > 0.499 * ny) dy -= ny * rint(dy / ny);
+                UX[s] = dx;
+                UY[s] = dy;
             }
-            const double cx = (double)(r[0] % nx) + mx, cy = (double)(r[0] / nx) + my;
-            if (track) {
-                if (s > 0) {
-                    double dx = cx - qx, dy = cy - qy;
-                    dx -= nx * rint(dx / nx);
-                    dy -= ny * rint(dy / ny);
-                    px += dx;
-                    py += dy;
+            __syncwarp();
+            if (lane < 2) {
+                double *T = lane == 0 ? X : Y;
+                const double *D = lane == 0 ? UX : UY;
+                double p = 0.0;
+                T[0] = 0.0;
+                for (int s = 0; s + 1 < S1; ++s) {
+                    p += D[s];
+                    T[s + 1] = p;
                 }
-                tr[2 * s] = px;
-                tr[2 * s + 1] = py;
             }
-            qx = cx;
-            qy = cy;
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int k = lags[j] % every ? 0 : lags[j] / every;
+                if (k <= 0 || k >= S1) continue;
+                for (int s = lane; s + k < S1; s += 32) {
+                    const double dx = X[s + k] - X[s], dy = Y[s + k] - Y[s];
+                    acc[A_MSD + j] += dx * dx + dy * dy;
+                }
+                if (lane == 0) acc[A_MSD + 3 + j] += (double)(S1 - k);
+            }
+            double path = 0.0;
+            for (int s = lane; s < S1; s += 32) {
+                double ux = 0.0, uy = 0.0;
+                if (s + 1 < S1) {
+                    const double dx = X[s + 1] - X[s], dy = Y[s + 1] - Y[s];
+                    const double sq = dx * dx + dy * dy, nrm = sqrt(sq);
+                    path += nrm;
+                    acc[A_SP + 1] += sq;
+                    if (nrm > 0.0) {
+                        const double inv = 1.0 / nrm;
+                        ux = quotient(dx, nrm, inv);
+                        uy = quotient(dy, nrm, inv);
+                    }
+                }
+                UX[s] = ux;
+                UY[s] = uy;
+            }
+            path = warp_sum(path);
+            if (lane == 0 && S1 > 1) {
+                acc[A_SP] += path;
+                acc[A_SP + 2] += (double)(S1 - 1);
+                if (path > 0.0) {
+                    const double ex = X[S1 - 1] - X[0], ey = Y[S1 - 1] - Y[0];
+                    acc[A_ST] += sqrt(ex * ex + ey * ey) / path;
+                    acc[A_ST + 1] += 1.0;
+                }
+            }
+            if (k50 > 0 && 2 * k50 < S1) {
+                for (int s = lane; s + k50 < S1; s += 32) {
+                    const double ax = X[s + k50] - X[s], ay = Y[s + k50] - Y[s];
+                    const double na = sqrt(ax * ax + ay * ay);
+                    F[s] = na;
+                    acc[A_SLOW] += na / 50.0 < kArrestSpeed ? 1.0 : 0.0;
+                }
+                if (lane == 0) acc[A_SLOW + 1] += (double)(S1 - k50);
+                __syncwarp();
+                for (int s = lane; s + 2 * k50 < S1; s += 32) {
+                    const double ax = X[s + k50] - X[s], ay = Y[s + k50] - Y[s];
+                    const double bx = X[s + 2 * k50] - X[s + k50], by = Y[s + 2 * k50] - Y[s + k50];
+                    const double na = F[s], nb = F[s + k50];
+                    if (na > 0.0 && nb > 0.0) {
+                        acc[A_DAC] += (ax * bx + ay * by) / (na * nb);
+                        acc[A_DAC + 1] += 1.0;
+                    }
+                }
+            }
+            __syncwarp();
         }
-        atomicAdd(&acc[A_EL], el);
-        atomicAdd(&acc[A_EL + 1], eln);
-        if (!track) continue;
-        for (int j = 0; j < 3; ++j) {
-            if (lags[j] % every) continue;
-            const int k = lags[j] / every;
-            if (k <= 0 || k >= S1) continue;
+        __syncthreads();
+        // direction cosines of the chunk, lag by lag
+        for (int k = 1; k < n_ac; ++k) {
             double sum = 0.0;
-            for (int s = 0; s + k < S1; ++s) {
-                const double dx = tr[2 * (s + k)] - tr[2 * s], dy = tr[2 * (s + k) + 1] - tr[2 * s + 1];
-                sum += dx * dx + dy * dy;
+            int cnt = 0;
+            for (int c = warp; c < nc; c += kSumWarps) {
+                const double *UX = U + (size_t)c * 2 * S1, *UY = UX + S1;
+                for (int s = lane; s + k + 1 < S1; s += 32) {
+                    const double ax = UX[s], ay = UY[s], bx = UX[s + k], by = UY[s + k];
+                    sum = fma(ax, bx, fma(ay, by, sum));
+                    // a direction is (0, 0) only where there is none (no step)
+                    cnt += (ax != 0.0 || ay != 0.0) && (bx != 0.0 || by != 0.0) ? 1 : 0;
+                }
             }
-            atomicAdd(&acc[A_MSD + j], sum);
-            atomicAdd(&acc[A_MSD + 3 + j], (double)(S1 - k));
+            sum = warp_sum(sum);
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (one_chunk) {
+                if (lane == 0) {
+                    part[warp][A_AC] = sum;
+                    part[warp][A_AC + 1] = (double)cnt;
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    double cs = 0.0, cc = 0.0;
+                    for (int w = 0; w < kSumWarps; ++w) {
+                        cs += part[w][A_AC];
+                        cc += part[w][A_AC + 1];
+                    }
+                    const double ck = cc > 0.0 ? cs / cc : 0.0;
+                    if (ck > 0.0) pers_s += ck * every; else open_s = 0;
+                }
+                __syncthreads();
+                if (!open_s) break;
+            } else if (lane == k - 1) {
+                ac_sum += sum;
+                ac_cnt += (double)cnt;
+            }
         }
-        if (S1 > 1) {
-            double ssum = 0.0, ssq = 0.0, path = 0.0;
-            for (int s = 0; s + 1 < S1; ++s) {
-                const double dx = tr[2 * s + 2] - tr[2 * s], dy = tr[2 * s + 3] - tr[2 * s + 1];
-                const double nrm = sqrt(dx * dx + dy * dy);
-                ssum += nrm / every;
-                ssq += (nrm / every) * (nrm / every);
-                path += nrm;
-            }
-            atomicAdd(&acc[A_SP], ssum);
-            atomicAdd(&acc[A_SP + 1], ssq);
-            atomicAdd(&acc[A_SP + 2], (double)(S1 - 1));
-            if (path > 0.0) {
-                const double nx_ = tr[2 * (S1 - 1)] - tr[0], ny_ = tr[2 * (S1 - 1) + 1] - tr[1];
-                atomicAdd(&acc[A_ST], sqrt(nx_ * nx_ + ny_ * ny_) / path);
-                atomicAdd(&acc[A_ST + 1], 1.0);
-            }
+        __syncthreads();
+    }
+    if (!one_chunk) {
+        // the lags' totals over the warps, through the chunk's storage (at least 2 S1 doubles; 2 x 4 x 20 used)
+        double *tot = U;
+        if (lane < kMaxLag) {
+            tot[(warp * kMaxLag + lane) * 2] = ac_sum;
+            tot[(warp * kMaxLag + lane) * 2 + 1] = ac_cnt;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
             for (int k = 1; k < n_ac; ++k) {
-                double sum = 0.0, cnt = 0.0;
-                for (int s = 0; s + k + 1 < S1; ++s) {
-                    const double ax = tr[2 * s + 2] - tr[2 * s], ay = tr[2 * s + 3] - tr[2 * s + 1];
-                    const double bx = tr[2 * (s + k) + 2] - tr[2 * (s + k)];
-                    const double by = tr[2 * (s + k) + 3] - tr[2 * (s + k) + 1];
-                    const double na = sqrt(ax * ax + ay * ay), nb = sqrt(bx * bx + by * by);
-                    if (na > 0.0 && nb > 0.0) {
-                        sum += (ax / na) * (bx / nb) + (ay / na) * (by / nb);
-                        cnt += 1.0;
-                    }
+                double cs = 0.0, cc = 0.0;
+                for (int w = 0; w < kSumWarps; ++w) {
+                    cs += tot[(w * kMaxLag + k - 1) * 2];
+                    cc += tot[(w * kMaxLag + k - 1) * 2 + 1];
                 }
-                atomicAdd(&acc[A_AC + k], sum);
-                atomicAdd(&acc[A_ACN + k], cnt);
+                const double ck = cc > 0.0 ? cs / cc : 0.0;
+                if (!(ck > 0.0)) break;
+                pers_s += ck * every;
             }
-        }
-        if (k50 > 0 && 2 * k50 < S1) {
-            double dsum = 0.0, dcnt = 0.0, slow = 0.0;
-            for (int s = 0; s + k50 < S1; ++s) {
-                const double ax = tr[2 * (s + k50)] - tr[2 * s], ay = tr[2 * (s + k50) + 1] - tr[2 * s + 1];
-                const double na = sqrt(ax * ax + ay * ay);
-                slow += na / 50.0 < kArrestSpeed ? 1.0 : 0.0;
-                if (s + 2 * k50 < S1) {
-                    const double bx = tr[2 * (s + 2 * k50)] - tr[2 * (s + k50)];
-                    const double by = tr[2 * (s + 2 * k50) + 1] - tr[2 * (s + k50) + 1];
-                    const double nb = sqrt(bx * bx + by * by);
-                    if (na > 0.0 && nb > 0.0) {
-                        dsum += (ax * bx + ay * by) / (na * nb);
-                        dcnt += 1.0;
-                    }
-                }
-            }
-            atomicAdd(&acc[A_DAC], dsum);
-            atomicAdd(&acc[A_DAC + 1], dcnt);
-            atomicAdd(&acc[A_SLOW], slow);
-            atomicAdd(&acc[A_SLOW + 1], (double)(S1 - k50));
         }
     }
+#pragma unroll
+    for (int k = 0; k < A_AC; ++k) {
+        const double v = warp_sum(acc[k]);
+        if (lane == 0) part[warp][k] = v;
+    }
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (warp != 0) return;
+    // per-snapshot figures, lanes over the snapshots
+    double tv = 0.0, ta = 0.0, tn = 0.0, vv = 0.0, av = 0.0, nv = 0.0, cf = 0.0, cfn = 0.0;
+    for (int s = lane; s < S1; s += 32) {
+        const double n = (double)snap[s], sV = (double)snap[S1 + s], sA = (double)snap[3 * S1 + s];
+        tv += sV;
+        ta += sA;
+        tn += n;
+        if (n > 0.0) {
+            const double mv = sV / n, ma = sA / n;
+            vv += fmax((double)snap[2 * S1 + s] / n - mv * mv, 0.0);
+            av += fmax((double)snap[4 * S1 + s] / n - ma * ma, 0.0);
+            nv += 1.0;
+        }
+        const double cm = (double)member[2 * ((int64_t)s * n_items + run)];
+        const double cc = (sA - cm) / 2.0, tot = cc + cm;
+        if (tot > 0.0) {
+            cf += cc / tot;
+            cfn += 1.0;
+        }
+    }
+    tv = warp_sum(tv);
+    ta = warp_sum(ta);
+    tn = warp_sum(tn);
+    vv = warp_sum(vv);
+    av = warp_sum(av);
+    nv = warp_sum(nv);
+    cf = warp_sum(cf);
+    cfn = warp_sum(cfn);
+    if (lane != 0) return;
+    double t[A_AC];
+#pragma unroll
+    for (int k = 0; k < A_AC; ++k) {
+        t[k] = 0.0;
+        for (int w = 0; w < kSumWarps; ++w) t[k] += part[w][k];
+    }
     const double qnan = __longlong_as_double(0x7ff8000000000000ll);
     double *o = out + (int64_t)run * kSummaryStats;
     for (int k = 0; k < kSummaryStats; ++k) o[k] = qnan;
-    double tv = 0.0, ta = 0.0, tn = 0.0, vv = 0.0, av = 0.0, nv = 0.0;
-    for (int s = 0; s < S1; ++s) {
-        tv += sV[s];
-        ta += sA[s];
-        tn += sN[s];
-        if (sN[s] > 0.0) {
-            const double mv = sV[s] / sN[s], ma = sA[s] / sN[s];
-            vv += fmax(sV2[s] / sN[s] - mv * mv, 0.0);
-            av += fmax(sA2[s] / sN[s] - ma * ma, 0.0);
-            nv += 1.0;
-        }
-    }
     // a statistic scaled by a target of 0 (no volume or perimeter constraint) is undefined: NaN
     if (tn > 0.0) {
         if (it.v_ref != 0.0) o[0] = tv / tn / it.v_ref;
@@ -301,41 +506,24 @@ __global__ void __launch_bounds__(kSumThreads) summarize_kernel(const ObserveIte
         if (it.a_ref != 0.0) o[3] = sqrt(av / nv) / it.a_ref;
     }
     for (int j = 0; j < 3; ++j)
-        if (acc[A_MSD + 3 + j] > 0.0) o[4 + j] = acc[A_MSD + j] / acc[A_MSD + 3 + j];
-    if (acc[A_SP + 2] > 0.0) {
-        const double m = acc[A_SP] / acc[A_SP + 2];
+        if (t[A_MSD + 3 + j] > 0.0) o[4 + j] = t[A_MSD + j] / t[A_MSD + 3 + j];
+    if (t[A_SP + 2] > 0.0) {
+        const double m = t[A_SP] / every / t[A_SP + 2];
         o[7] = m;
-        o[8] = sqrt(fmax(acc[A_SP + 1] / acc[A_SP + 2] - m * m, 0.0));
+        o[8] = sqrt(fmax(t[A_SP + 1] / ((double)every * every) / t[A_SP + 2] - m * m, 0.0));
     }
-    if (acc[A_DAC + 1] > 0.0) o[9] = acc[A_DAC] / acc[A_DAC + 1];
-    if (S1 > 1) {
-        double pers = 0.5 * every;
-        for (int k = 1; k < n_ac; ++k) {
-            const double ck = acc[A_ACN + k] > 0.0 ? acc[A_AC + k] / acc[A_ACN + k] : 0.0;
-            if (!(ck > 0.0)) break;
-            pers += ck * every;
-        }
-        o[10] = pers;
-    }
-    if (acc[A_SLOW + 1] > 0.0) o[11] = acc[A_SLOW] / acc[A_SLOW + 1];
+    if (t[A_DAC + 1] > 0.0) o[9] = t[A_DAC] / t[A_DAC + 1];
+    if (S1 > 1) o[10] = pers_s;
+    if (t[A_SLOW + 1] > 0.0) o[11] = t[A_SLOW] / t[A_SLOW + 1];
     if (S1 > 1) {
         const int64_t m0 = member[2 * (int64_t)run + 1];
         const int64_t m1 = member[2 * ((int64_t)(S1 - 1) * n_items + run) + 1];
         const double sites = (double)it.nx * it.ny * it.nz;
         o[12] = (double)(m1 - m0) / ((double)(S1 - 1) * every * sites);
     }
-    double cf = 0.0, cfn = 0.0;
-    for (int s = 0; s < S1; ++s) {
-        const double cm = (double)member[2 * ((int64_t)s * n_items + run)];
-        const double cc = (sA[s] - cm) / 2.0, tot = cc + cm;
-        if (tot > 0.0) {
-            cf += cc / tot;
-            cfn += 1.0;
-        }
-    }
     if (cfn > 0.0) o[13] = cf / cfn;
-    if (acc[A_ST + 1] > 0.0) o[14] = acc[A_ST] / acc[A_ST + 1];
-    if (acc[A_EL + 1] > 0.0) o[15] = acc[A_EL] / acc[A_EL + 1];
+    if (t[A_ST + 1] > 0.0) o[14] = t[A_ST] / t[A_ST + 1];
+    if (t[A_EL + 1] > 0.0) o[15] = t[A_EL] / t[A_EL + 1];
 }
 
 // Persistence update (Eq. 6, Eq. 7) for every cell, one thread per cell,
@@ -406,20 +594,22 @@ cudaError_t launch_pers_update(const int64_t *cells, int32_t n_cells, uint32_t n
 }
 
 cudaError_t launch_summarize(const ObserveItem *d_items, uint32_t n_items, int32_t max_cells, const int64_t *cells,
-                             int64_t rows, const int64_t *member, int32_t n_snap, int32_t every, double *traj,
-                             double *out, cudaStream_t st)
+                             int64_t rows, const int64_t *member, int32_t n_snap, int32_t every, double *out,
+                             cudaStream_t st)
 {
     if (n_items == 0) return cudaSuccess;
     if (n_snap < 1 || n_snap > kSummaryMaxSnap || every < 1) return cudaErrorInvalidValue;
-    int threads = ((max_cells + 31) / 32) * 32;
-    threads = threads < 32 ? 32 : (threads > kSumThreads ? kSumThreads : threads);
-    const size_t smem = sizeof(double) * 5 * (size_t)n_snap;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(summarize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    summarize_kernel<<<n_items, threads, smem, st>>>(d_items, cells, rows, member, (int)n_items, n_snap, every, traj,
-                                                     out);
+    // cells whose step directions are held at a time, and room for the lags' totals of several chunks
+    const size_t per_cell = sizeof(double) * 2 * (size_t)n_snap;
+    size_t cap = kSumUnitBytes / per_cell;
+    cap = cap < 1 ? 1 : (cap > (size_t)max_cells ? (max_cells > 0 ? (size_t)max_cells : 1) : cap);
+    size_t units = cap * per_cell;
+    if (units < sizeof(double) * 2 * kSumWarps * kMaxLag) units = sizeof(double) * 2 * kSumWarps * kMaxLag;
+    const size_t smem = sizeof(double) * (5 + 3 * kSumWarps) * (size_t)n_snap + units;
+    const cudaError_t e = cudaFuncSetAttribute(summarize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    summarize_kernel<<<n_items, kSumThreads, smem, st>>>(d_items, cells, rows, member, (int)n_items, n_snap, every,
+                                                         (int)cap, out);
     return cudaPeekAtLastError();
 }
 
@@ -429,12 +619,18 @@ cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items
     if (n_items == 0) return cudaSuccess;
     if (n_items > 65535u) return cudaErrorInvalidValue;
     observe_init_kernel<<<n_items, 256, 0, st>>>(d_items, cells, member);
-    int64_t bx = (max_sites + kObsThreads - 1) / kObsThreads;
-    if (bx > 64) bx = 64;
+    // a walk per thread, for the largest member; a few CTAs per SM in all
+    int64_t bx = (max_sites / kWalk + kObsThreads - 1) / kObsThreads + 1;
+    const int64_t most = 152 * 16 / (int64_t)n_items + 16;
+    if (bx > most) bx = most;
     const dim3 grid((unsigned)bx, n_items);
-    observe_anchor_kernel<<<grid, kObsThreads, 0, st>>>(d_items, cells);
-    if (dim == 3) observe_sums_kernel<3><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
-    else observe_sums_kernel<2><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+    if (dim == 3) {
+        observe_anchor_kernel<3><<<grid, kObsThreads, 0, st>>>(d_items, cells);
+        observe_sums_kernel<3><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+    } else {
+        observe_anchor_kernel<2><<<grid, kObsThreads, 0, st>>>(d_items, cells);
+        observe_sums_kernel<2><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+    }
     return cudaPeekAtLastError();
 }
 
