@@ -348,6 +348,55 @@ int run_subpass(cpm_handle *h)
     return CPM_OK;
 }
 
+// Whether a lattice's rounds run as spans, and how: at most 16 x 256 attempts per round, one each per
+// thread of the largest cluster (with two each a launch per round is faster: 320^2 points 5.1 against 3.3
+// us per round, 3D tissue of 320^3 11.7 against 10.3).
+bool pick_span(const cpm_handle *h, SpanPos &p)
+{
+    if (h->n_active > 4096u) return false;
+    p.per_mcs = h->per_mcs;
+    p.C = h->C;
+    p.k = h->k;
+    p.n_cells = h->n_cells;
+    const uint64_t resident = span_bytes(h->n_sites, h->n_cells, h->n_active);
+    const bool fits = resident <= kSpanMaxSmem;
+    p.nc = 1;
+    while (p.nc < 16 && h->n_active > (fits ? 128u : 32u) * p.nc) p.nc *= 2;
+    p.resident = p.nc == 1 && fits ? (uint32_t)resident : 0;
+    p.lanes = ((h->n_active + p.nc - 1) / p.nc + 31) / 32 * 32;
+    p.threads = std::min(2 * p.lanes, kSpanThreads);
+    return true;
+}
+
+// n schedule units of the global schedule on a lattice that runs as spans
+int run_spans(cpm_handle *h, int64_t n, SpanPos p)
+{
+    RoundArgs args = round_args(h);
+    if (p.resident) args.stream_loads = 0;  // its words are in shared memory
+    while (n > 0) {
+        // up to the end of the MCS where something follows it, and some tens of milliseconds per launch at most
+        int64_t m = std::min<int64_t>(n, std::max<int64_t>(1, 32768 / (int64_t)h->k));
+        if (h->csum || h->pers) m = std::min<int64_t>(m, (int64_t)h->per_mcs - h->sp);
+        p.t = (uint32_t)h->t;
+        p.sp = (uint32_t)h->sp;
+        p.n_sub = (uint32_t)m;
+        p.par = (uint32_t)(h->g & 1);
+        const LatticeBufs l = lattice_bufs(h);
+        CUDA_TRY(h, h->dim == 3 ? launch_span_3d(h->perim, h->act, args, l, p, h->stream)
+                                : launch_span_2d(h->perim, h->act, args, l, p, h->stream));
+        h->launches += 1;
+        h->g += (uint64_t)m * h->k;
+        h->attempts += m * (int64_t)h->k * h->n_active;
+        const int64_t sp = h->sp + m;
+        h->t += sp / h->per_mcs;
+        h->sp = (int32_t)(sp % h->per_mcs);
+        n -= m;
+        if (h->sp == 0)
+            if (int rc = end_of_mcs(h)) return rc;
+    }
+    return CPM_OK;
+}
+
 // Tile grid offset of MCS t: per axis a multiple of a below T, from counter (0, 0, t, 2<<24).
 void tile_offset(const cpm_handle *h, int64_t t, uint32_t off[3])
 {
@@ -753,6 +802,8 @@ int cpm_step_subpasses(cpm_handle *h, int64_t n)
 {
     if (bad(h)) return CPM_E_HANDLE;
     if (n < 0) return fail(h, CPM_E_INVALID, "n must be >= 0");
+    SpanPos span{};
+    if (!h->tile && pick_span(h, span)) return run_spans(h, n, span);
     for (int64_t i = 0; i < n; i++) {
         int rc = h->tile ? run_epoch(h) : run_subpass(h);
         if (rc) return rc;
@@ -1018,6 +1069,8 @@ struct cpm_batch {
     int *d_err = nullptr;                // barrier timeout flag
     uint32_t loop_grid = 0;              // CTAs of the last persistent launch
     bool track = false;                  // composite variable tracking in every member
+    uint32_t span_threads = 0;           // threads of a CTA there
+    uint32_t span_smem = 0;              // shared memory per CTA where every member runs in one CTA, else 0
     bool descriptors_dirty = true;
     int64_t launches = 0;
     std::string err;
@@ -1252,6 +1305,19 @@ int cpm_batch_create(const cpm_config *cfgs, int32_t n, void *cuda_stream, cpm_b
         delete b;
         return bfail(nullptr, e == cudaErrorMemoryAllocation ? CPM_E_NOMEM : CPM_E_CUDA, cudaGetErrorString(e));
     }
+    // members small enough for a CTA each: a lattice in shared memory and an attempt per thread, or up to three
+    // where two members or more fall to every SM (64 runs of 96 x 96 sites take 2.1 times as long as with a launch
+    // per round, 300 of them 7% less, 2,048 25% less)
+    for (const cpm_handle *h : b->hs) {
+        const uint64_t bytes = span_bytes(h->n_sites, h->n_cells, h->n_active);
+        if (bytes > kSpanMaxSmem || h->n_active > (n >= 304 ? 3 : 1) * kBatchSpanThreads) {
+            b->span_smem = 0;
+            break;
+        }
+        b->span_smem = std::max<uint32_t>(b->span_smem, (uint32_t)bytes);
+        b->span_threads = std::max<uint32_t>(b->span_threads,
+                                             std::min(kBatchSpanThreads, (h->n_active + 31) / 32 * 32));
+    }
     n_colours = 0;
     for (BatchLattice &L : b->lats) {
         L.colours = b->d_colours + n_colours;
@@ -1324,6 +1390,19 @@ int cpm_batch_step(cpm_batch *b, int64_t n_mcs)
                              "a grid-barrier wait of the persistent loop timed out; the lattices are in an unspecified "
                              "state");
             done += chunk;
+        }
+    } else if (b->span_smem && !b->track) {
+        for (int64_t done = 0; done < n_mcs;) {
+            const uint32_t m = (uint32_t)std::min<int64_t>(n_mcs - done, 256);
+            const uint32_t n = (uint32_t)b->lats.size();
+            cudaError_t e = b->dim == 3
+                                ? launch_batch_span_3d(b->perim, b->act, b->d_lats, n, m, b->span_threads, b->span_smem,
+                                                       b->stream)
+                                : launch_batch_span_2d(b->perim, b->act, b->d_lats, n, m, b->span_threads, b->span_smem,
+                                                       b->stream);
+            if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
+            b->launches += 1;
+            done += m;
         }
     } else {
         if (!b->graph) {

@@ -161,6 +161,7 @@ struct RoundArgs {
     uint32_t brick_lx, brick_ly, brick_lz;  // log2 of the active blocks per CTA along each axis
     uint32_t nbr_x, nbr_y;     // bricks along x and y where the grid is linear, else 0
     uint32_t uni;              // the type of every cell when they all share one, else 0
+    uint32_t narrow;           // 1: every type's weights and targets admit the 32-bit products of the round kernels
     float h_scale, h_eps;      // the test's logarithm: 16 T ln 2, and the margin within which the table decides
     const int16_t *chem;       // chemotaxis field, dim int16 per site (Q14), or null
     const double *pers_dir;    // persistence directions, 3 per cell id, or null
@@ -195,6 +196,29 @@ __host__ __device__ __forceinline__ RoundBufs round_bufs(const LatticeBufs &l, u
     return b;
 }
 
+// A span of rounds of one lattice in one launch (cpm_span.cuh).
+constexpr uint32_t kSpanThreads = 512;         // most threads of a CTA
+constexpr uint32_t kSpanMaxSmem = 200 * 1024;  // most dynamic shared memory (a resident lattice)
+struct SpanPos {
+    uint32_t t, sp;            // MCS (low 32 bits) and sub-pass of the first round
+    uint32_t per_mcs, C, k;    // sub-passes per MCS, colours, rounds per sub-pass
+    uint32_t n_sub;            // sub-passes to run (>= 1)
+    uint32_t par;              // parity of the first round's index
+    uint32_t nc, lanes;        // CTAs of the cluster, attempts per CTA and stripe (<= 256, a multiple of 32)
+    uint32_t threads;          // of a CTA
+    uint32_t resident;         // bytes of shared memory that hold the lattice (nc = 1), or 0
+    int32_t n_cells;
+};
+// shared memory of a resident lattice: words, both buffers of the tallies, both of the flags
+inline uint64_t span_bytes(uint64_t n_sites, int32_t n_cells, uint32_t n_active)
+{
+    return (4 * n_sites + 16 * ((uint64_t)n_cells + 1) + 2 * (uint64_t)n_active + 15) / 16 * 16;
+}
+cudaError_t launch_span_2d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,
+                           cudaStream_t st);
+cudaError_t launch_span_3d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,
+                           cudaStream_t st);
+
 // Batched ensembles: one lattice of the batch; the round of lattice l at batch step q is round
 // g_start + q of that lattice, in MCS t_start.
 constexpr uint32_t kBatchMaxThreads = 256;
@@ -207,6 +231,12 @@ struct BatchLattice {
     uint64_t g_start;
     uint8_t *colours;    // colour of every sub-pass of the current MCS (R / k entries, see launch_batch_colours)
 };
+// n_mcs MCS of every member in one launch, a CTA of `threads` each (cpm_span.cuh); smem: the largest member's span_bytes
+constexpr uint32_t kBatchSpanThreads = 256;  // most threads of a CTA
+cudaError_t launch_batch_span_2d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
+                                 uint32_t smem, cudaStream_t st);
+cudaError_t launch_batch_span_3d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
+                                 uint32_t smem, cudaStream_t st);
 // after_round: the kernel before it on the stream is a round of the same MCS (programmatic dependent launch)
 cudaError_t launch_batch_round(int dim, bool perim, bool act, bool track, const BatchLattice *lats,
                                const int4 *items, uint32_t n_items, uint32_t q, uint32_t threads, bool after_round,
@@ -321,7 +351,7 @@ inline void pick_bricks(int dim, RoundArgs &a)
     }
 }
 
-// The fields of RoundArgs that follow from the schedule and the temperature alone.
+// The fields of RoundArgs that follow from the schedule, the model (a.tp) and the temperature.
 inline void fill_round_constants(RoundArgs &a, double temperature)
 {
     a.s_log2 = 32;
@@ -329,6 +359,15 @@ inline void fill_round_constants(RoundArgs &a, double temperature)
         if (a.s == (1u << k)) a.s_log2 = k;
     a.h_scale = (float)(16.0 * 0.69314718055994531 * temperature);
     a.h_eps = (float)(1.0 + 1e-3 * temperature);
+    // 2 lambda_V, 52 lambda_P, 2 V_t and 2 A_t (and their sums with 26) in 32 bits, lambda_Act < 2^19
+    a.narrow = 1;
+    for (int t = 0; t < kMaxTypes; t++) {
+        const auto within = [](int32_t v, int32_t m) { return v > -m && v < m; };
+        if (!within(a.tp.lambda_v[t], 1 << 30) || !within(a.tp.lambda_p[t], 1 << 25) ||
+            !within(a.tp.lambda_act[t], 1 << 19) || !within(a.tp.v_target[t], 1 << 29) ||
+            !within(a.tp.a_target[t], 1 << 29))
+            a.narrow = 0;
+    }
 }
 
 // Launchers (defined in the per-dimension translation units).

@@ -198,7 +198,6 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
     a.n_active = (uint32_t)n_active;
     a.key0 = (uint32_t)c.seed;
     a.key1 = (uint32_t)(c.seed >> 32);
-    fill_round_constants(a, c.temperature);
     pick_bricks(c.dim, a);
     memcpy(a.tp.J, c.J, sizeof a.tp.J);
     memcpy(a.tp.lambda_v, c.lambda_v, sizeof a.tp.lambda_v);
@@ -208,6 +207,7 @@ extern "C" int cpm_step_noalloc(const cpm_config *cfg, int32_t *lattice, int32_t
     memcpy(a.tp.lambda_act, c.lambda_act, sizeof a.tp.lambda_act);
     memcpy(a.tp.max_act, c.max_act, sizeof a.tp.max_act);
     a.tp.obstacle_type = c.obstacle_type;
+    fill_round_constants(a, c.temperature);
     bool perim = false;
     for (int k = 0; k < CPM_MAX_TYPES; k++)
         if (c.lambda_p[k]) perim = true;

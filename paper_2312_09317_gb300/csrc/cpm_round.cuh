@@ -13,26 +13,61 @@
 namespace cpmgb {
 namespace {
 
+// What the energy change needs of a type, in the order it is read (four 16-byte loads).
+struct __align__(16) TypeRow {
+    int32_t Ju, J0, Jf, lv2;  // adhesion with the cells' one type, the medium, obstacles; 2 lambda_V
+    int64_t cvi, cvj;         // lambda_V (1 - 2 V_t) for the gaining cell, lambda_V (1 + 2 V_t) for the losing one
+    int32_t lp, at2, la, ma;  // lambda_P, 2 A_t, lambda_Act, Max_Act
+    uint32_t div_m, div_s;    // floor(u / Max_Act) = u div_m >> div_s for u < 2^30
+    int32_t act_lo, gm_max;   // TypeParams::act_lo, gm_max
+};
+constexpr int kNoCell = kMaxTypes;  // the row of the medium: no volume, perimeter or Act term
+constexpr int kMaxCount = 27;       // sites of a 3^3 window
+
 struct SmemTables {
+    TypeRow row[kMaxTypes + 1];
     int32_t J[kMaxTypes * kMaxTypes];
-    int32_t lv[kMaxTypes], vt[kMaxTypes], lp[kMaxTypes], at[kMaxTypes], la[kMaxTypes], ma[kMaxTypes];
+    int32_t act_hi[kMaxTypes * kMaxTypes];
     int32_t ln[kLnEntries];
+    uint32_t inv[kMaxCount + 1];    // floor(n / d) = mulhi(2 n, inv[d]) for n < 2^31 / 27
 };
 
-__device__ __forceinline__ void load_tables(SmemTables &sm, const RoundArgs &a, bool with_ln)
+__device__ __forceinline__ void load_tables(SmemTables &sm, const RoundArgs &a, bool with_act)
 {
-    for (int k = threadIdx.x; k < kMaxTypes * kMaxTypes; k += blockDim.x) sm.J[k] = a.tp.J[k / kMaxTypes][k % kMaxTypes];
-    if (threadIdx.x < kMaxTypes) {
-        const int k = threadIdx.x;
-        sm.lv[k] = a.tp.lambda_v[k];
-        sm.vt[k] = a.tp.v_target[k];
-        sm.lp[k] = a.tp.lambda_p[k];
-        sm.at[k] = a.tp.a_target[k];
-        sm.la[k] = a.tp.lambda_act[k];
-        sm.ma[k] = a.tp.max_act[k];
+    for (int k = threadIdx.x; k < kMaxTypes * kMaxTypes; k += blockDim.x) {
+        sm.J[k] = a.tp.J[k / kMaxTypes][k % kMaxTypes];
+        if (with_act) sm.act_hi[k] = (int32_t)a.tp.act_hi[k / kMaxTypes][k % kMaxTypes];
     }
-    if (with_ln)
+    if (threadIdx.x <= kNoCell) {
+        const int k = threadIdx.x, t = k == kNoCell ? 0 : k;
+        TypeRow r{};
+        r.Ju = a.tp.J[t][a.uni];
+        r.J0 = a.tp.J[t][0];
+        r.Jf = a.tp.J[t][a.tp.obstacle_type];
+        if (k != kNoCell) {
+            const int64_t lv = a.tp.lambda_v[k], vt = a.tp.v_target[k];
+            r.lv2 = (int32_t)(2u * (uint32_t)a.tp.lambda_v[k]);
+            r.cvi = lv * (1 - 2 * vt);
+            r.cvj = lv * (1 + 2 * vt);
+            r.lp = a.tp.lambda_p[k];
+            r.at2 = (int32_t)(2u * (uint32_t)a.tp.a_target[k]);
+            r.la = a.tp.lambda_act[k];
+            r.ma = a.tp.max_act[k];
+            r.act_lo = (int32_t)a.tp.act_lo[k];
+            r.gm_max = a.tp.gm_max[k];
+            // M = ceil(2^(30+l) / Max) <= 2^31 with 2^l >= Max: the error u (M Max - 2^(30+l)) stays below 2^(30+l)
+            uint32_t l = 0;
+            while ((1 << l) < r.ma) ++l;
+            r.div_s = 30 + l;
+            r.div_m = r.ma > 0 ? (uint32_t)(((1ull << r.div_s) + r.ma - 1) / (uint32_t)r.ma) : 0u;
+        }
+        sm.row[k] = r;
+    }
+    if (with_act) {
         for (int k = threadIdx.x; k < kLnEntries; k += blockDim.x) sm.ln[k] = a.ln_tab[k];
+        // M = ceil(2^31 / d): the error 2 n (M d - 2^31) stays below 2^32 for n < 2^31 / 27
+        for (uint32_t d = 1 + threadIdx.x; d <= kMaxCount; d += blockDim.x) sm.inv[d] = (0x80000000u + d - 1) / d;
+    }
 }
 
 // Type of a lattice id.  When every cell has the same type (a.uni), it follows from the id alone,
@@ -77,16 +112,47 @@ __device__ __noinline__ int64_t floor_div_pos(int64_t num, int64_t den)
     return q;
 }
 
-// floor(num / (4096 mx)) for 1 <= mx <= 127: floor(floor(num / 4096) / mx), the second division in
-// 32 bits where the first quotient fits (any Act weight below 2^19 scaled), which keeps the 64-bit
-// division, some hundred instructions, off the usual path.
-__device__ __forceinline__ int64_t act_quotient(int64_t num, int32_t mx)
+// Energies in 64 bits, for any parameters; and in 32 bits with weights that RoundArgs::narrow admits,
+// where a sum is clamped to +-2^30 once: the Act term that follows is at most 16 lambda_Act < 2^23, and
+// every threshold lies below 2^22, so a clamped sum is decided as the sum itself.
+struct Wide {
+    using E = int64_t;
+    __device__ __forceinline__ static E energy(int64_t h) { return h; }
+    // floor(lambda_Act g / (4096 Max_Act))
+    __device__ __forceinline__ static E act(const TypeRow &r, int32_t g)
+    {
+        return floor_div_pos((int64_t)r.la * g, (int64_t)r.ma * 4096);
+    }
+    __device__ __forceinline__ static E act_lo(const RoundArgs &a, const SmemTables &, int t) { return a.tp.act_lo[t]; }
+    __device__ __forceinline__ static E act_hi(const RoundArgs &a, const SmemTables &, int t, int tj)
+    {
+        return a.tp.act_hi[t][tj];
+    }
+};
+struct Narrow {
+    using E = int32_t;
+    __device__ __forceinline__ static E energy(int64_t h)
+    {
+        const int64_t m = 1 << 30;
+        return (int32_t)(h > m ? m : (h < -m ? -m : h));
+    }
+    // floor(floor(lambda_Act g / 4096) / Max_Act): the inner quotient is below 2^30 in magnitude, a negative one is
+    // divided as its complement
+    __device__ __forceinline__ static E act(const TypeRow &r, int32_t g)
+    {
+        const int32_t q = (int32_t)(((int64_t)r.la * g) >> 12), s = q >> 31;
+        return (int32_t)((uint64_t)(uint32_t)(q ^ s) * r.div_m >> r.div_s) ^ s;
+    }
+    __device__ __forceinline__ static E act_lo(const RoundArgs &, const SmemTables &sm, int t) { return sm.row[t].act_lo; }
+    __device__ __forceinline__ static E act_hi(const RoundArgs &, const SmemTables &sm, int t, int tj)
+    {
+        return sm.act_hi[t * kMaxTypes + tj];
+    }
+};
+// floor(sum / count) of an Act log-sum, as an index of EXPQ
+__device__ __forceinline__ uint32_t mean_index(const SmemTables &sm, int32_t sum, int32_t count)
 {
-    const int64_t q = num >> 12;
-    const int32_t q32 = (int32_t)q;
-    if (q != (int64_t)q32) return floor_div_pos(q, mx);
-    const int32_t s = q32 >> 31;  // floor for negative values: ~((~q) / mx)
-    return (int64_t)((int32_t)((uint32_t)(q32 ^ s) / (uint32_t)mx) ^ s);
+    return __umulhi(2u * (uint32_t)sum, sm.inv[count]) >> 6;
 }
 
 // Motility terms (Eq. 4, Eq. 5) of the copy from the source (stencil index
@@ -366,10 +432,11 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
 #pragma unroll
         for (int k = 0; k < K; ++k) wn[k] = Win::has(k, sub) ? lat_word<ACT>(a, b, s.off + win.step(k, sub)) : 0;
         const int ti = type_of(a, si), tj = type_of(a, sj);
+        const TypeRow &ri = sm.row[si > 0 ? ti : kNoCell], &rj = sm.row[sj > 0 ? tj : kNoCell];
         // Counts of the neighbours in sigma_i, in sigma_j, in the medium and on obstacles, a byte each.
         // Target's Act log-sum over its same-cell window: 24 bits (at most 26 x LN[127]), the number of
         // zero Act values above them.
-        const int maxj = ACT && sj > 0 ? (int)sm.ma[tj] : 0;
+        const int maxj = ACT ? rj.ma : 0;
         int32_t counts = 0, lsj = 0;
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -390,9 +457,9 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
         if (a.uni) {
             // every cell has one type: the adhesion follows from the counts
             const int n0 = (counts >> 16) & 255, nf = (counts >> 24) & 255, nc = NB - n0 - nf;
-            const int32_t *Ji = sm.J + ti * kMaxTypes, *Jj = sm.J + tj * kMaxTypes;
-            adhesion = Ji[a.uni] * (nc - (si > 0 ? mi : 0)) + Ji[0] * (n0 - (si > 0 ? 0 : mi)) + Ji[a.tp.obstacle_type] * nf;
-            adhesion -= Jj[a.uni] * (nc - (sj > 0 ? mj : 0)) + Jj[0] * (n0 - (sj > 0 ? 0 : mj)) + Jj[a.tp.obstacle_type] * nf;
+            const TypeRow &Ji = sm.row[ti], &Jj = sm.row[tj];
+            adhesion = Ji.Ju * (nc - (si > 0 ? mi : 0)) + Ji.J0 * (n0 - (si > 0 ? 0 : mi)) + Ji.Jf * nf;
+            adhesion -= Jj.Ju * (nc - (sj > 0 ? mj : 0)) + Jj.J0 * (n0 - (sj > 0 ? 0 : mj)) + Jj.Jf * nf;
         } else {
             adhesion = 0;
 #pragma unroll
@@ -406,14 +473,28 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
             adhesion = group_sum<G>(adhesion);
         }
         const int32_t Vi = __shfl_sync(0xffffffffu, tal, 0, G), Vj = __shfl_sync(0xffffffffu, tal, 1, G);
+        const int32_t Ai = PERIM ? __shfl_sync(0xffffffffu, tal, 2, G) : 0;
+        const int32_t Aj = PERIM ? __shfl_sync(0xffffffffu, tal, 3, G) : 0;
+        if (ACT) lsj = group_sum<G>(lsj);
         const int dAi = NB - 2 * mi, dAj = 2 * mj - NB;
+        // a cell of type t that grows by a site: lambda_V (2 (V - V_t) + 1), that shrinks: lambda_V (1 - 2 (V - V_t));
+        // its interfaces change by d: lambda_P d (2 (A - A_t) + d).  Products of 32-bit factors (RoundArgs::narrow
+        // says that they are), sums in 64 bits.
         int64_t dh = adhesion;
-        if (si > 0) dh += (int64_t)sm.lv[ti] * (2 * ((int64_t)Vi - sm.vt[ti]) + 1);
-        if (sj > 0) dh += (int64_t)sm.lv[tj] * (1 - 2 * ((int64_t)Vj - sm.vt[tj]));
-        if (PERIM) {
-            const int32_t Ai = __shfl_sync(0xffffffffu, tal, 2, G), Aj = __shfl_sync(0xffffffffu, tal, 3, G);
-            if (si > 0) dh += (int64_t)sm.lp[ti] * dAi * (2 * ((int64_t)Ai - sm.at[ti]) + dAi);
-            if (sj > 0) dh += (int64_t)sm.lp[tj] * dAj * (2 * ((int64_t)Aj - sm.at[tj]) + dAj);
+        if (a.narrow) {
+            dh += (int64_t)ri.lv2 * Vi + ri.cvi + rj.cvj - (int64_t)rj.lv2 * Vj;
+            if (PERIM) {
+                const int32_t pi = ri.lp * dAi, pj = rj.lp * dAj;
+                dh += (int64_t)pi * (dAi - ri.at2) + (int64_t)(2 * pi) * Ai + (int64_t)pj * (dAj - rj.at2) +
+                      (int64_t)(2 * pj) * Aj;
+            }
+        } else {
+            if (si > 0) dh += (int64_t)a.tp.lambda_v[ti] * (2 * ((int64_t)Vi - a.tp.v_target[ti]) + 1);
+            if (sj > 0) dh += (int64_t)a.tp.lambda_v[tj] * (1 - 2 * ((int64_t)Vj - a.tp.v_target[tj]));
+            if (PERIM && si > 0)
+                dh += (int64_t)a.tp.lambda_p[ti] * dAi * (2 * ((int64_t)Ai - a.tp.a_target[ti]) + dAi);
+            if (PERIM && sj > 0)
+                dh += (int64_t)a.tp.lambda_p[tj] * dAj * (2 * ((int64_t)Aj - a.tp.a_target[tj]) + dAj);
         }
         int64_t dhq = 16 * dh;
         const uint32_t dir = s.i_dir >> kDirShift<DIM>;
@@ -429,75 +510,74 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
         // h but the few within a.h_eps (over ten times its error bound) of that value, for which the
         // table is read; a test thus mostly ends without another dependent load.
         const float hs = a.h_scale * (32.0f - __log2f((float)s.w2 + 1.0f));
-        const int64_t h_lo = (int64_t)(int32_t)floorf(hs - a.h_eps), h_hi = (int64_t)(int32_t)ceilf(hs + a.h_eps);
-        const auto below = [&](int64_t h) {
+        const int32_t h_lo = (int32_t)floorf(hs - a.h_eps), h_hi = (int32_t)ceilf(hs + a.h_eps);
+        const auto below = [&](auto h) {
             if (h <= h_lo) return true;
             if (h > h_hi) return false;
             return h < a.L && s.w2 < __ldg(a.thr + h);
         };
-        // decided: 1 accept, 0 reject, -1 open
-        int decided = !on || (sj > 0 && Vj <= 1) ? 0 : -1;
-        if (ACT) {
-            lsj = group_sum<G>(lsj);
-            const int tp = si > 0 ? ti : tj;
-            const int64_t lam = sm.la[tp];
-            const int32_t mx = sm.ma[tp];
-            bool window = false;  // the source's window is needed
-            int64_t gj = 0;
-            if (decided < 0 && lam != 0 && mx != 0) {
-                // the Act term lies in [act_lo, act_hi] = [floor(-lam Gmax_i / (Max 4096)), floor(lam Gmax_j / (Max
-                // 4096))] (GM in [0, Gmax] per cell, lambda >= 0); when every value in that range gives the same
-                // outcome of the test below (THR is non-increasing), the geometric means are not needed
-                const int64_t lo = dhq + (si > 0 ? a.tp.act_lo[ti] : 0);
-                const int64_t hi = dhq + (sj > 0 ? a.tp.act_hi[tp][tj] : 0);
-                if (hi <= 0) decided = 1;
-                else if (lo > 0 && !below(lo)) decided = 0;
-                else if (below(hi)) decided = 1;
-                else {
-                    // target: the log-sum gathered above (the centre and the mj same-cell neighbours; 0 when any of
-                    // their Act values is 0)
-                    if (sj > 0) {
-                        const int cv = act_value(word_stamp(s.wj), t8, maxj);
-                        if (cv != 0 && lsj < 1 << 24)
-                            gj = (int64_t)__ldg(a.expq + ((uint32_t)(lsj + sm.ln[cv]) / (uint32_t)(mj + 1) >> 6));
+        const bool barred = !on || (sj > 0 && Vj <= 1);  // no survivor, or a cell's last site
+        const auto test = [&](auto arith) {
+            using Ar = decltype(arith);
+            using E = typename Ar::E;
+            E h = Ar::energy(dhq);
+            int decided = barred ? 0 : -1;  // 1 accept, 0 reject, -1 open
+            if (ACT) {
+                const int tp = si > 0 ? ti : tj;
+                const TypeRow &rm = sm.row[tp];  // of the moving cell
+                bool window = false;             // the source's window is needed
+                int32_t gj = 0;
+                if (decided < 0 && rm.la != 0 && rm.ma != 0) {
+                    // the Act term lies in [act_lo, act_hi] = [floor(-lam Gmax_i / (Max 4096)), floor(lam Gmax_j /
+                    // (Max 4096))] (GM in [0, Gmax] per cell, lambda >= 0); when every value in that range gives the
+                    // same outcome of the test (THR is non-increasing), the geometric means are not needed
+                    const E lo = h + (si > 0 ? Ar::act_lo(a, sm, ti) : 0), hi = h + (sj > 0 ? Ar::act_hi(a, sm, tp, tj) : 0);
+                    if (hi <= 0) decided = 1;
+                    else if (lo > 0 && !below(lo)) decided = 0;
+                    else if (below(hi)) decided = 1;
+                    else {
+                        // target: the log-sum gathered above (the centre and the mj same-cell neighbours; 0 when any
+                        // of their Act values is 0)
+                        if (sj > 0) {
+                            const int cv = act_value(word_stamp(s.wj), t8, maxj);
+                            if (cv != 0 && lsj < 1 << 24) gj = __ldg(a.expq + mean_index(sm, lsj + sm.ln[cv], mj + 1));
+                        }
+                        // the same with the target's mean known: [floor(lam (G_j - Gmax_i) / ..), floor(lam G_j / ..)]
+                        const E hi1 = h + Ar::act(rm, gj), lo1 = h + Ar::act(rm, gj - ri.gm_max);
+                        if (hi1 <= 0 || below(hi1)) decided = 1;
+                        else if (lo1 > 0 && !below(lo1)) decided = 0;
+                        else window = true;  // si > 0: otherwise lo1 = hi1, and one of the two holds
                     }
-                    // the same with the target's mean known: [floor(lam (G_j - Gmax_i) / ..), floor(lam G_j / ..)]
-                    const int64_t hi1 = dhq + act_quotient(lam * gj, mx);
-                    const int64_t lo1 = dhq + act_quotient(lam * (gj - (si > 0 ? a.tp.gm_max[ti] : 0)), mx);
-                    if (hi1 <= 0 || below(hi1)) decided = 1;
-                    else if (lo1 > 0 && !below(lo1)) decided = 0;
-                    else window = true;  // si > 0: otherwise lo1 = hi1, and one of the two holds
+                }
+                if (__any_sync(0xffffffffu, window)) {
+                    const uint32_t xi = wrap_step(s.x, ox - 1, a.nx), yi = wrap_step(s.y, oy - 1, a.ny);
+                    const uint32_t zi = DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0;
+                    const uint32_t src = site_off(a, xi, yi, zi);
+                    const Win win_i(a, sub, xi, yi, zi);
+#pragma unroll
+                    for (int k = 0; k < K; ++k)
+                        wn[k] = window && Win::has(k, sub) ? lat_word<ACT>(a, b, src + win_i.step(k, sub)) : 0;
+                    int32_t ci = 0, lsi = 0;
+#pragma unroll
+                    for (int k = 0; k < K; ++k)
+                        if (Win::has(k, sub) && cell_id(wn[k]) == si) {
+                            const int av = act_value(word_stamp(wn[k]), t8, ri.ma);
+                            ci += 1;
+                            lsi += av == 0 ? 1 << 24 : sm.ln[av];
+                        }
+                    ci = group_sum<G>(ci);
+                    lsi = group_sum<G>(lsi);
+                    if (window) {
+                        int32_t gi = 0;
+                        const int cv = act_value(word_stamp(s.wi), t8, ri.ma);
+                        if (cv != 0 && lsi < 1 << 24) gi = __ldg(a.expq + mean_index(sm, lsi + sm.ln[cv], ci + 1));
+                        h += Ar::act(rm, gj - gi);
+                    }
                 }
             }
-            if (__any_sync(0xffffffffu, window)) {
-                const uint32_t xi = wrap_step(s.x, ox - 1, a.nx), yi = wrap_step(s.y, oy - 1, a.ny);
-                const uint32_t zi = DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0;
-                const uint32_t src = site_off(a, xi, yi, zi);
-                const Win win_i(a, sub, xi, yi, zi);
-#pragma unroll
-                for (int k = 0; k < K; ++k)
-                    wn[k] = window && Win::has(k, sub) ? lat_word<ACT>(a, b, src + win_i.step(k, sub)) : 0;
-                const int maxi = sm.ma[ti];
-                int32_t ci = 0, lsi = 0;
-#pragma unroll
-                for (int k = 0; k < K; ++k)
-                    if (Win::has(k, sub) && cell_id(wn[k]) == si) {
-                        const int av = act_value(word_stamp(wn[k]), t8, maxi);
-                        ci += 1;
-                        lsi += av == 0 ? 1 << 24 : sm.ln[av];
-                    }
-                ci = group_sum<G>(ci);
-                lsi = group_sum<G>(lsi);
-                if (window) {
-                    int64_t gi = 0;
-                    const int cv = act_value(word_stamp(s.wi), t8, maxi);
-                    if (cv != 0 && lsi < 1 << 24)
-                        gi = (int64_t)__ldg(a.expq + ((uint32_t)(lsi + sm.ln[cv]) / (uint32_t)(ci + 1) >> 6));
-                    dhq += act_quotient(lam * (gj - gi), mx);
-                }
-            }
-        }
-        const bool ok = decided >= 0 ? decided == 1 : (dhq <= 0 || below(dhq));
+            return decided >= 0 ? decided == 1 : (h <= 0 || below(h));
+        };
+        const bool ok = a.narrow ? test(Narrow{}) : test(Wide{});
         const bool leader = sub == 0 && ok;
         if (leader) {
             const uint32_t i = s.i_dir & kIndexMask;
