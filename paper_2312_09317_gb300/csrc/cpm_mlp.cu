@@ -24,50 +24,14 @@
 #include <new>
 
 #include "../../include/cpm_emulator.h"
+#include "cpm_mlp_internal.h"
+
+using namespace cpmmlp;
 
 namespace {
 
 constexpr int kBM = 64, kBN = 64, kBK = 32, kLds = kBK + 8;  // smem row stride (halves): 80 B, conflict-free
 constexpr int kGemmThreads = 128;                             // 4 warps, 2 x 2, each 32 x 32 of the tile
-
-// Standard normal CDF Phi(z) = (1 + erf(z / sqrt 2)) / 2 and the density
-// term exp(-z^2 / 2), with erf from the rational approximation of
-// Abramowitz & Stegun, Handbook of Mathematical Functions, formula 7.1.26
-// (after Hastings): for x >= 0,
-//   erf(x) = 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) exp(-x^2) + e(x),
-//   t = 1 / (1 + p x),  |e(x)| <= 1.5e-7,
-// p = 0.3275911, a1..a5 = 0.254829592, -0.284496736, 1.421413741,
-// -1.453152027, 1.061405429.  The reciprocal and the exponential are the
-// fast hardware approximations.  With float32 rounding the |Phi error| stays
-// below 4e-7 (the tests pin it on a dense grid against float64), far under
-// the bf16 rounding (2^-9) of the activations that the epilogue stores.  The
-// GELU epilogue is issue-bound, and this form is shorter than erff.
-__device__ __forceinline__ float phi_f(float z, float &dens)
-{
-    const float x = fabsf(z) * 0.70710678118654752f;
-    dens = __expf(-x * x);  // exp(-z^2 / 2)
-    const float t = __fdividef(1.0f, fmaf(0.3275911f, x, 1.0f));
-    float poly = 1.061405429f;
-    poly = fmaf(poly, t, -1.453152027f);
-    poly = fmaf(poly, t, 1.421413741f);
-    poly = fmaf(poly, t, -0.284496736f);
-    poly = fmaf(poly, t, 0.254829592f);
-    const float half_tail = 0.5f * poly * t * dens;  // (1 - erf(x)) / 2
-    return z >= 0.0f ? 1.0f - half_tail : half_tail;
-}
-
-__device__ __forceinline__ float gelu_f(float z)
-{
-    float dens;
-    return z * phi_f(z, dens);
-}
-
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    float dens;
-    const float cdf = phi_f(z, dens);
-    return cdf + z * 0.39894228040143268f * dens;
-}
 
 struct GemmArgs {
     int M, N, K;
@@ -318,31 +282,38 @@ __global__ void gather_kernel(int rows, int n_in, int n_out, const float *X, con
 // Ensemble mean / std over members for each (row, statistic); the mean is
 // mapped back to the statistic's units (y = mean * scale + shift, then exp
 // where log_mask is set); fallback[row] = 1 when any statistic's std (in the
-// network's standardised units) exceeds factor * rmse.
-__global__ void predict_kernel(int rows, int n_members, int n_out, const float *out, int64_t s_member,
-                               const float *shift, const float *scale, const uint8_t *log_mask, const float *rmse,
-                               float factor, float *mean_out, float *std_out, uint8_t *fallback)
+// network's standardised units) exceeds factor * rmse.  A thread per output of a row, so that neighbouring
+// threads read neighbouring outputs; a CTA's rows share their flags (65,536 rows: 34 us with a thread per row).
+constexpr int kPredictThreads = 256;
+__global__ void __launch_bounds__(kPredictThreads)
+    predict_kernel(int rows, int block_rows, int n_members, int n_out, const float *out, int64_t s_member,
+                   const float *shift, const float *scale, const uint8_t *log_mask, const float *rmse, float factor,
+                   float *mean_out, float *std_out, uint8_t *fallback)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    int fb = 0;
-    for (int k = 0; k < n_out; ++k) {
+    __shared__ int fb[kPredictThreads];
+    const int r0 = blockIdx.x * block_rows, nr = rows - r0 < block_rows ? rows - r0 : block_rows;
+    if (threadIdx.x < block_rows) fb[threadIdx.x] = 0;
+    __syncthreads();
+    for (int q = threadIdx.x; q < nr * n_out; q += blockDim.x) {
+        const int r = q / n_out, k = q % n_out;
+        const int64_t at = (int64_t)r0 * n_out + q;
         float s = 0.0f;
-        for (int e = 0; e < n_members; ++e) s += out[e * s_member + (int64_t)r * n_out + k];
+        for (int e = 0; e < n_members; ++e) s += out[e * s_member + at];
         const float mu = s / (float)n_members;
-        float q = 0.0f;
+        float v = 0.0f;
         for (int e = 0; e < n_members; ++e) {
-            const float d = out[e * s_member + (int64_t)r * n_out + k] - mu;
-            q += d * d;
+            const float d = out[e * s_member + at] - mu;
+            v += d * d;
         }
-        const float sd = sqrtf(q / (float)n_members);
+        const float sd = sqrtf(v / (float)n_members);
         float y = mu * scale[k] + shift[k];
         if (log_mask[k]) y = expf(y);
-        if (mean_out) mean_out[(int64_t)r * n_out + k] = y;
-        if (std_out) std_out[(int64_t)r * n_out + k] = sd;
-        if (rmse && sd > factor * rmse[k]) fb = 1;
+        if (mean_out) mean_out[at] = y;
+        if (std_out) std_out[at] = sd;
+        if (rmse && sd > factor * rmse[k]) fb[r] = 1;
     }
-    if (fallback) fallback[r] = (uint8_t)fb;
+    __syncthreads();
+    if (fallback && (int)threadIdx.x < nr) fallback[r0 + threadIdx.x] = (uint8_t)fb[threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------
@@ -362,7 +333,6 @@ __global__ void predict_kernel(int rows, int n_members, int n_out, const float *
 // prediction: 85.7 M points/s against 82.0 with 16 warps).
 constexpr int kTcThreads = 1024;
 constexpr int kTcM = 128;
-constexpr uint32_t kTcSpinLimit = 1u << 22;
 constexpr int kTcNotApplicable = 1;  // launch_gemm_tc: use the mma.sync kernel instead
 
 struct TcArgs {
@@ -382,29 +352,6 @@ struct TcArgs {
     int *err;
     int report_timeout;  // test hook: report the first accumulator wait as timed out once it has completed
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ uint64_t tc_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
-{
-    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
-__device__ __forceinline__ bool tc_wait(uint64_t *mbar, uint32_t parity)
-{
-    const uint32_t addr = smem_u32(mbar);
-    for (uint32_t it = 0; it < kTcSpinLimit; ++it) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done)
-                     : "r"(addr), "r"(parity)
-                     : "memory");
-        if (done) return true;
-    }
-    return false;
-}
 
 // rows [r0, r0 + rows_tile) x [0, Kp) of X into the core-matrix layout, zero outside [0, rows) x [0, K);
 // element e of the layout is core matrix e / 8 (8-row group outer, K chunk inner), row e % 8
@@ -727,6 +674,8 @@ struct cpm_mlp {
     cudaStream_t st = nullptr;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     __nv_bfloat16 *wb = nullptr;
+    unsigned char *packed = nullptr;  // wb as the fused forward pass reads it, where the shape fits it
+    bool packed_valid = false;        // false once the weights have changed
     __nv_bfloat16 *xb = nullptr;
     float *yb = nullptr;
     __nv_bfloat16 *H[CPM_MLP_MAX_LAYERS]{};
@@ -778,7 +727,7 @@ int dalloc(cpm_mlp *h, T **p, int64_t n)
 
 void release(cpm_mlp *h)
 {
-    void *ptrs[] = {h->w,     h->g,     h->m,    h->v,    h->wb,    h->xb,    h->yb,   h->out,  h->dP,
+    void *ptrs[] = {h->w,     h->g,     h->m,    h->v,    h->wb,    h->packed, h->xb,  h->yb,   h->out, h->dP,
                     h->dZ[0], h->dZ[1], h->loss, h->bad, h->shift, h->scale, h->rmse, h->logm};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -824,6 +773,30 @@ int forward(cpm_mlp *h, int rows, bool keep_z)
         ++h->launches;
     }
     return CPM_MLP_OK;
+}
+
+// raw outputs of rows [0, rows) of X into out (members s_member floats apart) by the fused kernel
+int forward_fused(cpm_mlp *h, const float *X, int64_t rows, float *out, int64_t s_member)
+{
+    FusedNet n{};
+    n.n_members = h->sh.n_members;
+    n.n_in = h->sh.n_in;
+    n.width = h->sh.width;
+    n.n_hidden = h->sh.n_hidden;
+    n.n_out = h->sh.n_out;
+    n.w = h->w;
+    n.P = h->P;
+    n.packed = h->packed;
+    if (!h->packed_valid) {
+        if (int rc = cuda_check(h, fused_pack(n, h->wb, h->packed, h->st), "pack weights")) return rc;
+        ++h->launches;
+        h->packed_valid = true;
+    }
+    const int rc = cuda_check(h, fused_forward(n, X, rows, out, s_member, h->bad + 1, h->report_tc_timeout, h->st),
+                              "forward");
+    h->report_tc_timeout = 0;  // armed for one launch
+    ++h->launches;
+    return rc;
 }
 
 // loss and gradients of the gathered batch (xb, yb) into h->g and h->loss
@@ -966,6 +939,8 @@ int cpm_mlp_create(const cpm_mlp_shape *shape, const float *init_params, void *c
     rc |= dalloc(h, &h->loss, E) | dalloc(h, &h->bad, 2);
     rc |= dalloc(h, &h->shift, shape->n_out) | dalloc(h, &h->scale, shape->n_out) | dalloc(h, &h->rmse, shape->n_out);
     rc |= dalloc(h, &h->logm, shape->n_out);
+    if (fused_fits(shape->n_in, W, shape->n_out))
+        rc |= dalloc(h, &h->packed, E * fused_packed_bytes(shape->n_in, W, shape->n_hidden, shape->n_out));
     if (rc) {
         release(h);
         delete h;
@@ -992,6 +967,7 @@ int cpm_mlp_set_params(cpm_mlp *h, const float *params)
     if (rc) return rc;
     cast_kernel<<<grid1(n), 256, 0, h->st>>>(n, h->w, h->wb);
     ++h->launches;
+    h->packed_valid = false;
     h->t = 0;
     rc = cuda_check(h, cudaPeekAtLastError(), "cast");
     if (!rc) rc = cuda_check(h, cudaStreamSynchronize(h->st), "sync");
@@ -1040,6 +1016,7 @@ int cpm_mlp_train(cpm_mlp *h, const float *X, const float *Y, int64_t n_total, c
         if (!rc) rc = grads(h, batch_rows);
         if (rc) return rc;
         ++h->t;
+        h->packed_valid = false;
         const float c1 = 1.0f - powf(beta1, (float)h->t), c2 = 1.0f - powf(beta2, (float)h->t);
         adam_kernel<<<grid1(nP), 256, 0, h->st>>>(nP, h->w, h->wb, h->g, h->m, h->v, lr, beta1, beta2, eps, c1, c2);
         ++h->launches;
@@ -1058,6 +1035,14 @@ int cpm_mlp_forward(cpm_mlp *h, const float *X, int64_t n_rows, float *out)
 {
     if (!h || n_rows < 0 || (n_rows > 0 && (!X || !out))) return CPM_MLP_E_INVALID;
     const int E = h->sh.n_members, no = h->sh.n_out;
+    if (h->packed) {
+        const int64_t most = 1 << 24;  // rows of a launch
+        for (int64_t r0 = 0; r0 < n_rows; r0 += most) {
+            const int64_t rows = n_rows - r0 < most ? n_rows - r0 : most;
+            if (int rc = forward_fused(h, X + r0 * h->sh.n_in, rows, out + r0 * no, n_rows * no)) return rc;
+        }
+        return check_bad(h);
+    }
     for (int64_t r0 = 0; r0 < n_rows; r0 += h->sh.max_rows) {
         const int rows = (int)(n_rows - r0 < h->sh.max_rows ? n_rows - r0 : h->sh.max_rows);
         int rc = gather(h, X, nullptr, nullptr, r0, n_rows, rows);
@@ -1099,11 +1084,17 @@ int cpm_mlp_predict(cpm_mlp *h, const float *X, int64_t n_rows, float *mean_out,
     const int E = h->sh.n_members, no = h->sh.n_out;
     for (int64_t r0 = 0; r0 < n_rows; r0 += h->sh.max_rows) {
         const int rows = (int)(n_rows - r0 < h->sh.max_rows ? n_rows - r0 : h->sh.max_rows);
-        int rc = gather(h, X, nullptr, nullptr, r0, n_rows, rows);
-        if (!rc) rc = forward(h, rows, false);
+        int rc;
+        if (h->packed) {
+            rc = forward_fused(h, X + r0 * h->sh.n_in, rows, h->out, (int64_t)rows * no);
+        } else {
+            rc = gather(h, X, nullptr, nullptr, r0, n_rows, rows);
+            if (!rc) rc = forward(h, rows, false);
+        }
         if (rc) return rc;
-        predict_kernel<<<(rows + 127) / 128, 128, 0, h->st>>>(
-            rows, E, no, h->out, (int64_t)rows * no, h->shift, h->scale, h->logm, h->have_rmse ? h->rmse : nullptr,
+        const int block_rows = no < kPredictThreads ? kPredictThreads / no : 1;
+        predict_kernel<<<(rows + block_rows - 1) / block_rows, kPredictThreads, 0, h->st>>>(
+            rows, block_rows, E, no, h->out, (int64_t)rows * no, h->shift, h->scale, h->logm, h->have_rmse ? h->rmse : nullptr,
             h->factor, mean_out ? mean_out + r0 * no : nullptr, std_out ? std_out + r0 * no : nullptr,
             fallback_out ? fallback_out + r0 : nullptr);
         ++h->launches;
