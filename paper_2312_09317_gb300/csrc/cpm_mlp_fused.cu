@@ -28,9 +28,9 @@
 namespace cpmmlp {
 namespace {
 
-constexpr int kRows = 128, kSlab = 32, kStages = 2, kStageBytes = 16 * 1024;
-constexpr int kEpiWarps = 8, kThreads = (kEpiWarps + 2) * 32;
-constexpr int kCols = 256;  // tensor-memory columns of a CTA
+constexpr int kRows = 128, kSlab = kFusedSlab, kStageBytes = 16 * 1024, kMaxStages = 6;
+// inference: two CTAs per SM, each with a ring of two stages; training: one, since a batch has few tiles
+constexpr int kInferWarps = 8, kInferStages = 2, kTrainWarps = 16, kTrainStages = 6;
 
 struct FusedArgs {
     FusedNet net;
@@ -43,13 +43,15 @@ struct FusedArgs {
     int k0p;              // inputs padded to a multiple of 16
     int64_t member_bytes; // packed weights per member
     int mtiles, items;
+    TrainArgs tr;
 };
 
 struct Barriers {
-    uint64_t wfull[kStages], wempty[kStages];
-    uint64_t hready, dfull;  // a hidden layer: output written (the next input), accumulator complete
+    uint64_t wfull[kMaxStages], wempty[kMaxStages];
+    uint64_t hready, dfull;  // a hidden layer (or its gradient): output written (the next input), accumulator complete
     uint64_t ofull, oread;   // the outputs: accumulator complete, read out
     uint64_t xready;         // the item's inputs written
+    uint64_t pready;         // training: the gradient of the outputs written
     uint64_t drain;
     volatile int abort;      // a wait ran out: every role leaves its loop
 };
@@ -124,12 +126,21 @@ __device__ __forceinline__ void tc_loaded(uint32_t (&v)[N])
                      :
                      : "memory");
 }
+// the data row of a batch's row, -1 (and the flag) where order[] points outside the data
+__device__ __forceinline__ int64_t batch_row(const TrainArgs &t, int64_t r)
+{
+    const int64_t src = t.order ? (int64_t)t.order[t.off + r] : t.off + r;
+    if (src >= 0 && src < t.n_total) return src;
+    *t.bad = 1;
+    return -1;
+}
 // bytes of the packed weights: layer 0, a slab of a hidden layer, the last layer
 __host__ __device__ __forceinline__ int first_bytes(int k0p, int width) { return width * k0p * 2; }
 __host__ __device__ __forceinline__ int slab_bytes(int width) { return width * kSlab * 2; }
 __host__ __device__ __forceinline__ int last_bytes(int width, int n_out) { return n_out * width * 2; }
 
-__global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedArgs p)
+template <int kEpiWarps, int kStages, bool TRAIN>
+__device__ __forceinline__ void fused_body(const FusedArgs &p)
 {
     extern __shared__ __align__(1024) unsigned char fused_smem[];
     __shared__ __align__(8) Barriers bars;
@@ -138,7 +149,8 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
     unsigned char *Ws = fused_smem;                                  // kStages stages
     unsigned char *As = Ws + kStages * kStageBytes;                  // 128 x width
     unsigned char *Xs = As + kRows * width * 2;                      // 128 x k0p
-    float *bias_s = reinterpret_cast<float *>(Xs + kRows * p.k0p * 2);  // two items' biases, layer after layer
+    unsigned char *Ps = Xs + kRows * p.k0p * 2;                      // training: 128 x n_out
+    float *bias_s = reinterpret_cast<float *>(Ps + (TRAIN ? kRows * n_out * 2 : 0));  // two items' biases, layer after layer
     const int n_bias = n_hidden * width + n_out;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
@@ -156,6 +168,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
         bar_init(&bars.ofull, 1);
         bar_init(&bars.oread, kEpiWarps);
         bar_init(&bars.xready, kEpiWarps);
+        bar_init(&bars.pready, kEpiWarps);
         bar_init(&bars.drain, 1);
         bars.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -195,6 +208,13 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
                 for (int k = 0; k < (n_hidden - 1) * slabs && ok; ++k, src += slab_bytes(width))
                     ok = load(src, slab_bytes(width));
                 if (ok) ok = load(src, last_bytes(width, n_out));
+                if (TRAIN && ok) {
+                    const unsigned char *t = p.tr.packed_t + i / p.mtiles * p.tr.member_bytes_t;
+                    ok = load(t, last_bytes(width, n_out));
+                    t += last_bytes(width, n_out);
+                    for (int k = 0; k < (n_hidden - 1) * slabs && ok; ++k, t += slab_bytes(width))
+                        ok = load(t, slab_bytes(width));
+                }
             }
             // (after an abort) the copies in flight land before the CTA's shared memory is given up
             for (uint32_t k = n_slab > kStages ? n_slab - kStages : 0; k < n_slab; ++k)
@@ -212,6 +232,8 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
             const uint64_t dw = tc_desc(smem_u32(Ws), 128u, (uint32_t)(kSlab / 8) * 128u);
             const uint64_t dw_x = tc_desc(smem_u32(Ws), 128u, (uint32_t)(p.k0p / 8) * 128u);
             const uint64_t dw_a = tc_desc(smem_u32(Ws), 128u, (uint32_t)(width / 8) * 128u);
+            const uint64_t dp = tc_desc(smem_u32(Ps), 128u, (uint32_t)(n_out / 8) * 128u);
+            const uint64_t dw_p = tc_desc(smem_u32(Ws), 128u, (uint32_t)(n_out / 8) * 128u);
             const uint32_t idesc = tc_idesc(width), idesc_out = tc_idesc(n_out);
             const auto slab = [&]() { return bar_wait(bars, &bars.wfull[stage], parity); };
             const auto at = [&](uint64_t d) { return d + stage * (kStageBytes / 16); };
@@ -231,27 +253,45 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
                 for (int ks = 0; ks < p.k0p / 16; ++ks) tc_mma(tmem, dx + ks * 16, at(dw_x) + ks * 16, idesc, ks > 0);
                 slab_done();
                 tc_commit(&bars.dfull);
+                // a hidden layer, or a gradient's way through one: K = width, slab by slab
+                const auto hidden = [&]() {
+                    uint64_t d = da;
+                    for (int kc = 0; kc < slabs; ++kc) {
+                        if (kc > 0 && !slab()) return false;
+#pragma unroll
+                        for (int ks = 0; ks < kSlab / 16; ++ks, d += 16)
+                            tc_mma(tmem, d, at(dw) + ks * 16, idesc, kc + ks > 0);
+                        slab_done();
+                    }
+                    tc_commit(&bars.dfull);
+                    return true;
+                };
                 for (int l = 1; l <= n_hidden && ok; ++l, ++n_h) {
                     ok = slab() && bar_wait(bars, &bars.hready, n_h & 1u);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     if (l < n_hidden) {
-                        uint64_t d = da;
-                        for (int kc = 0; kc < slabs; ++kc) {
-                            if (kc > 0) ok = slab();
-                            if (!ok) break;
-#pragma unroll
-                            for (int ks = 0; ks < kSlab / 16; ++ks, d += 16)
-                                tc_mma(tmem, d, at(dw) + ks * 16, idesc, kc + ks > 0);
-                            slab_done();
-                        }
-                        if (ok) tc_commit(&bars.dfull);
+                        ok = hidden();
                     } else {
                         // the outputs: all of K from one stage
                         for (int ks = 0; ks < width / 16; ++ks)
                             tc_mma(tmem, da + ks * 16, at(dw_a) + ks * 16, idesc_out, ks > 0);
                         slab_done();
                         tc_commit(&bars.ofull);
+                    }
+                }
+                if (TRAIN && ok) {
+                    ok = slab() && bar_wait(bars, &bars.pready, (uint32_t)(i - i0) & 1u);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    for (int ks = 0; ks < n_out / 16; ++ks) tc_mma(tmem, dp + ks * 16, at(dw_p) + ks * 16, idesc, ks > 0);
+                    slab_done();
+                    tc_commit(&bars.dfull);
+                    for (int l = n_hidden - 1; l >= 1 && ok; --l, ++n_h) {
+                        ok = slab() && bar_wait(bars, &bars.hready, n_h & 1u);
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        ok = hidden();
                     }
                 }
             }
@@ -264,6 +304,7 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
         __syncwarp();
     } else {
         // ---- epilogue
+        constexpr int kStep = kEpiWarps / 4 * 32;  // columns from one of a warp's blocks to the next
         const int q = warp & 3, part = warp >> 2, r = q * 32 + lane;
         const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
         unsigned char *arow = As + (size_t)(r >> 3) * (width / 8) * 128 + (r & 7) * 16;
@@ -288,12 +329,16 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
             for (int g = threadIdx.x; g < kRows * kc; g += kEpiWarps * 32) {
                 const int rr = g & 7, k8 = (g >> 3) % kc, r8 = (g >> 3) / kc;
                 const int64_t xrow = (int64_t)(i % p.mtiles) * kRows + r8 * 8 + rr;
+                int64_t src = xrow < p.rows ? xrow : -1;
+                if (TRAIN && src >= 0) src = batch_row(p.tr, src);
                 __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = k8 * 8 + j;
-                    h[j] = __float2bfloat16(xrow < p.rows && k < n_in ? p.X[xrow * n_in + k] : 0.0f);
+                    h[j] = __float2bfloat16(src >= 0 && k < n_in ? p.X[src * n_in + k] : 0.0f);
                 }
+                if (TRAIN && e == 0 && xrow < p.rows)
+                    *reinterpret_cast<uint4 *>(p.tr.xb + xrow * p.k0p + k8 * 8) = *reinterpret_cast<const uint4 *>(h);
                 *reinterpret_cast<uint4 *>(Xs + (size_t)g * 16) = *reinterpret_cast<const uint4 *>(h);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -310,8 +355,8 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // sixteen columns at a time, the next ones on their way while these are worked on
                 uint32_t v[2][16];
-                tc_load16(v[0], lanes + (uint32_t)(part * 32));
-                for (int n0 = part * 32; n0 < width; n0 += 64) {
+                if (part * 32 < width) tc_load16(v[0], lanes + (uint32_t)(part * 32));
+                for (int n0 = part * 32; n0 < width; n0 += kStep) {
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         float4 bv[4];
@@ -320,25 +365,46 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
                             bv[j] = reinterpret_cast<const float4 *>(bias + n0 + 16 * half)[j];
                         tc_loaded(v[half]);
                         if (half == 0) tc_load16(v[1], lanes + (uint32_t)(n0 + 16));
-                        else if (n0 + 64 < width) tc_load16(v[0], lanes + (uint32_t)(n0 + 64));
+                        else if (n0 + kStep < width) tc_load16(v[0], lanes + (uint32_t)(n0 + kStep));
                         __align__(16) __nv_bfloat162 h[8];
                         uint64_t z[8];
                         float zmax = 0.0f;
+                        float gp[TRAIN ? 16 : 1];  // GELU', kept for the way back
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             z[j] = add2(pack2(__uint_as_float(v[half][2 * j]), __uint_as_float(v[half][2 * j + 1])),
                                         j % 2 == 0 ? pack2(bv[j / 2].x, bv[j / 2].y) : pack2(bv[j / 2].z, bv[j / 2].w));
                             const float2 zj = unpack2(z[j]);
                             zmax = fmaxf(zmax, fmaxf(fabsf(zj.x), fabsf(zj.y)));
-                            const float2 g = unpack2(gelu2_f(z[j]));
+                            uint64_t grad;
+                            const float2 g = unpack2(gelu2_f<TRAIN>(z[j], grad));
                             h[j] = __floats2bfloat162_rn(g.x, g.y);
+                            if (TRAIN) {
+                                const float2 d = unpack2(grad);
+                                gp[2 * j] = d.x;
+                                gp[2 * j + 1] = d.y;
+                            }
                         }
                         if (!(zmax <= kGelu2Max)) {  // (a NaN is ignored by fmaxf and propagates through either form)
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
                                 const float2 zj = unpack2(z[j]);
                                 h[j] = __floats2bfloat162_rn(gelu_f(zj.x), gelu_f(zj.y));
+                                if (TRAIN) {
+                                    gp[2 * j] = gelu_grad_f(zj.x);
+                                    gp[2 * j + 1] = gelu_grad_f(zj.y);
+                                }
                             }
+                        }
+                        if (TRAIN && row < p.rows) {
+                            const int64_t at = ((int64_t)(e * width + n0 + 16 * half) / 8) * p.rows + row;
+                            uint4 *ho = reinterpret_cast<uint4 *>(p.tr.H[l]) + at;
+                            ho[0] = reinterpret_cast<const uint4 *>(h)[0];
+                            ho[p.rows] = reinterpret_cast<const uint4 *>(h)[1];
+                            float4 *go = reinterpret_cast<float4 *>(p.tr.G[l]) + 2 * at - row;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                go[j * p.rows] = make_float4(gp[4 * j], gp[4 * j + 1], gp[4 * j + 2], gp[4 * j + 3]);
                         }
                         unsigned char *o = arow + (n0 / 8 + 2 * half) * 128;
                         *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(h)[0];
@@ -361,11 +427,84 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
                 uint32_t v[16];
                 tc_load16(v, lanes + (uint32_t)n0);
                 tc_loaded(v);
-                if (row < p.rows) {
-                    float *o = p.out + e * p.s_member + row * n_out + n0;
+                if (!TRAIN) {
+                    if (row < p.rows) {
+                        float *o = p.out + e * p.s_member + row * n_out + n0;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) o[j] = __uint_as_float(v[j]) + bias[n0 + j];
+                        for (int j = 0; j < 16; ++j) o[j] = __uint_as_float(v[j]) + bias[n0 + j];
+                    }
+                } else {
+                    // loss, and the gradient of the outputs: the first input of the way back
+                    const int64_t src = row < p.rows ? batch_row(p.tr, row) : -1;
+                    float sq = 0.0f;
+                    __align__(16) __nv_bfloat16 g[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const float d = src >= 0 ? __uint_as_float(v[j]) + bias[n0 + j] - p.tr.Y[src * n_out + n0 + j] : 0.0f;
+                        g[j] = __float2bfloat16(2.0f * d * p.tr.inv);
+                        sq += d * d;
+                    }
+                    unsigned char *o = Ps + (size_t)((r >> 3) * (n_out / 8) + n0 / 8) * 128 + (r & 7) * 16;
+                    *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(g)[0];
+                    *reinterpret_cast<uint4 *>(o + 128) = reinterpret_cast<const uint4 *>(g)[1];
+                    if (row < p.rows) {
+                        uint4 *d = reinterpret_cast<uint4 *>(p.tr.dP + (e * p.rows + row) * n_out + n0);
+                        d[0] = reinterpret_cast<const uint4 *>(g)[0];
+                        d[1] = reinterpret_cast<const uint4 *>(g)[1];
+                    }
+#pragma unroll
+                    for (int d = 16; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
+                    if (lane == 0) atomicAdd(p.tr.loss + e, sq * p.tr.inv);
                 }
+            }
+            if (TRAIN) {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) bar_arrive(&bars.pready);
+                // the way back: dZ_l = (dZ_{l+1} W_{l+1}) GELU'(Z_l), over the activations of its last input
+                for (int l = n_hidden - 1; l >= 0; --l, ++n_d) {
+                    ok = warp_wait(bars, &bars.dfull, n_d & 1u);
+                    if (!ok) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    for (int n0 = part * 32; n0 < width; n0 += kStep) {
+#pragma unroll
+                        for (int half = 0; half < 2; ++half) {
+                            uint32_t v[16];
+                            tc_load16(v, lanes + (uint32_t)(n0 + 16 * half));
+                            float4 *go = reinterpret_cast<float4 *>(p.tr.G[l]) +
+                                         ((int64_t)(e * width + n0 + 16 * half) / 4) * p.rows + row;
+                            float4 gp[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                gp[j] = row < p.rows ? go[j * p.rows] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                            tc_loaded(v);
+                            __align__(16) __nv_bfloat162 h[8];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                h[2 * j] = __floats2bfloat162_rn(__uint_as_float(v[4 * j]) * gp[j].x,
+                                                                 __uint_as_float(v[4 * j + 1]) * gp[j].y);
+                                h[2 * j + 1] = __floats2bfloat162_rn(__uint_as_float(v[4 * j + 2]) * gp[j].z,
+                                                                     __uint_as_float(v[4 * j + 3]) * gp[j].w);
+                            }
+                            unsigned char *o = arow + (n0 / 8 + 2 * half) * 128;
+                            *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(h)[0];
+                            *reinterpret_cast<uint4 *>(o + 128) = reinterpret_cast<const uint4 *>(h)[1];
+                            if (row < p.rows) {
+                                uint4 *d = reinterpret_cast<uint4 *>(go);  // over the GELU' just read
+                                d[0] = reinterpret_cast<const uint4 *>(h)[0];
+                                d[2 * p.rows] = reinterpret_cast<const uint4 *>(h)[1];
+                            }
+                        }
+                    }
+                    if (l > 0) {
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                        __syncwarp();
+                        if (lane == 0) bar_arrive(&bars.hready);
+                    }
+                }
+                if (!ok) break;
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -376,6 +515,50 @@ __global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedA
     __syncthreads();
     if (threadIdx.x == 0 && bars.abort && p.err) atomicExch(p.err, 1);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+}
+
+__global__ void __launch_bounds__((kInferWarps + 2) * 32, 2) fused_forward_kernel(const FusedArgs p)
+{
+    fused_body<kInferWarps, kInferStages, false>(p);
+}
+
+// One training batch, forward and back: writes the bf16 inputs and activations of every layer and the bf16
+// gradients of every pre-activation, from which fused_update forms the weights' gradients.  A batch of
+// 1,024 rows is 40 tiles for five members, so a CTA has an SM to itself: 16 epilogue warps, a ring of six
+// stages.  GELU' is kept in FP32 from the way forward, where its exponential is at hand.
+__global__ void __launch_bounds__((kTrainWarps + 2) * 32, 1) fused_train_kernel(const FusedArgs p)
+{
+    fused_body<kTrainWarps, kTrainStages, true>(p);
+}
+
+// The transposed weights as the way back reads them: B[n][k] = W[k][n], the last layer first.
+__global__ void fused_pack_t_kernel(const FusedNet n, const __nv_bfloat16 *wb, unsigned char *packed, int64_t member_bytes)
+{
+    const int slabs = n.width / kSlab;
+    const int64_t pieces = member_bytes / 16;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < pieces * n.n_members;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int e = (int)(t / pieces);
+        int64_t at = (t % pieces) * 16;
+        const int64_t hidden = (int64_t)n.width * n.width + n.width, layer = (int64_t)slabs * slab_bytes(n.width);
+        const __nv_bfloat16 *W = wb + e * n.P + (int64_t)n.n_in * n.width + n.width;  // layer 1
+        int kc = n.n_out / 8, k_first = 0;
+        if (at < last_bytes(n.width, n.n_out)) {
+            W += (n.n_hidden - 1) * hidden;
+        } else {
+            at -= last_bytes(n.width, n.n_out);
+            W += (n.n_hidden - 2 - at / layer) * hidden;
+            at %= layer;
+            k_first = (int)(at / slab_bytes(n.width)) * kSlab;
+            at %= slab_bytes(n.width);
+            kc = kSlab / 8;
+        }
+        const int q = (int)(at / 16), rr = q & 7, k8 = (q >> 3) % kc, r8 = (q >> 3) / kc;
+        __align__(16) __nv_bfloat16 h[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) h[j] = W[(int64_t)(k_first + k8 * 8 + j) * n.width + r8 * 8 + rr];
+        *reinterpret_cast<uint4 *>(packed + t * 16) = *reinterpret_cast<const uint4 *>(h);
+    }
 }
 
 // One 16-byte piece of a packed layer per thread: 8 consecutive inputs of one output, in the canonical
@@ -441,32 +624,71 @@ cudaError_t fused_pack(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char
     return cudaPeekAtLastError();
 }
 
-cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float *out, int64_t s_member, int *err,
-                          int report_timeout, cudaStream_t st)
+int64_t fused_packed_t_bytes(int width, int n_hidden, int n_out)
 {
-    if (rows <= 0) return cudaSuccess;
+    return last_bytes(width, n_out) + (int64_t)(n_hidden - 1) * (width / kSlab) * slab_bytes(width);
+}
+
+cudaError_t fused_pack_t(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed_t, cudaStream_t st)
+{
+    const int64_t bytes = fused_packed_t_bytes(n.width, n.n_hidden, n.n_out);
+    const int64_t blocks = (bytes / 16 * n.n_members + 255) / 256;
+    fused_pack_t_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(n, wb, packed_t, bytes);
+    return cudaPeekAtLastError();
+}
+
+namespace {
+
+FusedArgs fused_args(const FusedNet &n, const float *X, int64_t rows, int *err, int report_timeout)
+{
     FusedArgs p{};
     p.net = n;
     p.X = X;
     p.rows = rows;
-    p.out = out;
-    p.s_member = s_member;
     p.err = err;
     p.report_timeout = report_timeout;
     p.k0p = padded_inputs(n.n_in);
     p.member_bytes = fused_packed_bytes(n.n_in, n.width, n.n_hidden, n.n_out);
     p.mtiles = (int)((rows + kRows - 1) / kRows);
     p.items = p.mtiles * n.n_members;
-    const int smem = kStages * kStageBytes + kRows * n.width * 2 + kRows * p.k0p * 2 +
+    return p;
+}
+
+template <typename K>
+cudaError_t fused_launch(K kernel, const FusedArgs &p, int warps, int stages, int per_sm, int extra, cudaStream_t st)
+{
+    const FusedNet &n = p.net;
+    const int smem = stages * kStageBytes + kRows * n.width * 2 + kRows * p.k0p * 2 + extra +
                      2 * 4 * (n.n_hidden * n.width + n.n_out);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      200 * 1024);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    fused_forward_kernel<<<p.items < 2 * sms ? p.items : 2 * sms, kThreads, smem, st>>>(p);
+    kernel<<<p.items < per_sm * sms ? p.items : per_sm * sms, (warps + 2) * 32, smem, st>>>(p);
     return cudaPeekAtLastError();
+}
+
+}  // namespace
+
+cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float *out, int64_t s_member, int *err,
+                          int report_timeout, cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    FusedArgs p = fused_args(n, X, rows, err, report_timeout);
+    p.out = out;
+    p.s_member = s_member;
+    return fused_launch(fused_forward_kernel, p, kInferWarps, kInferStages, 2, 0, st);
+}
+
+cudaError_t fused_train(const FusedNet &n, const TrainArgs &tr, const float *X, int64_t rows, int *err,
+                        int report_timeout, cudaStream_t st)
+{
+    if (rows <= 0) return cudaSuccess;
+    FusedArgs p = fused_args(n, X, rows, err, report_timeout);
+    p.tr = tr;
+    p.tr.member_bytes_t = fused_packed_t_bytes(n.width, n.n_hidden, n.n_out);
+    return fused_launch(fused_train_kernel, p, kTrainWarps, kTrainStages, 1, kRows * n.n_out * 2, st);
 }
 
 }  // namespace cpmmlp

@@ -16,12 +16,48 @@ struct FusedNet {
     int64_t P;                   // per member
     const unsigned char *packed; // weights as fused_pack lays them out
 };
+constexpr int kFusedSlab = 32;       // K of a packed slab of a hidden layer
+constexpr int kFusedMaxHidden = 16;
 bool fused_fits(int n_in, int width, int n_out);
 int64_t fused_packed_bytes(int n_in, int width, int n_hidden, int n_out);  // per member
 cudaError_t fused_pack(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed, cudaStream_t st);
 // out[e s_member + row n_out + k] of rows [0, rows) of X; err: set where a wait ran out; report_timeout: test hook
 cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float *out, int64_t s_member, int *err,
                           int report_timeout, cudaStream_t st);
+
+// A training batch: rows order[off ..] (or off ..) of X and Y, its activations and gradients.
+struct TrainArgs {
+    const float *Y;
+    const int32_t *order;
+    int64_t off, n_total;
+    __nv_bfloat16 *xb;                  // [rows][inputs padded to 16]
+    // Per hidden layer, 16-byte pieces of a row, neighbouring rows next to each other (a warp's lanes are rows):
+    __nv_bfloat16 *H[kFusedMaxHidden];  // [member][width / 8][row][8]: outputs
+    float *G[kFusedMaxHidden];          // [member][width / 4][row][4]: GELU'; the way back puts the bf16 gradients of
+                                        // the pre-activations over it, 8 in the first of each two pieces
+    __nv_bfloat16 *dP;                  // [member][row][n_out]: gradient of the outputs
+    float *loss;                        // per member, added to
+    float inv;                          // 1 / (rows n_out)
+    int *bad;                           // set where order[] points outside the data
+    const unsigned char *packed_t;      // transposed weights (fused_pack_t)
+    int64_t member_bytes_t;
+};
+int64_t fused_packed_t_bytes(int width, int n_hidden, int n_out);  // per member
+cudaError_t fused_pack_t(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed_t, cudaStream_t st);
+// forward and backward over a batch: xb, H, the gradients in G, dP and the losses
+cudaError_t fused_train(const FusedNet &n, const TrainArgs &tr, const float *X, int64_t rows, int *err,
+                        int report_timeout, cudaStream_t st);
+
+// Where the gradients of a batch go: to g as they are, or (update) through an Adam step into the weights and
+// both of their packed forms.
+struct UpdateArgs {
+    int update;
+    float *g;
+    float *w, *m, *v;
+    unsigned char *packed, *packed_t;
+    float lr, b1, b2, eps, c1, c2;
+};
+cudaError_t fused_update(const FusedNet &n, const TrainArgs &tr, const UpdateArgs &u, int64_t rows, cudaStream_t st);
 
 #ifdef __CUDACC__
 
@@ -106,7 +142,16 @@ __device__ __forceinline__ float rcp_approx(float a)
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
 }
-__device__ __forceinline__ uint64_t gelu2_f(uint64_t z)
+__device__ __forceinline__ float gelu_grad_f(float z)
+{
+    float dens;
+    const float cdf = phi_f(z, dens);
+    return cdf + z * 0.39894228040143268f * dens;
+}
+
+// with GRAD also the derivative, as gelu_grad_f
+template <bool GRAD>
+__device__ __forceinline__ uint64_t gelu2_f(uint64_t z, uint64_t &grad)
 {
     constexpr uint64_t kAbs = 0x7fffffff7fffffffull, kSign = ~kAbs;
     const uint64_t xs = mul2(z, both(0.70710678118654752f));
@@ -119,15 +164,11 @@ __device__ __forceinline__ uint64_t gelu2_f(uint64_t z)
     poly = fma2(poly, t, both(0.254829592f));
     const uint64_t minus_h = mul2(mul2(mul2(both(-0.5f), poly), t), dens);
     const uint64_t one = (z & kSign) | 0x3f8000003f800000ull;  // +-1, the sign of z
-    return mul2(z, fma2(one, minus_h, fma2(one, both(0.5f), both(0.5f))));
+    const uint64_t cdf = fma2(one, minus_h, fma2(one, both(0.5f), both(0.5f)));
+    if (GRAD) grad = fma2(mul2(z, both(0.39894228040143268f)), dens, cdf);
+    return mul2(z, cdf);
 }
 
-__device__ __forceinline__ float gelu_grad_f(float z)
-{
-    float dens;
-    const float cdf = phi_f(z, dens);
-    return cdf + z * 0.39894228040143268f * dens;
-}
 
 constexpr uint32_t kTcSpinLimit = 1u << 22;
 
