@@ -814,9 +814,9 @@ int forward_fused(cpm_mlp *h, const float *X, int64_t rows, float *out, int64_t 
 }
 
 // One batch by the fused kernels: its loss added to loss[0 .. E), its gradients to h->g or (u.update) into the
-// weights.  1,024 rows of 5 members of 7-256x4-16: 93 us; a kernel per layer and product, 23 launches: 455 us.
+// weights.  1,024 rows of 5 members of 7-256x4-16: 59 us; a kernel per layer and product, 23 launches: 455 us.
 int batch_fused(cpm_mlp *h, const float *X, const float *Y, const int32_t *order, int64_t off, int64_t n_total, int rows,
-                float *loss, UpdateArgs u)
+                float *loss, UpdateArgs u, bool chained)
 {
     if (int rc = pack(h)) return rc;
     const FusedNet n = fused_net(h);
@@ -835,6 +835,7 @@ int batch_fused(cpm_mlp *h, const float *X, const float *Y, const int32_t *order
     t.inv = 1.0f / (float)((int64_t)rows * n.n_out);
     t.bad = h->bad;
     t.packed_t = h->packed_t;
+    t.chained = chained;
     int rc = cuda_check(h, fused_train(n, t, X, rows, h->bad + 1, h->report_tc_timeout, h->st), "training batch");
     h->report_tc_timeout = 0;
     u.g = h->g;
@@ -980,10 +981,11 @@ int cpm_mlp_create(const cpm_mlp_shape *shape, const float *init_params, void *c
     int rc = 0;
     rc |= dalloc(h, &h->w, nP) | dalloc(h, &h->g, nP) | dalloc(h, &h->m, nP) | dalloc(h, &h->v, nP);
     const bool fused = fused_fits(shape->n_in, W, shape->n_out);
-    rc |= dalloc(h, &h->wb, nP) | dalloc(h, &h->xb, (int64_t)R * (fused ? (shape->n_in + 15) / 16 * 16 : shape->n_in));
+    const int64_t Rb = fused ? ((int64_t)R + 7) / 8 * 8 : R;  // the fused kernels keep rows in eights
+    rc |= dalloc(h, &h->wb, nP) | dalloc(h, &h->xb, Rb * (fused ? padded_inputs(shape->n_in) : shape->n_in));
     for (int l = 0; l < shape->n_hidden; ++l)
-        rc |= dalloc(h, &h->H[l], (int64_t)E * R * W) | dalloc(h, &h->Z[l], (int64_t)E * R * W);
-    rc |= dalloc(h, &h->out, (int64_t)E * R * shape->n_out) | dalloc(h, &h->dP, (int64_t)E * R * shape->n_out);
+        rc |= dalloc(h, &h->H[l], E * Rb * W) | dalloc(h, &h->Z[l], E * Rb * W);
+    rc |= dalloc(h, &h->out, (int64_t)E * R * shape->n_out) | dalloc(h, &h->dP, E * Rb * shape->n_out);
     if (!fused)
         rc |= dalloc(h, &h->yb, (int64_t)R * shape->n_out) | dalloc(h, &h->dZ[0], (int64_t)E * R * W) |
               dalloc(h, &h->dZ[1], (int64_t)E * R * W);
@@ -1043,7 +1045,7 @@ int cpm_mlp_grads(cpm_mlp *h, const float *X, const float *Y, int64_t n_total, c
     int rc;
     if (h->packed) {
         rc = cuda_check(h, cudaMemsetAsync(h->loss, 0, sizeof(float) * h->sh.n_members, h->st), "memset loss");
-        if (!rc) rc = batch_fused(h, X, Y, order, offset, n_total, rows, h->loss, UpdateArgs{});
+        if (!rc) rc = batch_fused(h, X, Y, order, offset, n_total, rows, h->loss, UpdateArgs{}, false);
     } else {
         rc = gather(h, X, Y, order, offset, n_total, rows);
         if (!rc) rc = grads(h, rows);
@@ -1085,7 +1087,7 @@ int cpm_mlp_train(cpm_mlp *h, const float *X, const float *Y, int64_t n_total, c
             u.c1 = 1.0f - powf(beta1, (float)(h->t + 1));
             u.c2 = 1.0f - powf(beta2, (float)(h->t + 1));
             if (int rc = batch_fused(h, X, Y, order, s * batch_rows, n_total, batch_rows,
-                                     loss_trace ? loss_trace + s * h->sh.n_members : loss, u))
+                                     loss_trace ? loss_trace + s * h->sh.n_members : loss, u, s > 0))
                 return rc;
             ++h->t;
         }

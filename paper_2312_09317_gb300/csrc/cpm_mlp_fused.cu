@@ -6,7 +6,7 @@
 // bf16, over the layer's input in shared memory, and the next layer reads it there.  Three roles:
 //   loader (one thread)  the weights, packed as the MMAs read them, by bulk copies into a ring of
 //                        two stages, a 32-deep K slab of a layer each;
-//   issuer (one thread)  a layer's MMAs, slab by slab, once its input is written;
+//   issuer (one warp)    a layer's MMAs, slab by slab, once its input is written;
 //   epilogue (8 warps)   warp w reads tensor-memory lanes 32 (w % 4) .. and every other 32 columns; it also
 //                        converts an item's inputs to bf16.
 // Two CTAs share an SM (100 KB of shared memory, half the tensor memory each), so that one's MMAs, copies
@@ -15,7 +15,7 @@
 //
 // What bounds it: the instructions of the epilogue (about 18 issue slots per 32 outputs, 55% of all slots
 // used) and, beside them, the ring: a hidden layer's MMAs take 5,300 cycles, of which 2,200 are the MMAs.
-// 65,536 rows of 5 members of 7-256x4-16: 318 us; with a launch per layer, whose activations go through HBM,
+// 65,536 rows of 5 members of 7-256x4-16: 312 us; with a launch per layer, whose activations go through HBM,
 // 700 us.  One CTA per SM with 16 epilogue warps that the next layer's MMAs follow in chunks of 64 or 128
 // columns: 338 and 326 us.
 #include <cuda_bf16.h>
@@ -24,13 +24,13 @@
 #include <cstdint>
 
 #include "cpm_mlp_internal.h"
+#include "cpm_mlp_tc.cuh"
 
 namespace cpmmlp {
 namespace {
 
-constexpr int kRows = 128, kSlab = kFusedSlab, kStageBytes = 16 * 1024, kMaxStages = 6;
-// inference: two CTAs per SM, each with a ring of two stages; training: one, since a batch has few tiles
-constexpr int kInferWarps = 8, kInferStages = 2, kTrainWarps = 16, kTrainStages = 6;
+constexpr int kStages = 2;
+constexpr int kEpiWarps = 8, kThreads = (kEpiWarps + 2) * 32;
 
 struct FusedArgs {
     FusedNet net;
@@ -43,104 +43,18 @@ struct FusedArgs {
     int k0p;              // inputs padded to a multiple of 16
     int64_t member_bytes; // packed weights per member
     int mtiles, items;
-    TrainArgs tr;
 };
 
 struct Barriers {
-    uint64_t wfull[kMaxStages], wempty[kMaxStages];
-    uint64_t hready, dfull;  // a hidden layer (or its gradient): output written (the next input), accumulator complete
+    uint64_t wfull[kStages], wempty[kStages];
+    uint64_t hready, dfull;  // a hidden layer: output written (the next input), accumulator complete
     uint64_t ofull, oread;   // the outputs: accumulator complete, read out
     uint64_t xready;         // the item's inputs written
-    uint64_t pready;         // training: the gradient of the outputs written
     uint64_t drain;
     volatile int abort;      // a wait ran out: every role leaves its loop
 };
 
-__device__ __forceinline__ void bar_init(uint64_t *b, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void bar_arrive(uint64_t *b)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-// bounded wait for the phase `parity` of b; false once a wait of the CTA ran out (this one or another)
-__device__ __forceinline__ bool bar_wait(Barriers &s, uint64_t *b, uint32_t parity)
-{
-    const uint32_t addr = smem_u32(b);
-    for (uint32_t it = 0; it < kTcSpinLimit; ++it) {
-        uint32_t done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done)
-                     : "r"(addr), "r"(parity)
-                     : "memory");
-        if (done) return true;
-        if (s.abort) return false;
-    }
-    s.abort = 1;
-    return false;
-}
-__device__ __forceinline__ void tc_commit(uint64_t *b)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b))
-                 : "memory");
-}
-__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, bool accumulate)
-{
-    asm volatile("{\n .reg .pred acc;\n setp.ne.b32 acc, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, acc;\n}" ::"r"(d),
-                 "l"(ad), "l"(bd), "r"(idesc), "r"(accumulate ? 1 : 0)
-                 : "memory");
-}
-__device__ __forceinline__ uint32_t tc_idesc(int n)
-{
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kRows >> 4) << 24);
-}
-
-// the same for a whole warp, which stays together whichever way it goes
-__device__ __forceinline__ bool warp_wait(Barriers &s, uint64_t *b, uint32_t parity)
-{
-    return __all_sync(0xffffffffu, bar_wait(s, b, parity));
-}
-// the accumulator's 16 columns from `addr` of this warp's 32 lanes; complete after tcgen05.wait::ld
-__device__ __forceinline__ void tc_load16(uint32_t (&v)[16], uint32_t addr)
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
-                 "%14, %15}, [%16];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                 : "r"(addr)
-                 : "memory");
-}
-// the loads of v have landed (v is an operand, so that no use of it moves before the wait)
-template <int N>
-__device__ __forceinline__ void tc_loaded(uint32_t (&v)[N])
-{
-#pragma unroll
-    for (int j = 0; j < N; j += 16)
-        asm volatile("tcgen05.wait::ld.sync.aligned;"
-                     : "+r"(v[j]), "+r"(v[j + 1]), "+r"(v[j + 2]), "+r"(v[j + 3]), "+r"(v[j + 4]), "+r"(v[j + 5]),
-                       "+r"(v[j + 6]), "+r"(v[j + 7]), "+r"(v[j + 8]), "+r"(v[j + 9]), "+r"(v[j + 10]), "+r"(v[j + 11]),
-                       "+r"(v[j + 12]), "+r"(v[j + 13]), "+r"(v[j + 14]), "+r"(v[j + 15])
-                     :
-                     : "memory");
-}
-// the data row of a batch's row, -1 (and the flag) where order[] points outside the data
-__device__ __forceinline__ int64_t batch_row(const TrainArgs &t, int64_t r)
-{
-    const int64_t src = t.order ? (int64_t)t.order[t.off + r] : t.off + r;
-    if (src >= 0 && src < t.n_total) return src;
-    *t.bad = 1;
-    return -1;
-}
-// bytes of the packed weights: layer 0, a slab of a hidden layer, the last layer
-__host__ __device__ __forceinline__ int first_bytes(int k0p, int width) { return width * k0p * 2; }
-__host__ __device__ __forceinline__ int slab_bytes(int width) { return width * kSlab * 2; }
-__host__ __device__ __forceinline__ int last_bytes(int width, int n_out) { return n_out * width * 2; }
-
-template <int kEpiWarps, int kStages, bool TRAIN>
-__device__ __forceinline__ void fused_body(const FusedArgs &p)
+__global__ void __launch_bounds__(kThreads, 2) fused_forward_kernel(const FusedArgs p)
 {
     extern __shared__ __align__(1024) unsigned char fused_smem[];
     __shared__ __align__(8) Barriers bars;
@@ -149,8 +63,7 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
     unsigned char *Ws = fused_smem;                                  // kStages stages
     unsigned char *As = Ws + kStages * kStageBytes;                  // 128 x width
     unsigned char *Xs = As + kRows * width * 2;                      // 128 x k0p
-    unsigned char *Ps = Xs + kRows * p.k0p * 2;                      // training: 128 x n_out
-    float *bias_s = reinterpret_cast<float *>(Ps + (TRAIN ? kRows * n_out * 2 : 0));  // two items' biases, layer after layer
+    float *bias_s = reinterpret_cast<float *>(Xs + kRows * p.k0p * 2);  // two items' biases, layer after layer
     const int n_bias = n_hidden * width + n_out;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {
@@ -168,7 +81,6 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
         bar_init(&bars.ofull, 1);
         bar_init(&bars.oread, kEpiWarps);
         bar_init(&bars.xready, kEpiWarps);
-        bar_init(&bars.pready, kEpiWarps);
         bar_init(&bars.drain, 1);
         bars.abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -176,11 +88,11 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     const int i0 = (int)((int64_t)p.items * blockIdx.x / gridDim.x);
     const int i1 = (int)((int64_t)p.items * (blockIdx.x + 1) / gridDim.x);
 
-    if (warp == kEpiWarps + 1) {
+    if (warp == 1) {
         // ---- loader
         if (lane == 0) {
             uint32_t stage = 0, parity = 1;  // of the stage's last use; 1: none yet
@@ -208,104 +120,74 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
                 for (int k = 0; k < (n_hidden - 1) * slabs && ok; ++k, src += slab_bytes(width))
                     ok = load(src, slab_bytes(width));
                 if (ok) ok = load(src, last_bytes(width, n_out));
-                if (TRAIN && ok) {
-                    const unsigned char *t = p.tr.packed_t + i / p.mtiles * p.tr.member_bytes_t;
-                    ok = load(t, last_bytes(width, n_out));
-                    t += last_bytes(width, n_out);
-                    for (int k = 0; k < (n_hidden - 1) * slabs && ok; ++k, t += slab_bytes(width))
-                        ok = load(t, slab_bytes(width));
-                }
             }
             // (after an abort) the copies in flight land before the CTA's shared memory is given up
             for (uint32_t k = n_slab > kStages ? n_slab - kStages : 0; k < n_slab; ++k)
                 tc_wait(&bars.wfull[k % kStages], (k / kStages) & 1u);
         }
         __syncwarp();
-    } else if (warp == kEpiWarps) {
+    } else if (warp == 0) {
         // ---- issuer
-        if (lane == 0) {
-            uint32_t n_h = 0;                // hidden epilogues waited for
-            uint32_t stage = 0, parity = 0;  // of the next slab
-            // matrix descriptors: the address, in 16-byte units, is their low field
-            const uint64_t da = tc_desc(smem_u32(As), 128u, (uint32_t)(width / 8) * 128u);
-            const uint64_t dx = tc_desc(smem_u32(Xs), 128u, (uint32_t)(p.k0p / 8) * 128u);
-            const uint64_t dw = tc_desc(smem_u32(Ws), 128u, (uint32_t)(kSlab / 8) * 128u);
-            const uint64_t dw_x = tc_desc(smem_u32(Ws), 128u, (uint32_t)(p.k0p / 8) * 128u);
-            const uint64_t dw_a = tc_desc(smem_u32(Ws), 128u, (uint32_t)(width / 8) * 128u);
-            const uint64_t dp = tc_desc(smem_u32(Ps), 128u, (uint32_t)(n_out / 8) * 128u);
-            const uint64_t dw_p = tc_desc(smem_u32(Ws), 128u, (uint32_t)(n_out / 8) * 128u);
-            const uint32_t idesc = tc_idesc(width), idesc_out = tc_idesc(n_out);
-            const auto slab = [&]() { return bar_wait(bars, &bars.wfull[stage], parity); };
-            const auto at = [&](uint64_t d) { return d + stage * (kStageBytes / 16); };
-            const auto slab_done = [&]() {
-                tc_commit(&bars.wempty[stage]);
-                if (++stage == kStages) {
-                    stage = 0;
-                    parity ^= 1u;
-                }
-            };
-            bool ok = true;
-            for (int i = i0; i < i1 && ok; ++i) {
-                ok = slab() && bar_wait(bars, &bars.xready, (uint32_t)(i - i0) & 1u);
-                if (ok && i > i0) ok = bar_wait(bars, &bars.oread, (uint32_t)(i - i0 - 1) & 1u);
+        uint32_t n_h = 0;                // hidden epilogues waited for
+        uint32_t stage = 0, parity = 0;  // of the next slab
+        // matrix descriptors: the address, in 16-byte units, is their low field
+        const uint64_t da = tc_desc(smem_u32(As), 128u, (uint32_t)(width / 8) * 128u);
+        const uint64_t dx = tc_desc(smem_u32(Xs), 128u, (uint32_t)(p.k0p / 8) * 128u);
+        const uint64_t dw = tc_desc(smem_u32(Ws), 128u, (uint32_t)(kSlab / 8) * 128u);
+        const uint64_t dw_x = tc_desc(smem_u32(Ws), 128u, (uint32_t)(p.k0p / 8) * 128u);
+        const uint32_t idesc = tc_idesc(width), idesc_out = tc_idesc(n_out);
+        const auto slab = [&]() { return warp_wait(bars, &bars.wfull[stage], parity); };
+        const auto at = [&](uint64_t d) { return d + stage * (kStageBytes / 16); };
+        const auto slab_done = [&]() {
+            tc_commit(&bars.wempty[stage]);
+            if (++stage == kStages) {
+                stage = 0;
+                parity ^= 1u;
+            }
+        };
+        bool ok = true;
+        for (int i = i0; i < i1 && ok; ++i) {
+            ok = slab() && warp_wait(bars, &bars.xready, (uint32_t)(i - i0) & 1u);
+            if (ok && i > i0) ok = warp_wait(bars, &bars.oread, (uint32_t)(i - i0 - 1) & 1u);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            for (int ks = 0; ks < p.k0p / 16; ++ks) tc_mma(tmem, dx + ks * 16, at(dw_x) + ks * 16, idesc, ks > 0);
+            slab_done();
+            tc_commit(&bars.dfull);
+            for (int l = 1; l <= n_hidden && ok; ++l, ++n_h) {
+                ok = slab() && warp_wait(bars, &bars.hready, n_h & 1u);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                for (int ks = 0; ks < p.k0p / 16; ++ks) tc_mma(tmem, dx + ks * 16, at(dw_x) + ks * 16, idesc, ks > 0);
-                slab_done();
-                tc_commit(&bars.dfull);
-                // a hidden layer, or a gradient's way through one: K = width, slab by slab
-                const auto hidden = [&]() {
+                if (l < n_hidden) {
                     uint64_t d = da;
                     for (int kc = 0; kc < slabs; ++kc) {
-                        if (kc > 0 && !slab()) return false;
+                        if (kc > 0) ok = slab();
+                        if (!ok) break;
 #pragma unroll
                         for (int ks = 0; ks < kSlab / 16; ++ks, d += 16)
                             tc_mma(tmem, d, at(dw) + ks * 16, idesc, kc + ks > 0);
                         slab_done();
                     }
-                    tc_commit(&bars.dfull);
-                    return true;
-                };
-                for (int l = 1; l <= n_hidden && ok; ++l, ++n_h) {
-                    ok = slab() && bar_wait(bars, &bars.hready, n_h & 1u);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    if (l < n_hidden) {
-                        ok = hidden();
-                    } else {
-                        // the outputs: all of K from one stage
-                        for (int ks = 0; ks < width / 16; ++ks)
-                            tc_mma(tmem, da + ks * 16, at(dw_a) + ks * 16, idesc_out, ks > 0);
-                        slab_done();
-                        tc_commit(&bars.ofull);
-                    }
-                }
-                if (TRAIN && ok) {
-                    ok = slab() && bar_wait(bars, &bars.pready, (uint32_t)(i - i0) & 1u);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    for (int ks = 0; ks < n_out / 16; ++ks) tc_mma(tmem, dp + ks * 16, at(dw_p) + ks * 16, idesc, ks > 0);
+                    if (ok) tc_commit(&bars.dfull);
+                } else {
+                    // the outputs: every slab of K from one stage
+                    for (int kc = 0; kc < slabs; ++kc)
+#pragma unroll
+                        for (int ks = 0; ks < kSlab / 16; ++ks)
+                            tc_mma(tmem, da + kc * 32 + ks * 16, at(dw) + kc * (n_out * 4) + ks * 16, idesc_out, kc + ks > 0);
                     slab_done();
-                    tc_commit(&bars.dfull);
-                    for (int l = n_hidden - 1; l >= 1 && ok; --l, ++n_h) {
-                        ok = slab() && bar_wait(bars, &bars.hready, n_h & 1u);
-                        if (!ok) break;
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        ok = hidden();
-                    }
+                    tc_commit(&bars.ofull);
                 }
-            }
-            if (!ok) {
-                // the MMAs issued so far end before tensor memory is given up
-                tc_commit(&bars.drain);
-                tc_wait(&bars.drain, 0);
             }
         }
-        __syncwarp();
+        if (!ok) {
+            // the MMAs issued so far end before tensor memory is given up
+            tc_commit(&bars.drain);
+            tc_wait(&bars.drain, 0);
+        }
     } else {
         // ---- epilogue
-        constexpr int kStep = kEpiWarps / 4 * 32;  // columns from one of a warp's blocks to the next
-        const int q = warp & 3, part = warp >> 2, r = q * 32 + lane;
+        const int q = warp & 3, part = (warp - 2) >> 2, tid = threadIdx.x - 64, r = q * 32 + lane;
         const uint32_t lanes = tmem + ((uint32_t)(q * 32) << 16);
         unsigned char *arow = As + (size_t)(r >> 3) * (width / 8) * 128 + (r & 7) * 16;
         uint32_t n_d = 0;  // hidden layers done
@@ -318,7 +200,7 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
             // its first hidden layer came through
             float *bias = bias_s + ((i - i0) & 1) * n_bias;
             const float *w = p.net.w + e * p.net.P;
-            for (int g = threadIdx.x; g < n_bias; g += kEpiWarps * 32) {
+            for (int g = tid; g < n_bias; g += kEpiWarps * 32) {
                 const int l = g / width, k = g - l * width;  // b_l follows W_l
                 bias[g] = __ldg(w + (int64_t)p.net.n_in * width + (l > 0 ? width : 0) +
                                 (l > 1 ? (int64_t)(l - 1) * width : 0) +
@@ -326,19 +208,15 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
                                               : (int64_t)(n_hidden - 1) * width * width + (int64_t)n_out * width) + k);
             }
             const int kc = p.k0p / 8, n_in = p.net.n_in;
-            for (int g = threadIdx.x; g < kRows * kc; g += kEpiWarps * 32) {
+            for (int g = tid; g < kRows * kc; g += kEpiWarps * 32) {
                 const int rr = g & 7, k8 = (g >> 3) % kc, r8 = (g >> 3) / kc;
                 const int64_t xrow = (int64_t)(i % p.mtiles) * kRows + r8 * 8 + rr;
-                int64_t src = xrow < p.rows ? xrow : -1;
-                if (TRAIN && src >= 0) src = batch_row(p.tr, src);
                 __align__(16) __nv_bfloat16 h[8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const int k = k8 * 8 + j;
-                    h[j] = __float2bfloat16(src >= 0 && k < n_in ? p.X[src * n_in + k] : 0.0f);
+                    h[j] = __float2bfloat16(xrow < p.rows && k < n_in ? p.X[xrow * n_in + k] : 0.0f);
                 }
-                if (TRAIN && e == 0 && xrow < p.rows)
-                    *reinterpret_cast<uint4 *>(p.tr.xb + xrow * p.k0p + k8 * 8) = *reinterpret_cast<const uint4 *>(h);
                 *reinterpret_cast<uint4 *>(Xs + (size_t)g * 16) = *reinterpret_cast<const uint4 *>(h);
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -355,8 +233,8 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // sixteen columns at a time, the next ones on their way while these are worked on
                 uint32_t v[2][16];
-                if (part * 32 < width) tc_load16(v[0], lanes + (uint32_t)(part * 32));
-                for (int n0 = part * 32; n0 < width; n0 += kStep) {
+                tc_load16(v[0], lanes + (uint32_t)(part * 32));
+                for (int n0 = part * 32; n0 < width; n0 += 64) {
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         float4 bv[4];
@@ -365,46 +243,25 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
                             bv[j] = reinterpret_cast<const float4 *>(bias + n0 + 16 * half)[j];
                         tc_loaded(v[half]);
                         if (half == 0) tc_load16(v[1], lanes + (uint32_t)(n0 + 16));
-                        else if (n0 + kStep < width) tc_load16(v[0], lanes + (uint32_t)(n0 + kStep));
+                        else if (n0 + 64 < width) tc_load16(v[0], lanes + (uint32_t)(n0 + 64));
                         __align__(16) __nv_bfloat162 h[8];
                         uint64_t z[8];
                         float zmax = 0.0f;
-                        float gp[TRAIN ? 16 : 1];  // GELU', kept for the way back
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             z[j] = add2(pack2(__uint_as_float(v[half][2 * j]), __uint_as_float(v[half][2 * j + 1])),
                                         j % 2 == 0 ? pack2(bv[j / 2].x, bv[j / 2].y) : pack2(bv[j / 2].z, bv[j / 2].w));
                             const float2 zj = unpack2(z[j]);
                             zmax = fmaxf(zmax, fmaxf(fabsf(zj.x), fabsf(zj.y)));
-                            uint64_t grad;
-                            const float2 g = unpack2(gelu2_f<TRAIN>(z[j], grad));
+                            const float2 g = unpack2(gelu2_f(z[j]));
                             h[j] = __floats2bfloat162_rn(g.x, g.y);
-                            if (TRAIN) {
-                                const float2 d = unpack2(grad);
-                                gp[2 * j] = d.x;
-                                gp[2 * j + 1] = d.y;
-                            }
                         }
                         if (!(zmax <= kGelu2Max)) {  // (a NaN is ignored by fmaxf and propagates through either form)
 #pragma unroll
                             for (int j = 0; j < 8; ++j) {
                                 const float2 zj = unpack2(z[j]);
                                 h[j] = __floats2bfloat162_rn(gelu_f(zj.x), gelu_f(zj.y));
-                                if (TRAIN) {
-                                    gp[2 * j] = gelu_grad_f(zj.x);
-                                    gp[2 * j + 1] = gelu_grad_f(zj.y);
-                                }
                             }
-                        }
-                        if (TRAIN && row < p.rows) {
-                            const int64_t at = ((int64_t)(e * width + n0 + 16 * half) / 8) * p.rows + row;
-                            uint4 *ho = reinterpret_cast<uint4 *>(p.tr.H[l]) + at;
-                            ho[0] = reinterpret_cast<const uint4 *>(h)[0];
-                            ho[p.rows] = reinterpret_cast<const uint4 *>(h)[1];
-                            float4 *go = reinterpret_cast<float4 *>(p.tr.G[l]) + 2 * at - row;
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                go[j * p.rows] = make_float4(gp[4 * j], gp[4 * j + 1], gp[4 * j + 2], gp[4 * j + 3]);
                         }
                         unsigned char *o = arow + (n0 / 8 + 2 * half) * 128;
                         *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(h)[0];
@@ -427,84 +284,11 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
                 uint32_t v[16];
                 tc_load16(v, lanes + (uint32_t)n0);
                 tc_loaded(v);
-                if (!TRAIN) {
-                    if (row < p.rows) {
-                        float *o = p.out + e * p.s_member + row * n_out + n0;
+                if (row < p.rows) {
+                    float *o = p.out + e * p.s_member + row * n_out + n0;
 #pragma unroll
-                        for (int j = 0; j < 16; ++j) o[j] = __uint_as_float(v[j]) + bias[n0 + j];
-                    }
-                } else {
-                    // loss, and the gradient of the outputs: the first input of the way back
-                    const int64_t src = row < p.rows ? batch_row(p.tr, row) : -1;
-                    float sq = 0.0f;
-                    __align__(16) __nv_bfloat16 g[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float d = src >= 0 ? __uint_as_float(v[j]) + bias[n0 + j] - p.tr.Y[src * n_out + n0 + j] : 0.0f;
-                        g[j] = __float2bfloat16(2.0f * d * p.tr.inv);
-                        sq += d * d;
-                    }
-                    unsigned char *o = Ps + (size_t)((r >> 3) * (n_out / 8) + n0 / 8) * 128 + (r & 7) * 16;
-                    *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(g)[0];
-                    *reinterpret_cast<uint4 *>(o + 128) = reinterpret_cast<const uint4 *>(g)[1];
-                    if (row < p.rows) {
-                        uint4 *d = reinterpret_cast<uint4 *>(p.tr.dP + (e * p.rows + row) * n_out + n0);
-                        d[0] = reinterpret_cast<const uint4 *>(g)[0];
-                        d[1] = reinterpret_cast<const uint4 *>(g)[1];
-                    }
-#pragma unroll
-                    for (int d = 16; d > 0; d >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, d);
-                    if (lane == 0) atomicAdd(p.tr.loss + e, sq * p.tr.inv);
+                    for (int j = 0; j < 16; ++j) o[j] = __uint_as_float(v[j]) + bias[n0 + j];
                 }
-            }
-            if (TRAIN) {
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) bar_arrive(&bars.pready);
-                // the way back: dZ_l = (dZ_{l+1} W_{l+1}) GELU'(Z_l), over the activations of its last input
-                for (int l = n_hidden - 1; l >= 0; --l, ++n_d) {
-                    ok = warp_wait(bars, &bars.dfull, n_d & 1u);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    for (int n0 = part * 32; n0 < width; n0 += kStep) {
-#pragma unroll
-                        for (int half = 0; half < 2; ++half) {
-                            uint32_t v[16];
-                            tc_load16(v, lanes + (uint32_t)(n0 + 16 * half));
-                            float4 *go = reinterpret_cast<float4 *>(p.tr.G[l]) +
-                                         ((int64_t)(e * width + n0 + 16 * half) / 4) * p.rows + row;
-                            float4 gp[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                gp[j] = row < p.rows ? go[j * p.rows] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                            tc_loaded(v);
-                            __align__(16) __nv_bfloat162 h[8];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                h[2 * j] = __floats2bfloat162_rn(__uint_as_float(v[4 * j]) * gp[j].x,
-                                                                 __uint_as_float(v[4 * j + 1]) * gp[j].y);
-                                h[2 * j + 1] = __floats2bfloat162_rn(__uint_as_float(v[4 * j + 2]) * gp[j].z,
-                                                                     __uint_as_float(v[4 * j + 3]) * gp[j].w);
-                            }
-                            unsigned char *o = arow + (n0 / 8 + 2 * half) * 128;
-                            *reinterpret_cast<uint4 *>(o) = reinterpret_cast<const uint4 *>(h)[0];
-                            *reinterpret_cast<uint4 *>(o + 128) = reinterpret_cast<const uint4 *>(h)[1];
-                            if (row < p.rows) {
-                                uint4 *d = reinterpret_cast<uint4 *>(go);  // over the GELU' just read
-                                d[0] = reinterpret_cast<const uint4 *>(h)[0];
-                                d[2 * p.rows] = reinterpret_cast<const uint4 *>(h)[1];
-                            }
-                        }
-                    }
-                    if (l > 0) {
-                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-                        __syncwarp();
-                        if (lane == 0) bar_arrive(&bars.hready);
-                    }
-                }
-                if (!ok) break;
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -515,50 +299,6 @@ __device__ __forceinline__ void fused_body(const FusedArgs &p)
     __syncthreads();
     if (threadIdx.x == 0 && bars.abort && p.err) atomicExch(p.err, 1);
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
-}
-
-__global__ void __launch_bounds__((kInferWarps + 2) * 32, 2) fused_forward_kernel(const FusedArgs p)
-{
-    fused_body<kInferWarps, kInferStages, false>(p);
-}
-
-// One training batch, forward and back: writes the bf16 inputs and activations of every layer and the bf16
-// gradients of every pre-activation, from which fused_update forms the weights' gradients.  A batch of
-// 1,024 rows is 40 tiles for five members, so a CTA has an SM to itself: 16 epilogue warps, a ring of six
-// stages.  GELU' is kept in FP32 from the way forward, where its exponential is at hand.
-__global__ void __launch_bounds__((kTrainWarps + 2) * 32, 1) fused_train_kernel(const FusedArgs p)
-{
-    fused_body<kTrainWarps, kTrainStages, true>(p);
-}
-
-// The transposed weights as the way back reads them: B[n][k] = W[k][n], the last layer first.
-__global__ void fused_pack_t_kernel(const FusedNet n, const __nv_bfloat16 *wb, unsigned char *packed, int64_t member_bytes)
-{
-    const int slabs = n.width / kSlab;
-    const int64_t pieces = member_bytes / 16;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < pieces * n.n_members;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int e = (int)(t / pieces);
-        int64_t at = (t % pieces) * 16;
-        const int64_t hidden = (int64_t)n.width * n.width + n.width, layer = (int64_t)slabs * slab_bytes(n.width);
-        const __nv_bfloat16 *W = wb + e * n.P + (int64_t)n.n_in * n.width + n.width;  // layer 1
-        int kc = n.n_out / 8, k_first = 0;
-        if (at < last_bytes(n.width, n.n_out)) {
-            W += (n.n_hidden - 1) * hidden;
-        } else {
-            at -= last_bytes(n.width, n.n_out);
-            W += (n.n_hidden - 2 - at / layer) * hidden;
-            at %= layer;
-            k_first = (int)(at / slab_bytes(n.width)) * kSlab;
-            at %= slab_bytes(n.width);
-            kc = kSlab / 8;
-        }
-        const int q = (int)(at / 16), rr = q & 7, k8 = (q >> 3) % kc, r8 = (q >> 3) / kc;
-        __align__(16) __nv_bfloat16 h[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) h[j] = W[(int64_t)(k_first + k8 * 8 + j) * n.width + r8 * 8 + rr];
-        *reinterpret_cast<uint4 *>(packed + t * 16) = *reinterpret_cast<const uint4 *>(h);
-    }
 }
 
 // One 16-byte piece of a packed layer per thread: 8 consecutive inputs of one output, in the canonical
@@ -584,12 +324,13 @@ __global__ void fused_pack_kernel(const FusedNet n, const __nv_bfloat16 *wb, uns
                 at %= layer;
                 k_first = (int)(at / slab_bytes(n.width)) * kSlab;
                 at %= slab_bytes(n.width);
-                kc = kSlab / 8;
             } else {
                 at -= layer * (n.n_hidden - 1);
                 W += (int64_t)(n.n_hidden - 1) * ((int64_t)n.width * n.width + n.width);
-                kc = n.width / 8;
+                k_first = (int)(at / slab_bytes(n.n_out)) * kSlab;
+                at %= slab_bytes(n.n_out);
             }
+            kc = kSlab / 8;
         }
         const int q = (int)(at / 16), rr = q & 7, k8 = (q >> 3) % kc, r8 = (q >> 3) / kc;
         const __nv_bfloat16 *src = W + (int64_t)(r8 * 8 + rr) * K + k_first + k8 * 8;
@@ -599,8 +340,6 @@ __global__ void fused_pack_kernel(const FusedNet n, const __nv_bfloat16 *wb, uns
         *reinterpret_cast<uint4 *>(packed + t * 16) = *reinterpret_cast<const uint4 *>(h);
     }
 }
-
-int padded_inputs(int n_in) { return (n_in + 15) / 16 * 16; }
 
 }  // namespace
 
@@ -624,71 +363,32 @@ cudaError_t fused_pack(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char
     return cudaPeekAtLastError();
 }
 
-int64_t fused_packed_t_bytes(int width, int n_hidden, int n_out)
+cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float *out, int64_t s_member, int *err,
+                          int report_timeout, cudaStream_t st)
 {
-    return last_bytes(width, n_out) + (int64_t)(n_hidden - 1) * (width / kSlab) * slab_bytes(width);
-}
-
-cudaError_t fused_pack_t(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed_t, cudaStream_t st)
-{
-    const int64_t bytes = fused_packed_t_bytes(n.width, n.n_hidden, n.n_out);
-    const int64_t blocks = (bytes / 16 * n.n_members + 255) / 256;
-    fused_pack_t_kernel<<<(unsigned)(blocks < 2432 ? blocks : 2432), 256, 0, st>>>(n, wb, packed_t, bytes);
-    return cudaPeekAtLastError();
-}
-
-namespace {
-
-FusedArgs fused_args(const FusedNet &n, const float *X, int64_t rows, int *err, int report_timeout)
-{
+    if (rows <= 0) return cudaSuccess;
     FusedArgs p{};
     p.net = n;
     p.X = X;
     p.rows = rows;
+    p.out = out;
+    p.s_member = s_member;
     p.err = err;
     p.report_timeout = report_timeout;
     p.k0p = padded_inputs(n.n_in);
     p.member_bytes = fused_packed_bytes(n.n_in, n.width, n.n_hidden, n.n_out);
     p.mtiles = (int)((rows + kRows - 1) / kRows);
     p.items = p.mtiles * n.n_members;
-    return p;
-}
-
-template <typename K>
-cudaError_t fused_launch(K kernel, const FusedArgs &p, int warps, int stages, int per_sm, int extra, cudaStream_t st)
-{
-    const FusedNet &n = p.net;
-    const int smem = stages * kStageBytes + kRows * n.width * 2 + kRows * p.k0p * 2 + extra +
+    const int smem = kStages * kStageBytes + kRows * n.width * 2 + kRows * p.k0p * 2 +
                      2 * 4 * (n.n_hidden * n.width + n.n_out);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      200 * 1024);
     if (e != cudaSuccess) return e;
-    kernel<<<p.items < per_sm * sms ? p.items : per_sm * sms, (warps + 2) * 32, smem, st>>>(p);
+    fused_forward_kernel<<<p.items < 2 * sms ? p.items : 2 * sms, kThreads, smem, st>>>(p);
     return cudaPeekAtLastError();
-}
-
-}  // namespace
-
-cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float *out, int64_t s_member, int *err,
-                          int report_timeout, cudaStream_t st)
-{
-    if (rows <= 0) return cudaSuccess;
-    FusedArgs p = fused_args(n, X, rows, err, report_timeout);
-    p.out = out;
-    p.s_member = s_member;
-    return fused_launch(fused_forward_kernel, p, kInferWarps, kInferStages, 2, 0, st);
-}
-
-cudaError_t fused_train(const FusedNet &n, const TrainArgs &tr, const float *X, int64_t rows, int *err,
-                        int report_timeout, cudaStream_t st)
-{
-    if (rows <= 0) return cudaSuccess;
-    FusedArgs p = fused_args(n, X, rows, err, report_timeout);
-    p.tr = tr;
-    p.tr.member_bytes_t = fused_packed_t_bytes(n.width, n.n_hidden, n.n_out);
-    return fused_launch(fused_train_kernel, p, kTrainWarps, kTrainStages, 1, kRows * n.n_out * 2, st);
 }
 
 }  // namespace cpmmlp

@@ -16,8 +16,8 @@ struct FusedNet {
     int64_t P;                   // per member
     const unsigned char *packed; // weights as fused_pack lays them out
 };
-constexpr int kFusedSlab = 32;       // K of a packed slab of a hidden layer
 constexpr int kFusedMaxHidden = 16;
+inline int padded_inputs(int n_in) { return (n_in + 15) / 16 * 16; }  // K of the first layer
 bool fused_fits(int n_in, int width, int n_out);
 int64_t fused_packed_bytes(int n_in, int width, int n_hidden, int n_out);  // per member
 cudaError_t fused_pack(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed, cudaStream_t st);
@@ -30,17 +30,19 @@ struct TrainArgs {
     const float *Y;
     const int32_t *order;
     int64_t off, n_total;
-    __nv_bfloat16 *xb;                  // [rows][inputs padded to 16]
-    // Per hidden layer, 16-byte pieces of a row, neighbouring rows next to each other (a warp's lanes are rows):
-    __nv_bfloat16 *H[kFusedMaxHidden];  // [member][width / 8][row][8]: outputs
-    float *G[kFusedMaxHidden];          // [member][width / 4][row][4]: GELU'; the way back puts the bf16 gradients of
-                                        // the pre-activations over it, 8 in the first of each two pieces
-    __nv_bfloat16 *dP;                  // [member][row][n_out]: gradient of the outputs
+    // Operands of the weight gradients, 8 rows of a column in 16 bytes (R = rows / 8, rounded up; rows past the
+    // batch are zero):
+    __nv_bfloat16 *xb;                  // [R][inputs padded to 16][8]
+    __nv_bfloat16 *H[kFusedMaxHidden];  // per hidden layer [member][R][width][8]: outputs
+    float *G[kFusedMaxHidden];          // [member][R][2][width][4]: GELU'; the way back puts the bf16 gradients of
+                                        // the pre-activations over the first half, [width][8]
+    __nv_bfloat16 *dP;                  // [member][R][n_out][8]: gradient of the outputs
     float *loss;                        // per member, added to
     float inv;                          // 1 / (rows n_out)
     int *bad;                           // set where order[] points outside the data
     const unsigned char *packed_t;      // transposed weights (fused_pack_t)
     int64_t member_bytes_t;
+    bool chained;                       // the launch before this one in the stream is a fused_update
 };
 int64_t fused_packed_t_bytes(int width, int n_hidden, int n_out);  // per member
 cudaError_t fused_pack_t(const FusedNet &n, const __nv_bfloat16 *wb, unsigned char *packed_t, cudaStream_t st);
@@ -168,7 +170,11 @@ __device__ __forceinline__ uint64_t gelu2_f(uint64_t z, uint64_t &grad)
     if (GRAD) grad = fma2(mul2(z, both(0.39894228040143268f)), dens, cdf);
     return mul2(z, cdf);
 }
-
+__device__ __forceinline__ uint64_t gelu2_f(uint64_t z)
+{
+    uint64_t grad;
+    return gelu2_f<false>(z, grad);
+}
 
 constexpr uint32_t kTcSpinLimit = 1u << 22;
 
