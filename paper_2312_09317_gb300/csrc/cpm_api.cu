@@ -1069,6 +1069,7 @@ struct cpm_batch {
     int *d_err = nullptr;                // barrier timeout flag
     uint32_t loop_grid = 0;              // CTAs of the last persistent launch
     bool track = false;                  // composite variable tracking in every member
+    bool motile = false;                 // a member has a field or persistence directions
     uint32_t span_threads = 0;           // threads of a CTA there
     uint32_t span_smem = 0;              // shared memory per CTA where every member runs in one CTA, else 0
     bool descriptors_dirty = true;
@@ -1189,7 +1190,7 @@ int batch_build_graph(cpm_batch *b)
     size_t active = b->order.size();
     for (uint32_t q = 0; q < r_max && e == cudaSuccess; q++) {
         while (active > 0 && b->lats[b->order[active - 1]].R <= q) active--;
-        e = launch_batch_round(b->dim, b->perim, b->act, b->track, b->d_lats, b->d_items, b->items_upto[active], q,
+        e = launch_batch_round(b->dim, b->perim, b->act, b->track || b->motile, b->d_lats, b->d_items, b->items_upto[active], q,
                                batch_threads(b), q > 0, b->capture_stream);
         n++;
     }
@@ -1284,6 +1285,7 @@ int cpm_batch_create(const cpm_config *cfgs, int32_t n, void *cuda_stream, cpm_b
         BatchLattice L;
         memset(&L, 0, sizeof L);
         L.base = round_args(h);
+        b->motile = b->motile || L.base.chem || L.base.pers_dir;
         L.bufs = lattice_bufs(h);
         L.k = h->k;
         L.C = h->C;
@@ -1378,7 +1380,7 @@ int cpm_batch_step(cpm_batch *b, int64_t n_mcs)
             p.next = b->d_next;
             cudaError_t e = cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned long long), b->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(b->d_next, 0, sizeof(unsigned) * p.r_max, b->stream);
-            if (e == cudaSuccess) e = launch_batch_loop(b->dim, b->perim, b->act, p, batch_threads(b), b->stream,
+            if (e == cudaSuccess) e = launch_batch_loop(b->dim, b->perim, b->act, b->motile, p, batch_threads(b), b->stream,
                                                         &b->loop_grid);
             int timed_out = 0;
             if (e == cudaSuccess) e = cudaMemcpyAsync(&timed_out, b->d_err, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
@@ -1396,10 +1398,10 @@ int cpm_batch_step(cpm_batch *b, int64_t n_mcs)
             const uint32_t m = (uint32_t)std::min<int64_t>(n_mcs - done, 256);
             const uint32_t n = (uint32_t)b->lats.size();
             cudaError_t e = b->dim == 3
-                                ? launch_batch_span_3d(b->perim, b->act, b->d_lats, n, m, b->span_threads, b->span_smem,
-                                                       b->stream)
-                                : launch_batch_span_2d(b->perim, b->act, b->d_lats, n, m, b->span_threads, b->span_smem,
-                                                       b->stream);
+                                ? launch_batch_span_3d(b->perim, b->act, b->motile, b->d_lats, n, m, b->span_threads,
+                                                       b->span_smem, b->stream)
+                                : launch_batch_span_2d(b->perim, b->act, b->motile, b->d_lats, n, m, b->span_threads,
+                                                       b->span_smem, b->stream);
             if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
             b->launches += 1;
             done += m;

@@ -233,12 +233,13 @@ struct BatchLattice {
 };
 // n_mcs MCS of every member in one launch, a CTA of `threads` each (cpm_span.cuh); smem: the largest member's span_bytes
 constexpr uint32_t kBatchSpanThreads = 256;  // most threads of a CTA
-cudaError_t launch_batch_span_2d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
-                                 uint32_t smem, cudaStream_t st);
-cudaError_t launch_batch_span_3d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
-                                 uint32_t smem, cudaStream_t st);
+cudaError_t launch_batch_span_2d(bool perim, bool act, bool motile, BatchLattice *lats, uint32_t n, uint32_t n_mcs,
+                                 uint32_t threads, uint32_t smem, cudaStream_t st);
+cudaError_t launch_batch_span_3d(bool perim, bool act, bool motile, BatchLattice *lats, uint32_t n, uint32_t n_mcs,
+                                 uint32_t threads, uint32_t smem, cudaStream_t st);
 // after_round: the kernel before it on the stream is a round of the same MCS (programmatic dependent launch)
-cudaError_t launch_batch_round(int dim, bool perim, bool act, bool track, const BatchLattice *lats,
+// extra: members have tracked centroids, a field or persistence directions
+cudaError_t launch_batch_round(int dim, bool perim, bool act, bool extra, const BatchLattice *lats,
                                const int4 *items, uint32_t n_items, uint32_t q, uint32_t threads, bool after_round,
                                cudaStream_t st);
 // the colours of every member's sub-passes of its current MCS
@@ -264,7 +265,7 @@ struct BatchLoopArgs {
     uint32_t max_items;       // items of the fullest round (bounds the grid)
     int test_absent;          // test of the timeout path: CTA 0 leaves before its first barrier
 };
-cudaError_t launch_batch_loop(int dim, bool perim, bool act, const BatchLoopArgs &p, uint32_t threads, cudaStream_t st,
+cudaError_t launch_batch_loop(int dim, bool perim, bool act, bool motile, const BatchLoopArgs &p, uint32_t threads, cudaStream_t st,
                               uint32_t *grid_out);
 
 // Observations of a batch (cpm_batch_observe): one item per lattice.

@@ -34,7 +34,7 @@ __device__ __forceinline__ void around(uint32_t x, uint32_t n, uint32_t out[3])
 }
 
 // The attempts of one brick (kx, ky, kz) of active blocks by one CTA, a thread each (x fastest).
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __device__ __forceinline__ void round_brick(const RoundArgs &a, const RoundBufs &b, const RoundPos &p,
                                             const SmemTables &sm, Survivors &q, uint32_t kx, uint32_t ky, uint32_t kz)
 {
@@ -45,7 +45,7 @@ __device__ __forceinline__ void round_brick(const RoundArgs &a, const RoundBufs 
     const bool valid = ix < a.nax && iy < a.nay && iz < a.naz;
     Draw d{};
     if (valid) d = round_draw<DIM>(a, p, ix, iy, iz, ix + a.nax * (iy + a.nay * iz));
-    round_cta<DIM, PERIM, ACT, TRACK, 4>(a, b, p.t, sm, q, q.n[0], valid, d);
+    round_cta<DIM, PERIM, ACT, EXTRA, 4>(a, b, p.t, sm, q, q.n[0], valid, d);
 }
 
 // Resident CTAs per SM (register budget).  A round is bound by the instructions of its attempts and by
@@ -54,9 +54,9 @@ __device__ __forceinline__ void round_brick(const RoundArgs &a, const RoundBufs 
 // ms per MCS, 256^3 cube cells 0.61 / 0.63 ms.
 constexpr int kRoundMinBlocks = 5;
 
-// TRACK: composite variable tracking on (b.Sc, b.Sn, b.tpend_* set), a kernel
-// of its own so that the sweep without it carries none of its code
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+// EXTRA: composite variable tracking (b.Sc, b.Sn, b.tpend_* set), a field or persistence directions, a
+// kernel of its own so that the sweep without them carries none of their code
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kRoundMinBlocks)
     round_kernel(const RoundArgs a, const RoundBufs b, const RoundPos p)
 {
@@ -74,13 +74,13 @@ __global__ void __launch_bounds__(kThreads, kRoundMinBlocks)
         ky = kx / a.nbr_x % a.nbr_y;
         kx %= a.nbr_x;
     }
-    round_brick<DIM, PERIM, ACT, TRACK>(a, b, p, sm, queue, kx, ky, kz);
+    round_brick<DIM, PERIM, ACT, EXTRA>(a, b, p, sm, queue, kx, ky, kz);
 }
 
 // One (lattice, brick) item of batch round q: lattice it.x's round number
 // g_start + q, exactly as the single-lattice round kernel would run it (same
 // colour, counters and tallies).  ra, rb, rp, sm and queue are the CTA's shared set-up.
-template <int DIM, bool PERIM, bool ACT, bool TRACK = false>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __device__ __forceinline__ void batch_round_item(RoundArgs &ra, RoundBufs &rb, RoundPos &rp, SmemTables &sm,
                                                  Survivors &queue,
                                                  const BatchLattice *lats, int4 it, uint32_t q, uint32_t pdl)
@@ -107,12 +107,12 @@ __device__ __forceinline__ void batch_round_item(RoundArgs &ra, RoundBufs &rb, R
     }
     load_tables(sm, ra, ACT);
     __syncthreads();
-    round_brick<DIM, PERIM, ACT, TRACK>(ra, rb, rp, sm, queue, (uint32_t)it.y, (uint32_t)it.z, (uint32_t)it.w);
+    round_brick<DIM, PERIM, ACT, EXTRA>(ra, rb, rp, sm, queue, (uint32_t)it.y, (uint32_t)it.z, (uint32_t)it.w);
 }
 
 // Batched round: every CTA takes one (lattice, brick) item.
-// TRACK: every member keeps its tracked centroid sums (LatticeBufs::S)
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+// EXTRA: members keep tracked centroid sums (LatticeBufs::S), or have a field or persistence directions
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __global__ void __launch_bounds__(kBatchMaxThreads, kRoundMinBlocks)
     batch_round_kernel(const BatchLattice *lats, const int4 *items, uint32_t q)
 {
@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads, kRoundMinBlocks)
     __shared__ RoundPos rp;
     __shared__ SmemTables sm;
     __shared__ Survivors queue;
-    batch_round_item<DIM, PERIM, ACT, TRACK>(ra, rb, rp, sm, queue, lats, items[blockIdx.x], q, 1);
+    batch_round_item<DIM, PERIM, ACT, EXTRA>(ra, rb, rp, sm, queue, lats, items[blockIdx.x], q, 1);
 }
 
 // Colours of the sub-passes of one member's current MCS, one cycle per thread: a Fisher-Yates shuffle of
@@ -202,7 +202,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *bar, unsigned l
 // counters, each phase closed by a grid barrier.  The work and its order
 // within a phase are those of the per-round launches, so the result is the
 // same bit for bit.
-template <int DIM, bool PERIM, bool ACT>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __global__ void __launch_bounds__(kBatchMaxThreads, kRoundMinBlocks)
     batch_loop_kernel(BatchLattice *lats, uint32_t n_lats, const int4 *items, const uint32_t *upto_q, uint32_t r_max,
                       const int2 *clamp, uint32_t n_clamp, uint32_t n_mcs, unsigned long long *bar, unsigned *next,
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads, kRoundMinBlocks)
                 __syncthreads();
                 const uint32_t k = claim_s;
                 if (k >= n_items) break;
-                batch_round_item<DIM, PERIM, ACT>(ra, rb, rp, sm, queue, lats, items[k], q, 0);
+                batch_round_item<DIM, PERIM, ACT, EXTRA>(ra, rb, rp, sm, queue, lats, items[k], q, 0);
             }
             target += gridDim.x;
             if (!grid_barrier(bar, target, max_polls, err, ok_s)) return;
@@ -320,7 +320,7 @@ unsigned grid_for(uint64_t n, unsigned threads)
     return (unsigned)(g == 0 ? 1 : g);
 }
 
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, cudaStream_t st)
 {
     const auto bricks = [](uint32_t n, uint32_t log2) { return (n + (1u << log2) - 1) >> log2; };
@@ -334,7 +334,7 @@ cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, c
     }
     const unsigned threads = 1u << (a.brick_lx + a.brick_ly + (DIM == 3 ? a.brick_lz : 0));
     if (!a.pdl) {
-        round_kernel<DIM, PERIM, ACT, TRACK><<<blocks, threads, 0, st>>>(a, b, p);
+        round_kernel<DIM, PERIM, ACT, EXTRA><<<blocks, threads, 0, st>>>(a, b, p);
         return cudaGetLastError();
     }
     // programmatic dependent launch: the CTAs of this round may start while the
@@ -350,13 +350,14 @@ cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, round_kernel<DIM, PERIM, ACT, TRACK>, a, b, p);
+    return cudaLaunchKernelEx(&cfg, round_kernel<DIM, PERIM, ACT, EXTRA>, a, b, p);
 }
 
 template <int DIM, bool PERIM, bool ACT>
 cudaError_t launch_round_t(const RoundArgs &a, const RoundBufs &b, const RoundPos &p, cudaStream_t st)
 {
-    return b.Sc ? launch_round_t<DIM, PERIM, ACT, true>(a, b, p, st) : launch_round_t<DIM, PERIM, ACT, false>(a, b, p, st);
+    return b.Sc || a.chem || a.pers_dir ? launch_round_t<DIM, PERIM, ACT, true>(a, b, p, st)
+                                        : launch_round_t<DIM, PERIM, ACT, false>(a, b, p, st);
 }
 
 }  // namespace
@@ -411,10 +412,10 @@ cudaError_t launch_batch_advance(BatchLattice *lats, uint32_t n, cudaStream_t st
     return cudaGetLastError();
 }
 
-template <int DIM, bool PERIM, bool ACT>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 cudaError_t launch_batch_loop_t(const BatchLoopArgs &p, uint32_t threads, cudaStream_t st, uint32_t *grid_out)
 {
-    auto kern = batch_loop_kernel<DIM, PERIM, ACT>;
+    auto kern = batch_loop_kernel<DIM, PERIM, ACT, EXTRA>;
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -440,23 +441,23 @@ cudaError_t launch_batch_loop_t(const BatchLoopArgs &p, uint32_t threads, cudaSt
     return cudaLaunchCooperativeKernel((const void *)kern, dim3((unsigned)grid), dim3(threads), args, 0, st);
 }
 
-cudaError_t launch_batch_loop(int dim, bool perim, bool act, const BatchLoopArgs &p, uint32_t threads, cudaStream_t st,
-                              uint32_t *grid_out)
+cudaError_t launch_batch_loop(int dim, bool perim, bool act, bool motile, const BatchLoopArgs &p, uint32_t threads,
+                              cudaStream_t st, uint32_t *grid_out)
 {
+#define CPM_LOOP(D, PE, AC)                                                                                    \
+    (motile ? launch_batch_loop_t<D, PE, AC, true>(p, threads, st, grid_out)                                   \
+            : launch_batch_loop_t<D, PE, AC, false>(p, threads, st, grid_out))
     if (dim == 2) {
-        if (act) return perim ? launch_batch_loop_t<2, true, true>(p, threads, st, grid_out)
-                              : launch_batch_loop_t<2, false, true>(p, threads, st, grid_out);
-        return perim ? launch_batch_loop_t<2, true, false>(p, threads, st, grid_out)
-                     : launch_batch_loop_t<2, false, false>(p, threads, st, grid_out);
+        if (act) return perim ? CPM_LOOP(2, true, true) : CPM_LOOP(2, false, true);
+        return perim ? CPM_LOOP(2, true, false) : CPM_LOOP(2, false, false);
     }
-    if (act) return perim ? launch_batch_loop_t<3, true, true>(p, threads, st, grid_out)
-                          : launch_batch_loop_t<3, false, true>(p, threads, st, grid_out);
-    return perim ? launch_batch_loop_t<3, true, false>(p, threads, st, grid_out)
-                 : launch_batch_loop_t<3, false, false>(p, threads, st, grid_out);
+    if (act) return perim ? CPM_LOOP(3, true, true) : CPM_LOOP(3, false, true);
+    return perim ? CPM_LOOP(3, true, false) : CPM_LOOP(3, false, false);
+#undef CPM_LOOP
 }
 
 template <int DIM, bool PERIM, bool ACT>
-cudaError_t batch_round_t(bool track, const BatchLattice *lats, const int4 *items, uint32_t n_items, uint32_t q,
+cudaError_t batch_round_t(bool extra, const BatchLattice *lats, const int4 *items, uint32_t n_items, uint32_t q,
                           uint32_t threads, bool after_round, cudaStream_t st)
 {
     cudaLaunchConfig_t cfg = {};
@@ -468,25 +469,25 @@ cudaError_t batch_round_t(bool track, const BatchLattice *lats, const int4 *item
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = after_round ? 1 : 0;
-    return track ? cudaLaunchKernelEx(&cfg, batch_round_kernel<DIM, PERIM, ACT, true>, lats, items, q)
+    return extra ? cudaLaunchKernelEx(&cfg, batch_round_kernel<DIM, PERIM, ACT, true>, lats, items, q)
                  : cudaLaunchKernelEx(&cfg, batch_round_kernel<DIM, PERIM, ACT, false>, lats, items, q);
 }
 
-cudaError_t launch_batch_round(int dim, bool perim, bool act, bool track, const BatchLattice *lats,
+cudaError_t launch_batch_round(int dim, bool perim, bool act, bool extra, const BatchLattice *lats,
                                const int4 *items, uint32_t n_items, uint32_t q, uint32_t threads, bool after_round,
                                cudaStream_t st)
 {
     if (n_items == 0) return cudaSuccess;
     if (dim == 2) {
-        if (act) return perim ? batch_round_t<2, true, true>(track, lats, items, n_items, q, threads, after_round, st)
-                              : batch_round_t<2, false, true>(track, lats, items, n_items, q, threads, after_round, st);
-        return perim ? batch_round_t<2, true, false>(track, lats, items, n_items, q, threads, after_round, st)
-                     : batch_round_t<2, false, false>(track, lats, items, n_items, q, threads, after_round, st);
+        if (act) return perim ? batch_round_t<2, true, true>(extra, lats, items, n_items, q, threads, after_round, st)
+                              : batch_round_t<2, false, true>(extra, lats, items, n_items, q, threads, after_round, st);
+        return perim ? batch_round_t<2, true, false>(extra, lats, items, n_items, q, threads, after_round, st)
+                     : batch_round_t<2, false, false>(extra, lats, items, n_items, q, threads, after_round, st);
     }
-    if (act) return perim ? batch_round_t<3, true, true>(track, lats, items, n_items, q, threads, after_round, st)
-                          : batch_round_t<3, false, true>(track, lats, items, n_items, q, threads, after_round, st);
-    return perim ? batch_round_t<3, true, false>(track, lats, items, n_items, q, threads, after_round, st)
-                 : batch_round_t<3, false, false>(track, lats, items, n_items, q, threads, after_round, st);
+    if (act) return perim ? batch_round_t<3, true, true>(extra, lats, items, n_items, q, threads, after_round, st)
+                          : batch_round_t<3, false, true>(extra, lats, items, n_items, q, threads, after_round, st);
+    return perim ? batch_round_t<3, true, false>(extra, lats, items, n_items, q, threads, after_round, st)
+                 : batch_round_t<3, false, false>(extra, lats, items, n_items, q, threads, after_round, st);
 }
 
 cudaError_t launch_recount(int dim, const int32_t *lat, const uint8_t *, int32_t *V, int32_t *A, uint32_t nx,

@@ -155,73 +155,7 @@ __device__ __forceinline__ uint32_t mean_index(const SmemTables &sm, int32_t sum
     return __umulhi(2u * (uint32_t)sum, sm.inv[count]) >> 6;
 }
 
-// Motility terms (Eq. 4, Eq. 5) of the copy from the source (stencil index
-// ox, oy, oz around the target) into the target, in 1/16 energy units: the
-// moving cell is si (sj when si is the medium), d = target - source, and
-// each term is floor(e) with e formed by the same rounded double operations,
-// in the same order, as the replay: chemotaxis
-// e = ((double)(-16 lambda (d . C_q)) / 16384) * (1/|d|), persistence
-// e = ((d_x p_x + d_y p_y + d_z p_z) * (double)(-16 lambda)) * (1/|d|).
-// Kept out of line: the round kernels call it only when a field or a
-// persistence direction is set, and inlining its FP64 code into every round
-// kernel enlarges them (instruction-fetch stalls).
-template <int DIM>
-__device__ __noinline__ int64_t motility_q(const RoundArgs &a, int32_t si, int32_t sj, int ti, int tj, int ox,
-                                              int oy, int oz, uint32_t isite)
-{
-    const int32_t m = si > 0 ? si : sj;
-    const int tp = si > 0 ? ti : tj;
-    const int dx = 1 - ox, dy = 1 - oy, dz = DIM == 3 ? 1 - oz : 0;
-    const double il = a.tp.inv_len[dx * dx + dy * dy + dz * dz];
-    int64_t dh = 0;
-    if (a.chem && a.tp.lambda_chem[tp] != 0) {
-        const int16_t *c = a.chem + (size_t)isite * DIM;
-        int64_t dc = (int64_t)dx * c[0] + (int64_t)dy * c[1];
-        if (DIM == 3) dc += (int64_t)dz * c[2];
-        const double e = __dmul_rn((double)(-16 * (int64_t)a.tp.lambda_chem[tp] * dc) / 16384.0, il);
-        dh += (int64_t)floor(e);
-    }
-    if (a.pers_dir && a.tp.lambda_pers[tp] != 0 && m > 0) {
-        const double *ph = a.pers_dir + 3 * (size_t)m;
-        double sd = __dmul_rn((double)dx, ph[0]);
-        sd = __dadd_rn(sd, __dmul_rn((double)dy, ph[1]));
-        sd = __dadd_rn(sd, __dmul_rn((double)dz, ph[2]));
-        const double e = __dmul_rn(__dmul_rn(sd, (double)(-16 * (int64_t)a.tp.lambda_pers[tp])), il);
-        dh += (int64_t)floor(e);
-    }
-    return dh;
-}
-
-// Composite variable tracking (Eq. 11).  A copy into site j adds j to sigma_i and
-// removes it from sigma_j, each at its periodic image nearest that cell's centroid
-// as the round began (Sc / Vc); the image shifts (-3..3 per axis, 3 bits each:
-// sigma_i's in bits 0..8, sigma_j's in bits 9..17) travel with the pending change,
-// so that the next round adds the same amounts to the other buffer.
-template <int DIM>
-__device__ __noinline__ int2 track_accept(const RoundArgs &a, const RoundBufs &b, int32_t si, int32_t sj, uint32_t j, uint32_t jx,
-                                          uint32_t jy, uint32_t jz)
-{
-    uint32_t bits = 0;
-    const int64_t Vi = si > 0 ? b.Vc[si] : 0, Vj = sj > 0 ? b.Vc[sj] : 0;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-        const int64_t x = d == 0 ? jx : (d == 1 ? jy : jz);
-        const int64_t n = d == 0 ? a.nx : (d == 1 ? a.ny : a.nz);
-        if (si > 0) {
-            const int64_t k = track_image_shift(x, b.Sc[3 * si + d], Vi, n);
-            atomicAdd((unsigned long long *)(b.Sn + 3 * si + d), (unsigned long long)(x + n * k));
-            bits |= (uint32_t)(k + 3) << (3 * d);
-        }
-        if (sj > 0) {
-            const int64_t k = track_image_shift(x, b.Sc[3 * sj + d], Vj, n);
-            atomicAdd((unsigned long long *)(b.Sn + 3 * sj + d), (unsigned long long)(-(x + n * k)));
-            bits |= (uint32_t)(k + 3) << (9 + 3 * d);
-        }
-    }
-    return make_int2((int32_t)j, (int32_t)bits);
-}
-
-// the previous round's tracked change (see track_accept) into the other buffer
+// the previous round's tracked change (see round_cta) into the other buffer
 template <int DIM>
 __device__ __noinline__ void track_carry(const RoundArgs &a, const RoundBufs &b, int32_t si, int32_t sj, int2 e)
 {
@@ -359,7 +293,7 @@ __device__ __forceinline__ Draw round_draw(const RoundArgs &a, const RoundPos &p
 // Measured against that (ms per MCS): 256^3 cube cells 0.911 -> 0.597, 1024^3 fibre tissue
 // 189.2 -> 143.3, 64 uneven lattices of a sweep 5.00 -> 2.90.  Eight lanes per survivor and a queue
 // per warp: 0.976 and 180.7; two attempts per lane (half the warps): 1.46 and 336.
-template <int DIM, bool PERIM, bool ACT, bool TRACK, int G>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, int G>
 __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b, uint32_t t, const SmemTables &sm,
                                           Survivors &q, uint32_t &n_queue, bool valid, const Draw &d,
                                           uint32_t first_warp = 0)
@@ -391,7 +325,7 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
                 const int4 e = b.pend_prev[i];
                 if (e.x > 0) { atomicAdd(b.Vn + e.x, 1); atomicAdd(b.An + e.x, e.z); }
                 if (e.y > 0) { atomicAdd(b.Vn + e.y, -1); atomicAdd(b.An + e.y, e.w); }
-                if (TRACK) track_carry<DIM>(a, b, e.x, e.y, b.tpend_prev[i]);
+                if (EXTRA && b.Sc) track_carry<DIM>(a, b, e.x, e.y, b.tpend_prev[i]);
             }
             const int32_t sj = cell_id(wj), si = cell_id(wi);
             alive = si != sj && si >= 0 && sj >= 0;
@@ -426,6 +360,39 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
         if (sub < (PERIM ? 4u : 2u)) {
             const int32_t cell = sub & 1u ? sj : si;
             if (cell > 0) tal = (sub & 2u ? b.Ac : b.Vc)[cell];
+        }
+        const uint32_t dir = s.i_dir >> kDirShift<DIM>;
+        const int ox = (int)(dir % 3), oy = (int)((dir / 3) % 3), oz = DIM == 3 ? (int)(dir / 9) : 1;
+        // Motility (Eq. 4, Eq. 5) and tracked centroids (Eq. 11), read with the tallies: the field at the source by
+        // lane 0, the moving cell's persistence direction by lane 1, the tracked sums of both cells by a lane per
+        // cell and axis.
+        constexpr int kSums = EXTRA ? (2 * DIM + G - 1) / G : 0;
+        int32_t fx = 0, fy = 0, fz = 0;
+        double hx = 0.0, hy = 0.0, hz = 0.0;
+        int64_t sums[kSums > 0 ? kSums : 1];
+        if (EXTRA) {
+            const int32_t moving = si > 0 ? si : sj;
+            if (a.chem && sub == 0) {
+                const uint32_t isite = wrap_step(s.x, ox - 1, a.nx) +
+                                       a.nx * (wrap_step(s.y, oy - 1, a.ny) +
+                                               a.ny * (DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0));
+                const int16_t *c = a.chem + (size_t)isite * DIM;
+                fx = c[0];
+                fy = c[1];
+                if (DIM == 3) fz = c[2];
+            }
+            if (a.pers_dir && sub == 1 && moving > 0) {
+                const double *p = a.pers_dir + 3 * (size_t)moving;
+                hx = p[0];
+                hy = p[1];
+                if (DIM == 3) hz = p[2];
+            }
+#pragma unroll
+            for (int k = 0; k < kSums; ++k) {
+                const int at = (int)sub + k * G;  // cell at / DIM, axis at % DIM
+                const int32_t cell = at < DIM ? si : sj;
+                sums[k] = b.Sc && at < 2 * DIM && cell > 0 ? b.Sc[3 * cell + at % DIM] : 0;
+            }
         }
         const Win win(a, sub, s.x, s.y, s.z);
         int32_t wn[K];
@@ -497,13 +464,26 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
                 dh += (int64_t)a.tp.lambda_p[tj] * dAj * (2 * ((int64_t)Aj - a.tp.a_target[tj]) + dAj);
         }
         int64_t dhq = 16 * dh;
-        const uint32_t dir = s.i_dir >> kDirShift<DIM>;
-        const int ox = (int)(dir % 3), oy = (int)((dir / 3) % 3), oz = DIM == 3 ? (int)(dir / 9) : 1;
-        if (a.chem || a.pers_dir) {
-            const uint32_t isite = wrap_step(s.x, ox - 1, a.nx) +
-                                   a.nx * (wrap_step(s.y, oy - 1, a.ny) +
-                                           a.ny * (DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0));
-            dhq += motility_q<DIM>(a, si, sj, ti, tj, ox, oy, oz, isite);
+        if (EXTRA && (a.chem || a.pers_dir)) {
+            // Each term, in 1/16 energy units, is floor(e) with e formed by the rounded double operations of the
+            // replay, d = target - source: chemotaxis e = ((double)(-16 lambda (d . C)) / 16384) * (1/|d|),
+            // persistence e = ((d_x p_x + d_y p_y + d_z p_z) * (double)(-16 lambda)) * (1/|d|).  Double precision is
+            // what a round of motile cells waits for (64 results a warp instruction take an SM 16 cycles), so both
+            // terms go through the same operations, lane 0's chemotaxis and lane 1's persistence; products with
+            // d = -1, 0, 1 and the division by a power of two are exact (256^2 motile cells: 6.2 us a
+            // round with each lane computing both in turn, 4.3 so).
+            const int tp = si > 0 ? ti : tj;
+            const int dx = 1 - ox, dy = 1 - oy, dz = DIM == 3 ? 1 - oz : 0;
+            const bool chem = sub == 0;
+            const auto times = [](int d, double x) { return d == 0 ? 0.0 : (d < 0 ? -x : x); };
+            double v = __dadd_rn(times(dx, hx), times(dy, hy));
+            if (DIM == 3) v = __dadd_rn(v, times(dz, hz));
+            const int64_t along = (int64_t)dx * fx + (int64_t)dy * fy + (int64_t)dz * fz;
+            const double w = (double)(chem ? -16 * (int64_t)a.tp.lambda_chem[tp] * along
+                                           : -16 * (int64_t)a.tp.lambda_pers[tp]);
+            const double e = __dmul_rn(__dmul_rn(chem ? 1.0 / 16384.0 : v, w), a.tp.inv_len[dx * dx + dy * dy + dz * dz]);
+            const int64_t term = (int64_t)floor(e);
+            dhq += __shfl_sync(0xffffffffu, term, 0, G) + __shfl_sync(0xffffffffu, term, 1, G);
         }
         // the test of Eq. 2 at an energy h > 0 (w2 < THR[h]): THR[h] = floor(2^32 exp(-h / 16T)), so it
         // holds exactly for h <= 16 T ln(2^32 / (w2 + 1)).  The logarithm in single precision decides all
@@ -579,6 +559,25 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
         };
         const bool ok = a.narrow ? test(Narrow{}) : test(Wide{});
         const bool leader = sub == 0 && ok;
+        int32_t shifts = 0;
+        if (EXTRA && b.Sc) {
+            // The copy adds its site to sigma_i's sums and removes it from sigma_j's, at the periodic image nearest
+            // that cell's centroid as the round began; the image shifts (-3..3 per axis, 3 bits each: sigma_i's in
+            // bits 0..8, sigma_j's in bits 9..17) travel with the pending change, so that the next round adds the
+            // same amounts to the other buffer.
+#pragma unroll
+            for (int k = 0; k < kSums; ++k) {
+                const int at = (int)sub + k * G, d = at % DIM;
+                const bool of_i = at < DIM;
+                const int32_t cell = of_i ? si : sj;
+                if (!ok || at >= 2 * DIM || cell <= 0) continue;
+                const int64_t x = d == 0 ? s.x : (d == 1 ? s.y : s.z), n = d == 0 ? a.nx : (d == 1 ? a.ny : a.nz);
+                const int64_t shift = track_image_shift(x, sums[k], of_i ? Vi : Vj, n), image = x + n * shift;
+                atomicAdd((unsigned long long *)(b.Sn + 3 * cell + d), (unsigned long long)(of_i ? image : -image));
+                shifts |= (int32_t)(shift + 3) << ((of_i ? 0 : 9) + 3 * d);
+            }
+            shifts = group_sum<G>(shifts);
+        }
         if (leader) {
             const uint32_t i = s.i_dir & kIndexMask;
             // a copy stamps the site with this MCS (a medium copy: age 128, no activity)
@@ -587,8 +586,7 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
             if (sj > 0) { atomicAdd(b.Vn + sj, -1); atomicAdd(b.An + sj, dAj); }
             b.pend_cur[i] = make_int4(si, sj, dAi, dAj);
             b.flag_cur[i] = 1;
-            if (TRACK)
-                b.tpend_cur[i] = track_accept<DIM>(a, b, si, sj, s.x + a.nx * (s.y + a.ny * s.z), s.x, s.y, s.z);
+            if (EXTRA && b.Sc) b.tpend_cur[i] = make_int2((int32_t)(s.x + a.nx * (s.y + a.ny * s.z)), shifts);
         }
         accepted += (uint32_t)__popc(__ballot_sync(0xffffffffu, leader));
     }

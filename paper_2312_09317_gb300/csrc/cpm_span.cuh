@@ -29,7 +29,7 @@ __device__ __forceinline__ uint32_t cluster_rank()
 }
 
 // The rounds p.sp, ... of n_sub sub-passes on the buffers l, by the nc CTAs of a cluster.
-template <int DIM, bool PERIM, bool ACT, bool TRACK, int G>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, int G>
 __device__ __forceinline__ void span_run(const RoundArgs &a, const LatticeBufs &l, const SpanPos &p, uint32_t nc,
                                          const SmemTables &sm, Survivors &q, uint16_t *colours)
 {
@@ -99,7 +99,7 @@ __device__ __forceinline__ void span_run(const RoundArgs &a, const LatticeBufs &
                 if (valid) d = round_draw<DIM>(a, pos, i % a.nax, i / a.nax % a.nay, i / (a.nax * a.nay), i);
             }
             // the warps without attempts of their own are the first to evaluate; the others draw their next ones
-            round_cta<DIM, PERIM, ACT, TRACK, G>(a, b, pos.t, sm, q, q.n[stage & 1u], valid, d, p.lanes / 32);
+            round_cta<DIM, PERIM, ACT, EXTRA, G>(a, b, pos.t, sm, q, q.n[stage & 1u], valid, d, p.lanes / 32);
             if (tid == 0) q.n[(stage & 1u) ^ 1u] = 0;  // last read in the previous stage, used in the next
         }
         arrive();
@@ -187,7 +187,7 @@ __device__ __forceinline__ LatticeBufs span_view(const SpanResident &r, const La
 }
 
 // One lattice, a cluster of p.nc CTAs.
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __global__ void __launch_bounds__(kSpanThreads, 1) span_kernel(const RoundArgs a, const LatticeBufs l, const SpanPos p)
 {
     extern __shared__ __align__(16) unsigned char span_smem[];
@@ -202,14 +202,14 @@ __global__ void __launch_bounds__(kSpanThreads, 1) span_kernel(const RoundArgs a
     if (p.resident) span_load(res, l, n_sites, n_ids, a.n_active);
     if (threadIdx.x == 0) view = p.resident ? span_view(res, l, n_ids, a.n_active) : l;
     __syncthreads();
-    span_run<DIM, PERIM, ACT, TRACK, 8>(a, view, p, p.nc, sm, q, colours);
+    span_run<DIM, PERIM, ACT, EXTRA, 8>(a, view, p, p.nc, sm, q, colours);
     if (p.resident) span_store(res, l, n_sites, n_ids, a.n_active);
 }
 
-template <int DIM, bool PERIM, bool ACT, bool TRACK>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 cudaError_t launch_span_t(const RoundArgs &a, const LatticeBufs &l, SpanPos p, cudaStream_t st)
 {
-    auto kern = span_kernel<DIM, PERIM, ACT, TRACK>;
+    auto kern = span_kernel<DIM, PERIM, ACT, EXTRA>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanMaxSmem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
@@ -233,7 +233,7 @@ cudaError_t launch_span_t(const RoundArgs &a, const LatticeBufs &l, SpanPos p, c
 // three CTAs of 256 per SM (80); with four (64) the spills cost more than the warps give, with two (128)
 // too few members share an SM. us for 5 MCS of runs of 64 x 64 sites (80 rounds), 8 / 300 / 1,024 / 2,048
 // members: 257 / 418 / 972 / 1,571; with a launch per round 403 / 664 / 1,239 / 1,987.
-template <int DIM, bool PERIM, bool ACT>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 __global__ void __launch_bounds__(kBatchSpanThreads, 3) batch_span_kernel(BatchLattice *lats, uint32_t n_mcs)
 {
     extern __shared__ __align__(16) unsigned char span_smem[];
@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(kBatchSpanThreads, 3) batch_span_kernel(BatchL
     p.nc = 1;
     p.lanes = blockDim.x;
     __syncthreads();
-    span_run<DIM, PERIM, ACT, false, 4>(ra, view, p, 1, sm, q, colours);
+    span_run<DIM, PERIM, ACT, EXTRA, 4>(ra, view, p, 1, sm, q, colours);
     span_store(res, L.bufs, n_sites, n_ids, ra.n_active);
     if (threadIdx.x == 0) {
         L.t_start += n_mcs;
@@ -273,11 +273,11 @@ __global__ void __launch_bounds__(kBatchSpanThreads, 3) batch_span_kernel(BatchL
     }
 }
 
-template <int DIM, bool PERIM, bool ACT>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
 cudaError_t launch_batch_span_t(BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads, uint32_t smem,
                                 cudaStream_t st)
 {
-    auto kern = batch_span_kernel<DIM, PERIM, ACT>;
+    auto kern = batch_span_kernel<DIM, PERIM, ACT, EXTRA>;
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanMaxSmem);
     if (e != cudaSuccess) return e;
     kern<<<n, threads, smem, st>>>(lats, n_mcs);
@@ -285,22 +285,24 @@ cudaError_t launch_batch_span_t(BatchLattice *lats, uint32_t n, uint32_t n_mcs, 
 }
 
 template <int DIM>
-cudaError_t launch_batch_span_d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
-                                uint32_t smem, cudaStream_t st)
+cudaError_t launch_batch_span_d(bool perim, bool act, bool motile, BatchLattice *lats, uint32_t n, uint32_t n_mcs,
+                                uint32_t threads, uint32_t smem, cudaStream_t st)
 {
-    if (act) return perim ? launch_batch_span_t<DIM, true, true>(lats, n, n_mcs, threads, smem, st)
-                          : launch_batch_span_t<DIM, false, true>(lats, n, n_mcs, threads, smem, st);
-    return perim ? launch_batch_span_t<DIM, true, false>(lats, n, n_mcs, threads, smem, st)
-                 : launch_batch_span_t<DIM, false, false>(lats, n, n_mcs, threads, smem, st);
+#define CPM_SPAN(PE, AC)                                                                     \
+    (motile ? launch_batch_span_t<DIM, PE, AC, true>(lats, n, n_mcs, threads, smem, st)      \
+            : launch_batch_span_t<DIM, PE, AC, false>(lats, n, n_mcs, threads, smem, st))
+    if (act) return perim ? CPM_SPAN(true, true) : CPM_SPAN(false, true);
+    return perim ? CPM_SPAN(true, false) : CPM_SPAN(false, false);
+#undef CPM_SPAN
 }
 
 template <int DIM>
 cudaError_t launch_span_d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,
                           cudaStream_t st)
 {
-    const bool track = l.S[0] != nullptr;
+    const bool extra = l.S[0] || a.chem || a.pers_dir;
 #define CPM_SPAN(PE, AC) \
-    (track ? launch_span_t<DIM, PE, AC, true>(a, l, p, st) : launch_span_t<DIM, PE, AC, false>(a, l, p, st))
+    (extra ? launch_span_t<DIM, PE, AC, true>(a, l, p, st) : launch_span_t<DIM, PE, AC, false>(a, l, p, st))
     if (act) return perim ? CPM_SPAN(true, true) : CPM_SPAN(false, true);
     return perim ? CPM_SPAN(true, false) : CPM_SPAN(false, false);
 #undef CPM_SPAN

@@ -9,10 +9,10 @@ cudaError_t launch_span_3d(bool perim, bool act, const RoundArgs &a, const Latti
     return launch_span_d<3>(perim, act, a, l, p, st);
 }
 
-cudaError_t launch_batch_span_3d(bool perim, bool act, BatchLattice *lats, uint32_t n, uint32_t n_mcs, uint32_t threads,
-                                 uint32_t smem, cudaStream_t st)
+cudaError_t launch_batch_span_3d(bool perim, bool act, bool motile, BatchLattice *lats, uint32_t n, uint32_t n_mcs,
+                                 uint32_t threads, uint32_t smem, cudaStream_t st)
 {
-    return launch_batch_span_d<3>(perim, act, lats, n, n_mcs, threads, smem, st);
+    return launch_batch_span_d<3>(perim, act, motile, lats, n, n_mcs, threads, smem, st);
 }
 
 }  // namespace cpmgb
