@@ -1046,7 +1046,7 @@ struct cpm_batch {
     std::vector<uint32_t> order;         // lattice indices by rounds per MCS, descending
     std::vector<uint32_t> items_upto;    // round items of the first k lattices in that order
     uint32_t n_clamp_items = 0;
-    uint32_t brick[3] = {8, 4, 4};       // active blocks per CTA (x, y, z)
+    uint32_t brick[3] = {8, 8, 4};       // active blocks per CTA (x, y, z): the survivors of 256 even out best
     BatchLattice *d_lats = nullptr;
     int4 *d_items = nullptr;              // round items: member, brick x y z
     int2 *d_clamp = nullptr;

@@ -335,8 +335,11 @@ cudaError_t launch_tile_epoch(int dim, bool perim, bool act, const TileArgs &a, 
 // shared, and a warp's loads then fall on 16 consecutive 64-byte granules of a row.
 inline void pick_bricks(int dim, RoundArgs &a)
 {
-    uint32_t log2 = 8;
-    while (log2 > 5 && a.n_active < (152u * 2) << log2) log2--;
+    // The survivors of a CTA are shared out over its warps, so large CTAs even out where they cluster: 3D tissue on
+    // 512^3, with 64 / 128 / 256 threads: 28 / 15 / 14 us a round, on 144^3 with 32 / 256: 8.9 / 6.6, cube cells
+    // on 160^3 with 128 / 256: 5.5 / 5.1.  2D rounds are shorter: 400^2 points with 32 / 128 / 256 threads 3.4 / 3.2 /
+    // 3.3, motile cells 9.4 / 8.6 / 8.6.
+    const uint32_t log2 = dim == 3 || a.n_active >= (152u * 2) << 8 ? 8 : 7;
     if (dim == 2) {
         a.brick_lx = (log2 + 1) / 2;
         a.brick_ly = log2 - a.brick_lx;
