@@ -143,6 +143,7 @@ struct RoundPos {
 // What all rounds of a lattice share.
 struct RoundArgs {
     uint32_t packed;           // 1: the words carry Act stamps (Act on for this lattice)
+    uint32_t cubed;            // 1: the lattice lies in cubes (cubed_off)
     uint32_t stream_loads;     // 1: lattice words through the streaming cache path (Act, area edge >= 8)
     uint32_t pdl;              // 1: launched as a programmatic dependent of the previous round
     const uint8_t *cell_type;  // per cell id
@@ -329,8 +330,7 @@ struct TileArgs {
 size_t tile_dyn_smem(int dim, bool act, uint32_t T, uint32_t cap, uint32_t a, uint32_t thr_smem);
 cudaError_t launch_tile_epoch(int dim, bool perim, bool act, const TileArgs &a, uint32_t n_tiles, cudaStream_t st);
 
-// Brick of active blocks per CTA (2^lx x 2^ly x 2^lz, a thread each): 256 of them, fewer where that leaves SMs
-// without a CTA.  3D: 8 along x when active blocks are less than 16 sites apart, where the stencils of
+// Brick of active blocks per CTA (2^lx x 2^ly x 2^lz, a thread each).  3D: 8 along x when active blocks are less than 16 sites apart, where the stencils of
 // neighbouring threads share lines; 16 when they are 16 or more apart and a row has as many: no lines are
 // shared, and a warp's loads then fall on 16 consecutive 64-byte granules of a row.
 inline void pick_bricks(int dim, RoundArgs &a)
@@ -389,6 +389,8 @@ cudaError_t launch_track_init(int dim, const int32_t *lat, uint32_t nx, uint32_t
                               const int32_t *V, uint32_t *anchor, long long *S, cudaStream_t st);
 cudaError_t launch_track_rewrap(int dim, uint32_t nx, uint32_t ny, uint32_t nz, int32_t n_cells, const int32_t *V,
                                 long long *S_complete, long long *S_other, cudaStream_t st);
+// the lattice from rows to cubes (cpm_round.cuh, cubed_off) or back; extents multiples of 8
+cudaError_t launch_cubes(int32_t *cubes, int32_t *rows, uint32_t nx, uint32_t ny, uint32_t nz, bool to_rows, cudaStream_t st);
 cudaError_t launch_act_values(const int32_t *lat, const uint8_t *cell_type, const TypeParams &tp, uint64_t n,
                               uint32_t t_last, uint8_t *out, cudaStream_t st);
 // Lattice words <-> ids: unpack n words into ids; pack n ids into the words

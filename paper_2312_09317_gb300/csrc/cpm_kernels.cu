@@ -34,7 +34,7 @@ __device__ __forceinline__ void around(uint32_t x, uint32_t n, uint32_t out[3])
 }
 
 // The attempts of one brick (kx, ky, kz) of active blocks by one CTA, a thread each (x fastest).
-template <int DIM, bool PERIM, bool ACT, bool EXTRA>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, bool CUBED = false>
 __device__ __forceinline__ void round_brick(const RoundArgs &a, const RoundBufs &b, const RoundPos &p,
                                             const SmemTables &sm, Survivors &q, uint32_t kx, uint32_t ky, uint32_t kz)
 {
@@ -44,19 +44,19 @@ __device__ __forceinline__ void round_brick(const RoundArgs &a, const RoundBufs 
     const uint32_t iz = DIM == 3 ? (kz << a.brick_lz) + (slot >> (lx + ly)) : 0;
     const bool valid = ix < a.nax && iy < a.nay && iz < a.naz;
     Draw d{};
-    if (valid) d = round_draw<DIM>(a, p, ix, iy, iz, ix + a.nax * (iy + a.nay * iz));
-    round_cta<DIM, PERIM, ACT, EXTRA, 4>(a, b, p.t, sm, q, q.n[0], valid, d);
+    if (valid) d = round_draw<DIM, CUBED>(a, p, ix, iy, iz, ix + a.nax * (iy + a.nay * iz));
+    round_cta<DIM, PERIM, ACT, EXTRA, 4, CUBED>(a, b, p.t, sm, q, q.n[0], valid, d);
 }
 
 // Resident CTAs per SM (register budget).  A round is bound by the instructions of its attempts and by
 // the chain of dependent loads, so registers that hold a window's loads in flight are worth more than
-// the warps they cost: 48 registers (five CTAs of 256) against 40 (six): 1024^3 fibre tissue 145.5 / 165.0
-// ms per MCS, 256^3 cube cells 0.61 / 0.63 ms.
+// the warps they cost: 48 registers (five CTAs of 256) against 40 (six): 1024^3 fibre tissue in rows 145.5 /
+// 165.0 ms per MCS, 256^3 cube cells 0.61 / 0.63 ms.
 constexpr int kRoundMinBlocks = 5;
 
 // EXTRA: composite variable tracking (b.Sc, b.Sn, b.tpend_* set), a field or persistence directions, a
 // kernel of its own so that the sweep without them carries none of their code
-template <int DIM, bool PERIM, bool ACT, bool EXTRA>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, bool CUBED>
 __global__ void __launch_bounds__(kThreads, kRoundMinBlocks)
     round_kernel(const RoundArgs a, const RoundBufs b, const RoundPos p)
 {
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kThreads, kRoundMinBlocks)
         ky = kx / a.nbr_x % a.nbr_y;
         kx %= a.nbr_x;
     }
-    round_brick<DIM, PERIM, ACT, EXTRA>(a, b, p, sm, queue, kx, ky, kz);
+    round_brick<DIM, PERIM, ACT, EXTRA, CUBED>(a, b, p, sm, queue, kx, ky, kz);
 }
 
 // One (lattice, brick) item of batch round q: lattice it.x's round number
@@ -320,7 +320,7 @@ unsigned grid_for(uint64_t n, unsigned threads)
     return (unsigned)(g == 0 ? 1 : g);
 }
 
-template <int DIM, bool PERIM, bool ACT, bool EXTRA>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, bool CUBED>
 cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, cudaStream_t st)
 {
     const auto bricks = [](uint32_t n, uint32_t log2) { return (n + (1u << log2) - 1) >> log2; };
@@ -334,7 +334,7 @@ cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, c
     }
     const unsigned threads = 1u << (a.brick_lx + a.brick_ly + (DIM == 3 ? a.brick_lz : 0));
     if (!a.pdl) {
-        round_kernel<DIM, PERIM, ACT, EXTRA><<<blocks, threads, 0, st>>>(a, b, p);
+        round_kernel<DIM, PERIM, ACT, EXTRA, CUBED><<<blocks, threads, 0, st>>>(a, b, p);
         return cudaGetLastError();
     }
     // programmatic dependent launch: the CTAs of this round may start while the
@@ -350,14 +350,18 @@ cudaError_t launch_round_t(RoundArgs a, const RoundBufs &b, const RoundPos &p, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, round_kernel<DIM, PERIM, ACT, EXTRA>, a, b, p);
+    return cudaLaunchKernelEx(&cfg, round_kernel<DIM, PERIM, ACT, EXTRA, CUBED>, a, b, p);
 }
 
 template <int DIM, bool PERIM, bool ACT>
 cudaError_t launch_round_t(const RoundArgs &a, const RoundBufs &b, const RoundPos &p, cudaStream_t st)
 {
-    return b.Sc || a.chem || a.pers_dir ? launch_round_t<DIM, PERIM, ACT, true>(a, b, p, st)
-                                        : launch_round_t<DIM, PERIM, ACT, false>(a, b, p, st);
+    const bool extra = b.Sc || a.chem || a.pers_dir;
+    if (DIM == 3 && a.cubed)
+        return extra ? launch_round_t<DIM, PERIM, ACT, true, DIM == 3>(a, b, p, st)
+                     : launch_round_t<DIM, PERIM, ACT, false, DIM == 3>(a, b, p, st);
+    return extra ? launch_round_t<DIM, PERIM, ACT, true, false>(a, b, p, st)
+                 : launch_round_t<DIM, PERIM, ACT, false, false>(a, b, p, st);
 }
 
 }  // namespace
@@ -511,6 +515,32 @@ cudaError_t launch_compare(const int32_t *V, const int32_t *A, const int32_t *V2
 cudaError_t launch_clamp_stamps(int32_t *lat, uint64_t n, uint32_t t, cudaStream_t st)
 {
     clamp_kernel<<<grid_for(n, 256), 256, 0, st>>>(lat, n, t);
+    return cudaGetLastError();
+}
+
+// Rows to cubes (the layout of cubed_off) or back, 16 bytes a thread.  A warp has a quarter of a cube, a CTA those of
+// eight cubes next to each other along x, so that both sides are read and written in whole lines.
+__global__ void __launch_bounds__(256) cube_kernel(int4 *cubes, int4 *rows, uint32_t nx, uint32_t ny, uint32_t nz, int to_rows)
+{
+    const uint32_t kx = nx / 8, groups = (kx + 7) / 8, ky = ny / 8;
+    const uint32_t quarter = blockIdx.x & 3u;
+    const uint32_t x8 = (blockIdx.x >> 2) % groups * 8 + (threadIdx.x >> 5), y8 = (blockIdx.x >> 2) / groups % ky,
+                   z8 = (blockIdx.x >> 2) / groups / ky;
+    if (x8 >= kx) return;
+    const uint32_t w = quarter * 32 + (threadIdx.x & 31u);  // of the cube's 128 pieces
+    const uint32_t x = x8 * 8 + (w >> 2 & 1u) * 4, y = y8 * 8 + (w & 1u) + (w >> 3 & 3u) * 2,
+                   z = z8 * 8 + (w >> 1 & 1u) + (w >> 5) * 2;
+    const uint64_t cube = (x8 + (uint64_t)kx * (y8 + (uint64_t)ky * z8)) * 128 + w;
+    const uint64_t row = (x + (uint64_t)nx * (y + (uint64_t)ny * z)) / 4;
+    if (to_rows) __stcs(rows + row, __ldcs(cubes + cube));
+    else __stcs(cubes + cube, __ldcs(rows + row));
+}
+
+cudaError_t launch_cubes(int32_t *cubes, int32_t *rows, uint32_t nx, uint32_t ny, uint32_t nz, bool to_rows, cudaStream_t st)
+{
+    const uint64_t blocks = (uint64_t)((nx / 8 + 7) / 8) * (ny / 8) * (nz / 8) * 4;
+    cube_kernel<<<(unsigned)blocks, 256, 0, st>>>(reinterpret_cast<int4 *>(cubes), reinterpret_cast<int4 *>(rows), nx, ny,
+                                                  nz, to_rows ? 1 : 0);
     return cudaGetLastError();
 }
 

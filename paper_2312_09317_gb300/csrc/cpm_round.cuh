@@ -195,14 +195,26 @@ template <int DIM>
 constexpr int kDirShift = DIM == 3 ? 27 : 28;
 
 // Storage offset of a site, and the step in it from coordinate v to v + d (d in -1, 0, 1) on an axis.
+// CUBED (3D, extents multiples of 8): 8 x 8 x 8 cubes of 2 KB one after the other, x fastest, in each 4 x 2 x 2
+// boxes of 64 bytes, so that a window lies in a few boxes of mostly one cube (see cpm_api.cu, run_cubed).
+template <int AXIS>
+__device__ __forceinline__ uint32_t cubed_off(const RoundArgs &a, uint32_t v)
+{
+    if (AXIS == 0) return (v & 3u) | (v & 4u) << 2 | (v >> 3) << 9;
+    if (AXIS == 1) return ((v & 1u) << 2 | (v & 6u) << 4) + (v >> 3) * (64u * a.nx);
+    return ((v & 1u) << 3 | (v & 6u) << 6) + (v >> 3) * (8u * a.nx * a.ny);
+}
+template <bool CUBED>
 __device__ __forceinline__ uint32_t site_off(const RoundArgs &a, uint32_t x, uint32_t y, uint32_t z)
 {
+    if (CUBED) return cubed_off<0>(a, x) + cubed_off<1>(a, y) + cubed_off<2>(a, z);
     return x + a.nx * (y + a.ny * z);
 }
-template <int AXIS>
+template <int AXIS, bool CUBED>
 __device__ __forceinline__ uint32_t axis_step(const RoundArgs &a, uint32_t v, int d)
 {
     const uint32_t to = wrap_step(v, d, AXIS == 0 ? a.nx : (AXIS == 1 ? a.ny : a.nz));
+    if (CUBED) return cubed_off<AXIS>(a, to) - cubed_off<AXIS>(a, v);
     return (to - v) * (AXIS == 0 ? 1u : (AXIS == 1 ? a.nx : a.nx * a.ny));
 }
 
@@ -210,7 +222,7 @@ __device__ __forceinline__ uint32_t axis_step(const RoundArgs &a, uint32_t v, in
 // the eight columns (dx, dy) != (0, 0) are dealt out 8 / G to a lane, and in 3D lanes 0 and 1 also
 // take the sites below and above the centre.  The columns are the lane's for good, so an offset is
 // one addition of a column's and a plane's step, with no division and no shuffle per neighbour.
-template <int DIM, int G>
+template <int DIM, int G, bool CUBED>
 struct Window {
     static constexpr int COLS = 8 / G, K = DIM == 3 ? 3 * COLS + 1 : COLS;
     uint32_t col[COLS], below, above;  // steps of the columns and the planes
@@ -220,10 +232,10 @@ struct Window {
         for (int c = 0; c < COLS; ++c) {
             const uint32_t m = sub + (uint32_t)(G * c), idx = m + (m >= 4 ? 1u : 0u);  // skip the centre column
             const int dy = idx < 3 ? -1 : (idx < 6 ? 0 : 1), dx = (int)idx - 3 * dy - 4;
-            col[c] = axis_step<0>(a, x, dx) + axis_step<1>(a, y, dy);
+            col[c] = axis_step<0, CUBED>(a, x, dx) + axis_step<1, CUBED>(a, y, dy);
         }
-        below = DIM == 3 ? axis_step<2>(a, z, -1) : 0;
-        above = DIM == 3 ? axis_step<2>(a, z, 1) : 0;
+        below = DIM == 3 ? axis_step<2, CUBED>(a, z, -1) : 0;
+        above = DIM == 3 ? axis_step<2, CUBED>(a, z, 1) : 0;
     }
     // whether the lane has a k-th neighbour, and its offset from the centre
     __device__ __forceinline__ static bool has(int k, uint32_t sub) { return DIM == 2 || k < 3 * COLS || sub < 2; }
@@ -249,7 +261,7 @@ __device__ __forceinline__ int32_t group_sum(int32_t v)
 struct Draw {
     uint32_t i_dir, off, src, x, y, z, w2;
 };
-template <int DIM>
+template <int DIM, bool CUBED = false>
 __device__ __forceinline__ Draw round_draw(const RoundArgs &a, const RoundPos &p, uint32_t ix, uint32_t iy, uint32_t iz,
                                            uint32_t i)
 {
@@ -271,9 +283,9 @@ __device__ __forceinline__ Draw round_draw(const RoundArgs &a, const RoundPos &p
     const uint32_t idx = n + (n >= NB / 2 ? 1u : 0u);  // skip the centre of the 3^d stencil
     const int ox = (int)(idx % 3), oy = (int)((idx / 3) % 3), oz = DIM == 3 ? (int)(idx / 9) : 1;
     d.i_dir = i | (idx << kDirShift<DIM>);
-    d.off = site_off(a, d.x, d.y, d.z);
-    d.src = d.off + axis_step<0>(a, d.x, ox - 1) + axis_step<1>(a, d.y, oy - 1) +
-            (DIM == 3 ? axis_step<2>(a, d.z, oz - 1) : 0u);
+    d.off = site_off<CUBED>(a, d.x, d.y, d.z);
+    d.src = d.off + axis_step<0, CUBED>(a, d.x, ox - 1) + axis_step<1, CUBED>(a, d.y, oy - 1) +
+            (DIM == 3 ? axis_step<2, CUBED>(a, d.z, oz - 1) : 0u);
     d.w2 = w.v[2];
     return d;
 }
@@ -291,14 +303,14 @@ __device__ __forceinline__ Draw round_draw(const RoundArgs &a, const RoundPos &p
 // another (registers), and a warp's instructions run for the fifth of its lanes that survived:
 // 82 warp instructions per attempt on the 3D tissue, 10 of 32 lanes active.
 // Measured against that (ms per MCS): 256^3 cube cells 0.911 -> 0.597, 1024^3 fibre tissue
-// 189.2 -> 143.3, 64 uneven lattices of a sweep 5.00 -> 2.90.  Eight lanes per survivor and a queue
+// 189.2 -> 143.3 (in rows), 64 uneven lattices of a sweep 5.00 -> 2.90.  Eight lanes per survivor and a queue
 // per warp: 0.976 and 180.7; two attempts per lane (half the warps): 1.46 and 336.
-template <int DIM, bool PERIM, bool ACT, bool EXTRA, int G>
+template <int DIM, bool PERIM, bool ACT, bool EXTRA, int G, bool CUBED = false>
 __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b, uint32_t t, const SmemTables &sm,
                                           Survivors &q, uint32_t &n_queue, bool valid, const Draw &d,
                                           uint32_t first_warp = 0)
 {
-    using Win = Window<DIM, G>;
+    using Win = Window<DIM, G, CUBED>;
     static_assert(G == 4 || G == 8, "the four tallies take four lanes");
     constexpr int NB = DIM == 3 ? 26 : 8, K = Win::K;
     constexpr uint32_t kIndexMask = (1u << kDirShift<DIM>) - 1u;
@@ -532,7 +544,7 @@ __device__ __forceinline__ void round_cta(const RoundArgs &a, const RoundBufs &b
                 if (__any_sync(0xffffffffu, window)) {
                     const uint32_t xi = wrap_step(s.x, ox - 1, a.nx), yi = wrap_step(s.y, oy - 1, a.ny);
                     const uint32_t zi = DIM == 3 ? wrap_step(s.z, oz - 1, a.nz) : 0;
-                    const uint32_t src = site_off(a, xi, yi, zi);
+                    const uint32_t src = site_off<CUBED>(a, xi, yi, zi);
                     const Win win_i(a, sub, xi, yi, zi);
 #pragma unroll
                     for (int k = 0; k < K; ++k)
