@@ -403,7 +403,7 @@ int run_spans(cpm_handle *h, int64_t n, SpanPos p)
 // Whether a call's rounds run on the lattice in cubes.  A lattice that L2 does not hold is read in windows of
 // 3 x 3 x 3 at random places: nine rows, each its own 64 bytes of a different DRAM page.  In cubes a window is six
 // boxes of 64 bytes of mostly one 2 KB cube: fibre tissue on 1024^3, areas of 16^3, 143 -> 119 ms per MCS with the
-// way there and back (two passes over the lattice, 3 ms), 768^3 77 -> 69, 400^3 42 -> 38.  With areas of 8^3 and
+// way there and back (a pass over the lattice each), 768^3 77 -> 69, 400^3 42 -> 38.  With areas of 8^3 and
 // less, where the windows of neighbouring areas share lines of a row, there is nothing to gain (cubes of 304^3: 3.3
 // and 3.5, 384^3 with areas of 4^3: 2.0 and 2.1).  The call has to make at least half as many attempts as there are
 // sites; a persistence update reads the lattice in rows after every MCS.
@@ -413,13 +413,19 @@ bool in_cubes(cpm_handle *h, int64_t n)
     if (h->cfg.nx % 8 || h->cfg.ny % 8 || h->cfg.nz % 8) return false;
     if ((double)n * h->k * h->n_active < 0.5 * (double)h->n_sites) return false;
     if (h->cubes) return true;
-    // no memory for a second copy, or a stream under capture: in rows
+    // a copy that would take more than a quarter of the free memory, or a stream under capture: in rows
+    const size_t bytes = sizeof(int32_t) * h->n_sites;
+    size_t free_bytes = 0, total = 0;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // another thread's capture is not disturbed
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
     if (cudaStreamIsCapturing(h->stream, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone ||
-        cudaMalloc(&h->cubes, sizeof(int32_t) * h->n_sites) != cudaSuccess) {
+        cudaMemGetInfo(&free_bytes, &total) != cudaSuccess || bytes > free_bytes / 4 ||
+        cudaMalloc(&h->cubes, bytes) != cudaSuccess) {
         cudaGetLastError();
         h->cubes = nullptr;
     }
+    cudaThreadExchangeStreamCaptureMode(&mode);
     return h->cubes != nullptr;
 }
 
