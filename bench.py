@@ -118,7 +118,7 @@ NCU_TRAFFIC = {
 
 def kernel_hash() -> str:
     h = hashlib.sha1()
-    for f in ("cpm_kernels.cu", "cpm_internal.h"):
+    for f in ("cpm_kernels.cu", "cpm_round.cuh", "cpm_internal.h"):
         h.update(open(os.path.join(ROOT, "paper_2312_09317_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 
@@ -773,8 +773,8 @@ def emulator_sweep_measure(args, rank=0, ws_=1, dist=None):
             },
             "roofline": {"bound": "tensor", "achieved": tflops, "peak": pk[0], "unit": "TFLOP/s",
                          "frac": tflops / pk[0], "traffic": None, "peak_kind": "of %s" % pk[1],
-                         "kernel": "gemm_tc_kernel (tcgen05, TMEM accumulators) over the 1M-point prediction: "
-                                   "every forward layer, the gathers and the ensemble/fallback kernel",
+                         "kernel": "fused_forward_kernel (tcgen05, TMEM accumulators) over the 1M-point prediction: "
+                                   "all layers, and the ensemble/fallback kernel",
                          "inference_points_per_s": Xi.shape[0] / inf_s},
             "cpu_baseline": None,
             "e2e": {"value": value, "unit": "points/s", "h2d_bytes_per_step": block * 7 * 4,

@@ -238,7 +238,9 @@ void cpm_destroy(cpm_handle *h);
  * own configuration and seed; after cpm_batch_step(b, n) lattice i is
  * exactly what cpm_step(h_i, n) gives for a handle created from cfgs[i].  A
  * batch step launches one kernel per round for all lattices that still have
- * rounds in the call (lattices with fewer rounds per MCS finish earlier).
+ * rounds in the call (lattices with fewer rounds per MCS finish earlier), or,
+ * where every lattice fits one CTA's shared memory and none is tracked, one
+ * kernel for the call, a CTA per lattice.
  * All configurations of a batch must share dim and use the global schedule
  * (tile = 0).  The library owns all device memory; cfgs is borrowed for the
  * duration of cpm_batch_create. */
@@ -251,11 +253,13 @@ int cpm_batch_create(const cpm_config *cfgs, int32_t n, void *cuda_stream, cpm_b
 /* Advance every lattice by n_mcs MCS (asynchronous on the batch's stream).
  * One MCS of the whole batch is a CUDA graph, captured on first use: the Act
  * stamp clamp, one launch per round over the members that still have
- * rounds, and a device-side advance of every member's MCS counter. */
+ * rounds, and a device-side advance of every member's MCS counter; small
+ * lattices as described above run without one. */
 int cpm_batch_step(cpm_batch *b, int64_t n_mcs);
 
 /* Choose how cpm_batch_step runs the MCS loop.
- *   on = 0 (the default): one CUDA graph per MCS, replayed: the Act clamp,
+ *   on = 0 (the default): one launch per call for small lattices, else one
+ *          CUDA graph per MCS, replayed: the Act clamp,
  *          one kernel per round, and the advance of the members' counters.
  *   on = 1: one persistent, cooperative launch per call runs all n_mcs MCS:
  *          the same phases, separated by grid-wide barriers instead of

@@ -10,11 +10,12 @@
 // runs all members in one launch (grid.z = member), each member reading its
 // own slice of the flat parameter buffer.
 //
-// The forward layers (A [M][K] times W^T, N <= 256, K <= 256) run on the
-// fifth-generation tensor cores (tcgen05.mma into TMEM, gemm_tc_kernel).  The
-// backward GEMMs (transposed operands) use mma.sync m16n8k16 (bf16 x bf16 ->
-// f32) on 64 x 64 CTA tiles with a 32-deep K slab, double-buffered in shared
-// memory.  Bias, GELU and GELU' are fused into the epilogues.
+// Shapes that fused_fits takes run through all layers in one kernel (cpm_mlp_fused.cu for inference,
+// cpm_mlp_train.cu and cpm_mlp_update.cu for a training batch).  The kernels here serve the others, and
+// cpm_mlp_gemm: forward layers (A [M][K] times W^T, N <= 256, K <= 256) on the fifth-generation tensor cores
+// (tcgen05.mma into TMEM, gemm_tc_kernel), the backward GEMMs (transposed operands) on mma.sync m16n8k16
+// (bf16 x bf16 -> f32) on 64 x 64 CTA tiles with a 32-deep K slab, double-buffered in shared memory.  Bias,
+// GELU and GELU' are fused into the epilogues.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
