@@ -84,7 +84,8 @@ __device__ __forceinline__ void span_run(const RoundArgs &a, const LatticeBufs &
     if (valid) d = round_draw<DIM>(a, pos, x0, y0, z0, i0);
     uint32_t par = p.par, stage = 0;
     for (uint32_t left = p.n_sub; left > 0;) {
-        if (ACT && pos.sp == 0 && pos.r == 0 && pos.t % 64 == 0) {
+        // (a batch's kernel has ACT where any member has the term; the words of a member without it are plain ids)
+        if (ACT && a.packed && pos.sp == 0 && pos.r == 0 && pos.t % 64 == 0) {
             const uint32_t n = a.nx * a.ny * a.nz;
             for (uint32_t x = rank * blockDim.x + tid; x < n; x += nc * blockDim.x) clamp_word(l.lat + x, pos.t & 255u);
             arrive();
