@@ -412,7 +412,9 @@ cudaError_t fused_forward(const FusedNet &n, const float *X, int64_t rows, float
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the limit belongs to the kernel, not to the launch: every thread sets the same
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(fused_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFusedSmem);
     if (e != cudaSuccess) return e;
     fused_forward_kernel<<<p.items < sms ? p.items : sms, kThreads, smem, st>>>(p);
     return cudaPeekAtLastError();

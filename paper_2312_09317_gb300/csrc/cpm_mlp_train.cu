@@ -26,6 +26,7 @@ namespace {
 constexpr int kTrainWarps = 16, kTrainThreads = (kTrainWarps + 2) * 32;
 constexpr int kTrainStages = 3, kStage2 = 2 * kStageBytes;  // of the ring: two slabs of a hidden layer
 constexpr int kMaxTile = 128;
+constexpr int kTrainSmem = 224 * 1024;  // of a CTA, at most
 // The activations lie with the rows innermost (MN-major): core matrices of 8 K indices x 8 rows, K-adjacent ones
 // next to each other, so that a lane's 8 rows of an output are one 16-byte store, a warp's contiguous.
 constexpr uint32_t kRowsInner = 1u << 16;  // of the instruction descriptor, for the B operand
@@ -536,10 +537,12 @@ cudaError_t fused_train(const FusedNet &n, const TrainArgs &tr, const float *X, 
     while (p.tile < kMaxTile && (rows + p.tile - 1) / p.tile * n.n_members > sms) p.tile += 16;
     p.mtiles = (int)((rows + p.tile - 1) / p.tile);
     p.items = p.mtiles * n.n_members;
+    // (212,096 bytes for the largest shape that fused_fits takes: 32 inputs and outputs, 15 layers of 256, tiles of 128)
     const int smem = kTrainStages * kStage2 + p.tile * (n.width + n.n_out + p.k0p) * 2 + p.tile * n.n_out * 4 +
                4 * (n.n_hidden * n.width + n.n_out);
     const auto kernel = n.width > kRows ? fused_train_kernel<2> : fused_train_kernel<1>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the limit belongs to the kernel, not to the launch: every thread sets the same
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem);
     if (e != cudaSuccess) return e;
     return pdl_launch(kernel, p, p.items < sms ? p.items : sms, kTrainThreads, smem, tr.chained, st);
 }

@@ -314,6 +314,10 @@ __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
 constexpr int kSumThreads = 128, kSumWarps = kSumThreads / 32;
 constexpr int kMaxLag = 20;  // step-direction autocorrelation lags (x every MCS)
 constexpr size_t kSumUnitBytes = 48 * 1024;  // step directions held at a time (at least one cell's)
+// dynamic shared memory of a summary of the most snapshots
+constexpr size_t kSumMaxSmem = sizeof(double) * (5 + 3 * kSumWarps) * kSummaryMaxSnap + kSumUnitBytes;
+static_assert(sizeof(double) * 2 * kSummaryMaxSnap <= kSumUnitBytes && sizeof(double) * 2 * kSumWarps * kMaxLag <= kSumUnitBytes,
+              "a cell's directions and the lags' totals fit");
 // scalar accumulators of one lattice, a copy per warp
 enum {
     A_MSD = 0,       // 3 sums, then 3 counts
@@ -718,7 +722,8 @@ cudaError_t launch_summarize(const ObserveItem *d_items, uint32_t n_items, int32
     size_t units = cap * per_cell;
     if (units < sizeof(double) * 2 * kSumWarps * kMaxLag) units = sizeof(double) * 2 * kSumWarps * kMaxLag;
     const size_t smem = sizeof(double) * (5 + 3 * kSumWarps) * (size_t)n_snap + units;
-    const cudaError_t e = cudaFuncSetAttribute(summarize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit belongs to the kernel, not to the launch: every thread sets the same
+    const cudaError_t e = cudaFuncSetAttribute(summarize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSumMaxSmem);
     if (e != cudaSuccess) return e;
     summarize_kernel<<<n_items, kSumThreads, smem, st>>>(d_items, cells, rows, member, (int)n_items, n_snap, every,
                                                          (int)cap, out);
