@@ -1120,6 +1120,7 @@ struct cpm_batch {
     uint32_t loop_grid = 0;              // CTAs of the last persistent launch
     bool track = false;                  // composite variable tracking in every member
     bool motile = false;                 // a member has a field or persistence directions
+    bool tuning = false;                 // cpm_batch_autotune is timing the graph
     uint32_t span_threads = 0;           // threads of a CTA there
     uint32_t span_smem = 0;              // shared memory per CTA where every member runs in one CTA, else 0
     bool descriptors_dirty = true;
@@ -1443,7 +1444,7 @@ int cpm_batch_step(cpm_batch *b, int64_t n_mcs)
                              "state");
             done += chunk;
         }
-    } else if (b->span_smem && !b->track) {
+    } else if (b->span_smem && !b->track && !b->tuning) {
         for (int64_t done = 0; done < n_mcs;) {
             const uint32_t m = (uint32_t)std::min<int64_t>(n_mcs - done, 256);
             const uint32_t n = (uint32_t)b->lats.size();
@@ -1531,6 +1532,7 @@ int cpm_batch_autotune(cpm_batch *b, int32_t n_mcs_each, int32_t *choice)
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     int rc = CPM_OK;
+    b->tuning = true;  // the bricks shape the launches per round, also of a batch whose steps need none now
     // passes interleave the candidates, so that each is timed on a similar
     // spread of simulation states (the cost of an MCS drifts as cells grow)
     for (int pass = 0; pass < 1 + n_mcs_each && rc == CPM_OK; pass++) {
@@ -1551,6 +1553,7 @@ int cpm_batch_autotune(cpm_batch *b, int32_t n_mcs_each, int32_t *choice)
             if (pass > 0) total[k] += ms;
         }
     }
+    b->tuning = false;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (rc) return rc;
