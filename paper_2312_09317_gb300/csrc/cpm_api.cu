@@ -377,8 +377,8 @@ int run_spans(cpm_handle *h, int64_t n, SpanPos p)
     RoundArgs args = round_args(h);
     if (p.resident) args.stream_loads = 0;  // its words are in shared memory
     while (n > 0) {
-        // up to the end of the MCS where something follows it, and some tens of milliseconds per launch at most
-        int64_t m = std::min<int64_t>(n, std::max<int64_t>(1, 32768 / (int64_t)h->k));
+        // up to the end of the MCS where something follows it
+        int64_t m = std::min<int64_t>(n, std::max<uint32_t>(1, kSpanRounds / h->k));
         if (h->csum || h->pers) m = std::min<int64_t>(m, (int64_t)h->per_mcs - h->sp);
         p.t = (uint32_t)h->t;
         p.sp = (uint32_t)h->sp;
@@ -1445,8 +1445,9 @@ int cpm_batch_step(cpm_batch *b, int64_t n_mcs)
             done += chunk;
         }
     } else if (b->span_smem && !b->track && !b->tuning) {
+        const uint32_t most = std::max<uint32_t>(1, kSpanRounds / b->lats[b->order[0]].R);  // of the longest member
         for (int64_t done = 0; done < n_mcs;) {
-            const uint32_t m = (uint32_t)std::min<int64_t>(n_mcs - done, 256);
+            const uint32_t m = (uint32_t)std::min<int64_t>(n_mcs - done, most);
             const uint32_t n = (uint32_t)b->lats.size();
             cudaError_t e = b->dim == 3
                                 ? launch_batch_span_3d(b->perim, b->act, b->motile, b->d_lats, n, m, b->span_threads,

@@ -200,6 +200,8 @@ __host__ __device__ __forceinline__ RoundBufs round_bufs(const LatticeBufs &l, u
 // A span of rounds of one lattice in one launch (cpm_span.cuh).
 constexpr uint32_t kSpanThreads = 512;         // most threads of a CTA
 constexpr uint32_t kSpanMaxSmem = 200 * 1024;  // most dynamic shared memory (a resident lattice)
+constexpr uint32_t kSpanRounds = 32768;        // most rounds of a launch (40 to 190 ms at 1.3 to 5.8 us), or one
+                                               // sub-pass (a batch: one MCS) where that has more
 struct SpanPos {
     uint32_t t, sp;            // MCS (low 32 bits) and sub-pass of the first round
     uint32_t per_mcs, C, k;    // sub-passes per MCS, colours, rounds per sub-pass
