@@ -250,7 +250,8 @@ int ensure_stage(cpm_handle *h)
 // (and at creation): observe the lattice, record the centroids, update p_hat.
 int pers_step(cpm_handle *h)
 {
-    CUDA_TRY(h, launch_observe(h->dim, h->pers_item, 1, (int64_t)h->n_sites, h->pers_cells, h->pers_member,
+    CUDA_TRY(h, launch_observe(h->dim, h->pers_item, 1, (int64_t)h->n_sites,
+                               (uint32_t)(h->dim == 3 ? h->cfg.nz : h->cfg.ny), h->pers_cells, h->pers_member,
                                h->stream));
     CUDA_TRY(h, launch_pers_update(h->pers_cells, h->n_cells, (uint32_t)h->cfg.nx, (uint32_t)h->cfg.ny,
                                    (uint32_t)h->cfg.nz, h->cell_type, h->pp, h->pers_hist, h->pers_H, h->t,
@@ -1103,6 +1104,7 @@ struct cpm_batch {
     ObserveItem *d_obs = nullptr;        // observation items, built on first use
     TableCache *tables = nullptr;        // LN / EXPQ / THR shared by the members
     int64_t obs_max_sites = 0;
+    uint32_t obs_longest = 0;            // extent of the slowest axis
     int64_t obs_rows = 0;
     int32_t obs_max_cells = 0;
     uint8_t *d_colours = nullptr;        // BatchLattice::colours of every member
@@ -1649,6 +1651,7 @@ int batch_obs_items(cpm_batch *b)
             row += (int64_t)h->n_cells + 1;
             b->obs_max_sites = std::max<int64_t>(b->obs_max_sites, (int64_t)h->n_sites);
             b->obs_max_cells = std::max<int32_t>(b->obs_max_cells, h->n_cells);
+            b->obs_longest = std::max<uint32_t>(b->obs_longest, h->dim == 3 ? it.nz : it.ny);
         }
         b->obs_rows = row;
         cudaError_t e = cudaMalloc(&b->d_obs, sizeof(ObserveItem) * items.size());
@@ -1671,8 +1674,8 @@ int cpm_batch_observe(cpm_batch *b, int64_t *cells_out, int64_t *member_out)
     if (!b) return CPM_E_HANDLE;
     if (!cells_out || !member_out) return bfail(b, CPM_E_INVALID, "cells_out and member_out are required");
     if (int rc = batch_obs_items(b)) return rc;
-    cudaError_t e = launch_observe(b->dim, b->d_obs, (uint32_t)b->hs.size(), b->obs_max_sites, cells_out, member_out,
-                                   b->stream);
+    cudaError_t e = launch_observe(b->dim, b->d_obs, (uint32_t)b->hs.size(), b->obs_max_sites, b->obs_longest,
+                                   cells_out, member_out, b->stream);
     if (e != cudaSuccess) return bfail(b, CPM_E_CUDA, cudaGetErrorString(e));
     b->launches += 3;
     return CPM_OK;

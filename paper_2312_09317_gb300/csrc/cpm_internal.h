@@ -281,8 +281,9 @@ struct ObserveItem {
     int32_t n_cells, pad_;
     double v_ref, a_ref;  // V_t and A_t of cell 1's type: the scale of the volume / interface statistics
 };
-cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items, int64_t max_sites, int64_t *cells,
-                           int64_t *member, cudaStream_t st);
+// max_sites, longest: of the largest lattice, and the largest extent of the slowest axis
+cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items, int64_t max_sites, uint32_t longest,
+                           int64_t *cells, int64_t *member, cudaStream_t st);
 
 // Persistence update at the end of an MCS (Eq. 6, Eq. 7) from one observation of the lattice.
 struct PersParams {

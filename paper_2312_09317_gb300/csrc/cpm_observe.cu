@@ -121,7 +121,9 @@ __device__ __forceinline__ uint32_t quotient_of(uint32_t a, Inverse i)
 // walks; 1,024 runs of 64^2 sites 148 and 62 us.
 constexpr int kObsSlots = 128;      // cells whose sums a CTA holds
 constexpr int kSharedExtent = 1024; // the 32-bit sums of 4,096 sites hold offsets of lattices up to this extent
-template <int DIM>
+constexpr int kFarOffset = 11585;   // a run's 32-bit sum holds the squares of kWalk offsets up to this one
+// FAR: some lattice has larger offsets along the walk (a variant of its own: the test of every offset costs 4%)
+template <int DIM, bool FAR>
 __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
     observe_sums_kernel(const ObserveItem *items, int64_t *cells, int64_t *member)
 {
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
         };
         Run run{}, ended{};  // at hand, and one that has ended (3D)
         int aw = 0;          // anchor's coordinate along the walk
-        const auto add_run = [&](const Run &r) {
+        const auto add_run = [&](const Run &r, int64_t sww) {
             unsigned long long *row = reinterpret_cast<unsigned long long *>(cells + (it.row0 + r.id) * kObsFields);
             const auto add = [&](int f, int64_t v) { atomicAdd(row + f, (unsigned long long)v); };
             const int64_t c = r.cnt;
@@ -179,13 +181,13 @@ __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
                 add(3, c * r.oy);
                 add(4, r.sw);
                 add(7, c * r.oy * r.oy);
-                add(8, r.sww);
+                add(8, sww);
                 add(9, c * r.ox * r.oy);
                 add(10, (int64_t)r.sw * r.ox);
                 add(11, (int64_t)r.sw * r.oy);
             } else {
                 add(3, r.sw);
-                add(7, r.sww);
+                add(7, sww);
                 add(9, (int64_t)r.sw * r.ox);
             }
         };
@@ -236,7 +238,7 @@ __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
         };
         const auto end_run = [&](bool ends) {
             if (!shared) {
-                if (ends) add_run(run);
+                if (ends) add_run(run, run.sww);
                 return;
             }
             if (__any_sync(0xffffffffu, ends && ended.id > 0)) flush();
@@ -274,12 +276,18 @@ __global__ void __launch_bounds__(kObsThreads, DIM == 3 ? 3 : 4)
             }
             if (run.id > 0) {
                 const int same_next = equal(next);
-                run.iface += 3 * P - (same_prev + same_cur + same_next);
+                const int iface = 3 * P - (same_prev + same_cur + same_next);
                 medium += zero_prev + zero_cur + zero_next;
                 const int ow = min_image((int)z - aw, nw);
-                ++run.cnt;
-                run.sw += ow;
-                run.sww += ow * ow;
+                if (FAR && (ow > kFarOffset || ow < -kFarOffset)) {
+                    // a run of its own, its square in 64 bits
+                    add_run(Run{run.id, run.ox, run.oy, 1, ow, 0, iface}, (int64_t)ow * ow);
+                } else {
+                    ++run.cnt;
+                    run.iface += iface;
+                    run.sw += ow;
+                    run.sww += ow * ow;
+                }
                 same_prev = same_cur;
                 same_cur = same_next;
             }
@@ -730,8 +738,8 @@ cudaError_t launch_summarize(const ObserveItem *d_items, uint32_t n_items, int32
     return cudaPeekAtLastError();
 }
 
-cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items, int64_t max_sites, int64_t *cells,
-                           int64_t *member, cudaStream_t st)
+cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items, int64_t max_sites, uint32_t longest,
+                           int64_t *cells, int64_t *member, cudaStream_t st)
 {
     if (n_items == 0) return cudaSuccess;
     if (n_items > 65535u) return cudaErrorInvalidValue;
@@ -741,12 +749,15 @@ cudaError_t launch_observe(int dim, const ObserveItem *d_items, uint32_t n_items
     const int64_t most = 152 * 16 / (int64_t)n_items + 16;
     if (bx > most) bx = most;
     const dim3 grid((unsigned)bx, n_items);
+    const bool far = longest / 2 > (uint32_t)kFarOffset;
     if (dim == 3) {
         observe_anchor_kernel<3><<<grid, kObsThreads, 0, st>>>(d_items, cells);
-        observe_sums_kernel<3><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+        if (far) observe_sums_kernel<3, true><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+        else observe_sums_kernel<3, false><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
     } else {
         observe_anchor_kernel<2><<<grid, kObsThreads, 0, st>>>(d_items, cells);
-        observe_sums_kernel<2><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+        if (far) observe_sums_kernel<2, true><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
+        else observe_sums_kernel<2, false><<<grid, kObsThreads, 0, st>>>(d_items, cells, member);
     }
     return cudaPeekAtLastError();
 }
