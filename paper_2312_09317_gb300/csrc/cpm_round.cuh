@@ -51,15 +51,17 @@ __device__ __forceinline__ void load_tables(SmemTables &sm, const RoundArgs &a, 
             r.cvj = lv * (1 + 2 * vt);
             r.lp = a.tp.lambda_p[k];
             r.at2 = (int32_t)(2u * (uint32_t)a.tp.a_target[k]);
-            r.la = a.tp.lambda_act[k];
-            r.ma = a.tp.max_act[k];
-            r.act_lo = (int32_t)a.tp.act_lo[k];
-            r.gm_max = a.tp.gm_max[k];
-            // M = ceil(2^(30+l) / Max) <= 2^31 with 2^l >= Max: the error u (M Max - 2^(30+l)) stays below 2^(30+l)
-            uint32_t l = 0;
-            while ((1 << l) < r.ma) ++l;
-            r.div_s = 30 + l;
-            r.div_m = r.ma > 0 ? (uint32_t)(((1ull << r.div_s) + r.ma - 1) / (uint32_t)r.ma) : 0u;
+            if (with_act) {  // (Max_act in 0 .. 127: without Act it is any number, which nothing reads)
+                r.la = a.tp.lambda_act[k];
+                r.ma = a.tp.max_act[k];
+                r.act_lo = (int32_t)a.tp.act_lo[k];
+                r.gm_max = a.tp.gm_max[k];
+                // M = ceil(2^(30+l) / Max) <= 2^31 with 2^l >= Max: the error u (M Max - 2^(30+l)) stays below 2^(30+l)
+                uint32_t l = 0;
+                while ((1 << l) < r.ma) ++l;
+                r.div_s = 30 + l;
+                r.div_m = r.ma > 0 ? (uint32_t)(((1ull << r.div_s) + r.ma - 1) / (uint32_t)r.ma) : 0u;
+            }
         }
         sm.row[k] = r;
     }
