@@ -352,10 +352,15 @@ int run_subpass(cpm_handle *h)
     return CPM_OK;
 }
 
-// Whether a lattice's rounds run as spans, and how: at most 16 x 256 attempts per round, one each per
-// thread of the largest cluster (with two each a launch per round is faster: 320^2 points 5.1 against 3.3
-// us per round, 3D tissue of 320^3 11.7 against 10.3).
-bool pick_span(const cpm_handle *h, SpanPos &p)
+// Whether the rounds of a call of n schedule units run as spans, and how: at most 16 x 256 attempts per round, one
+// each per thread of the largest cluster (with two each a launch per round is faster: 320^2 points 5.1 against 3.3
+// us per round, 3D tissue of 320^3 11.7 against 10.3), and rounds enough in a launch to repay what it costs before
+// and after them.  That is the launch itself, some 6 us at 1 us or so a round, and for a resident lattice its way into
+// shared memory and back, about bytes / (20 threads) us: 200^2 points on areas of 40^2, us of a call of 1 / 16 / 64 /
+// 1,600 rounds as a span 121 / 135 / 194 / 1,950, with a launch each 2.8 / 34 / 130 / 3,130; Act cells of 64^2 on
+// areas of 16^2 21 / 45 / 122 / - and 2.9 / 39 / 156 / -; 3D Act cells of 64^3 on a cluster 10 / 51 / 181 / - and
+// 4.2 / 62 / 247 / -.
+bool pick_span(const cpm_handle *h, int64_t n, SpanPos &p)
 {
     if (h->n_active > 4096u) return false;
     p.per_mcs = h->per_mcs;
@@ -369,7 +374,9 @@ bool pick_span(const cpm_handle *h, SpanPos &p)
     p.resident = p.nc == 1 && fits ? (uint32_t)resident : 0;
     p.lanes = ((h->n_active + p.nc - 1) / p.nc + 31) / 32 * 32;
     p.threads = std::min(2 * p.lanes, kSpanThreads);
-    return true;
+    // rounds of a launch (run_spans)
+    const double rounds = (double)h->k * (double)(h->csum || h->pers ? std::min<int64_t>(n, h->per_mcs) : n);
+    return rounds >= 8.0 + p.resident / (20.0 * p.threads);
 }
 
 // n schedule units of the global schedule on a lattice that runs as spans
@@ -849,7 +856,7 @@ int cpm_step_subpasses(cpm_handle *h, int64_t n)
     if (bad(h)) return CPM_E_HANDLE;
     if (n < 0) return fail(h, CPM_E_INVALID, "n must be >= 0");
     SpanPos span{};
-    if (!h->tile && pick_span(h, span)) return run_spans(h, n, span);
+    if (!h->tile && pick_span(h, n, span)) return run_spans(h, n, span);
     const bool cubed = in_cubes(h, n);
     if (cubed)
         if (int rc = swap_cubes(h)) return rc;
