@@ -156,6 +156,13 @@ int cpm_step(cpm_handle *h, int64_t n_mcs);
  * (global) or (h, m * P_T * 2^d) (tiled).  Used for finer-grained checks. */
 int cpm_step_subpasses(cpm_handle *h, int64_t n);
 
+/* Bound the CTAs of the thread-block cluster that runs the rounds of a small
+ * lattice (at most 4,096 active blocks), 1..16; 16 at first.  The GPU's own
+ * bound, for the share of it that the process has, holds in any case; where
+ * the cluster cannot hold a round's attempts, rounds are launched one by one.
+ * Results do not depend on it. */
+int cpm_limit_cluster(cpm_handle *h, int32_t ctas);
+
 /* Copy the lattice (nx*ny*nz int32) to dst (host if dst_is_device == 0,
  * device otherwise).  Synchronises the handle's stream. */
 int cpm_read_lattice(cpm_handle *h, int32_t *dst, int dst_is_device);

@@ -64,6 +64,7 @@ _SIGNATURES = {
     "cpm_create": (ctypes.c_int, [ctypes.POINTER(Config), ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p)]),
     "cpm_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64]),
     "cpm_step_subpasses": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int64]),
+    "cpm_limit_cluster": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32]),
     "cpm_read_lattice": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]),
     "cpm_read_tallies": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]),
     "cpm_read_act": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]),
@@ -240,6 +241,10 @@ class Sim:
 
     def step_subpasses(self, n: int):
         self._check(self.lib.cpm_step_subpasses(self.h, n))
+
+    def limit_cluster(self, ctas: int):
+        """Bound the CTAs of the cluster that runs a small lattice's rounds (cpm_limit_cluster)."""
+        self._check(self.lib.cpm_limit_cluster(self.h, ctas))
 
     def read_lattice(self, out=None):
         if out is None:

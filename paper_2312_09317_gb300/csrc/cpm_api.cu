@@ -35,6 +35,8 @@ struct cpm_handle {
     int32_t *tallies = nullptr;  // V0, A0, V1, A1, Vtmp, Atmp; each n_cells + 1
     int32_t *cubes = nullptr;    // the lattice in cubes during a call (run_cubed), kept from the first such call
     bool cubed = false;          // lat and cubes have changed places: lat lies in cubes
+    uint32_t span_ctas[2] = {0, 0};  // the largest cluster of the span kernel without and with EXTRA, 0: not asked yet
+    uint32_t cluster_limit = 16;     // cpm_limit_cluster
     int4 *pend = nullptr;        // two buffers of n_active
     uint8_t *flags = nullptr;    // two buffers of n_active: pend entry valid
     uint32_t *thr = nullptr;
@@ -360,7 +362,7 @@ int run_subpass(cpm_handle *h)
 // 1,600 rounds as a span 121 / 135 / 194 / 1,950, with a launch each 2.8 / 34 / 130 / 3,130; Act cells of 64^2 on
 // areas of 16^2 21 / 45 / 122 / - and 2.9 / 39 / 156 / -; 3D Act cells of 64^3 on a cluster 10 / 51 / 181 / - and
 // 4.2 / 62 / 247 / -.
-bool pick_span(const cpm_handle *h, int64_t n, SpanPos &p)
+bool pick_span(cpm_handle *h, int64_t n, SpanPos &p)
 {
     if (h->n_active > 4096u) return false;
     p.per_mcs = h->per_mcs;
@@ -369,8 +371,13 @@ bool pick_span(const cpm_handle *h, int64_t n, SpanPos &p)
     p.n_cells = h->n_cells;
     const uint64_t resident = span_bytes(h->n_sites, h->n_cells, h->n_active);
     const bool fits = resident <= kSpanMaxSmem;
+    const bool extra = h->csum || h->chem || h->pers;
+    uint32_t &most = h->span_ctas[extra ? 1 : 0];
+    if (most == 0)
+        most = h->dim == 3 ? span_cluster_3d(h->perim, h->act, extra) : span_cluster_2d(h->perim, h->act, extra);
     p.nc = 1;
-    while (p.nc < 16 && h->n_active > (fits ? 128u : 32u) * p.nc) p.nc *= 2;
+    while (2 * p.nc <= std::min(most, h->cluster_limit) && h->n_active > (fits ? 128u : 32u) * p.nc) p.nc *= 2;
+    if (h->n_active > kSpanThreads / 2 * p.nc) return false;  // more than an attempt per thread
     p.resident = p.nc == 1 && fits ? (uint32_t)resident : 0;
     p.lanes = ((h->n_active + p.nc - 1) / p.nc + 31) / 32 * 32;
     p.threads = std::min(2 * p.lanes, kSpanThreads);
@@ -867,6 +874,14 @@ int cpm_step_subpasses(cpm_handle *h, int64_t n)
         if (!rc) rc = back;
     }
     return rc;
+}
+
+int cpm_limit_cluster(cpm_handle *h, int32_t ctas)
+{
+    if (bad(h)) return CPM_E_HANDLE;
+    if (ctas < 1 || ctas > 16) return fail(h, CPM_E_INVALID, "ctas must be in 1..16");
+    h->cluster_limit = (uint32_t)ctas;
+    return CPM_OK;
 }
 
 int cpm_step(cpm_handle *h, int64_t n_mcs)

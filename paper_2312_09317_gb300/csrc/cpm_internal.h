@@ -217,6 +217,10 @@ inline uint64_t span_bytes(uint64_t n_sites, int32_t n_cells, uint32_t n_active)
 {
     return (4 * n_sites + 16 * ((uint64_t)n_cells + 1) + 2 * (uint64_t)n_active + 15) / 16 * 16;
 }
+// CTAs of the largest cluster, 16 at most, that the kernel of such a lattice can be launched with (extra: tracked
+// centroids, a field or persistence directions); 1 where no cluster can be placed
+uint32_t span_cluster_2d(bool perim, bool act, bool extra);
+uint32_t span_cluster_3d(bool perim, bool act, bool extra);
 cudaError_t launch_span_2d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,
                            cudaStream_t st);
 cudaError_t launch_span_3d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,

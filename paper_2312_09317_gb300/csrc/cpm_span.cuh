@@ -208,25 +208,53 @@ __global__ void __launch_bounds__(kSpanThreads, 1) span_kernel(const RoundArgs a
 }
 
 template <int DIM, bool PERIM, bool ACT, bool EXTRA>
-cudaError_t launch_span_t(const RoundArgs &a, const LatticeBufs &l, SpanPos p, cudaStream_t st)
+cudaError_t span_limits()
 {
     auto kern = span_kernel<DIM, PERIM, ACT, EXTRA>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanMaxSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpanMaxSmem);
+    return e == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : e;
+}
+
+inline void span_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &attr, uint32_t nc, uint32_t threads)
+{
+    cfg.gridDim = dim3(nc);
+    cfg.blockDim = dim3(threads);
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = nc;
+    attr.val.clusterDim.y = 1;
+    attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+}
+
+// A cluster's CTAs share one of the GPU's SM groups; whether one has room for 16 is the GPU's affair, or that of the
+// share of it that the process has.
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
+uint32_t span_cluster_t()
+{
+    uint32_t nc = span_limits<DIM, PERIM, ACT, EXTRA>() == cudaSuccess ? 16 : 1;
+    for (; nc > 1; nc /= 2) {
+        cudaLaunchConfig_t cfg = {};
+        cudaLaunchAttribute attr = {};
+        span_config(cfg, attr, nc, kSpanThreads);
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, span_kernel<DIM, PERIM, ACT, EXTRA>, &cfg) == cudaSuccess && n > 0) break;
+    }
+    if (nc < 16) cudaGetLastError();  // a refusal is an answer
+    return nc;
+}
+
+template <int DIM, bool PERIM, bool ACT, bool EXTRA>
+cudaError_t launch_span_t(const RoundArgs &a, const LatticeBufs &l, SpanPos p, cudaStream_t st)
+{
+    const cudaError_t e = span_limits<DIM, PERIM, ACT, EXTRA>();
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(p.nc);
-    cfg.blockDim = dim3(p.threads);
+    cudaLaunchAttribute attr = {};
+    span_config(cfg, attr, p.nc, p.threads);
     cfg.dynamicSmemBytes = p.resident;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = p.nc;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, a, l, p);
+    return cudaLaunchKernelEx(&cfg, span_kernel<DIM, PERIM, ACT, EXTRA>, a, l, p);
 }
 
 // Members of a batch, a CTA each, n_mcs MCS of every member; the lattices are resident in shared memory.
@@ -292,6 +320,15 @@ cudaError_t launch_batch_span_d(bool perim, bool act, bool motile, BatchLattice 
 #define CPM_SPAN(PE, AC)                                                                     \
     (motile ? launch_batch_span_t<DIM, PE, AC, true>(lats, n, n_mcs, threads, smem, st)      \
             : launch_batch_span_t<DIM, PE, AC, false>(lats, n, n_mcs, threads, smem, st))
+    if (act) return perim ? CPM_SPAN(true, true) : CPM_SPAN(false, true);
+    return perim ? CPM_SPAN(true, false) : CPM_SPAN(false, false);
+#undef CPM_SPAN
+}
+
+template <int DIM>
+uint32_t span_cluster_d(bool perim, bool act, bool extra)
+{
+#define CPM_SPAN(PE, AC) (extra ? span_cluster_t<DIM, PE, AC, true>() : span_cluster_t<DIM, PE, AC, false>())
     if (act) return perim ? CPM_SPAN(true, true) : CPM_SPAN(false, true);
     return perim ? CPM_SPAN(true, false) : CPM_SPAN(false, false);
 #undef CPM_SPAN

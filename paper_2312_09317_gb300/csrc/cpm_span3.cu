@@ -3,6 +3,8 @@
 
 namespace cpmgb {
 
+uint32_t span_cluster_3d(bool perim, bool act, bool extra) { return span_cluster_d<3>(perim, act, extra); }
+
 cudaError_t launch_span_3d(bool perim, bool act, const RoundArgs &a, const LatticeBufs &l, const SpanPos &p,
                            cudaStream_t st)
 {
