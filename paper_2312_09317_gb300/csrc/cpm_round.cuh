@@ -114,9 +114,12 @@ __device__ __noinline__ int64_t floor_div_pos(int64_t num, int64_t den)
     return q;
 }
 
-// Energies in 64 bits, for any parameters; and in 32 bits with weights that RoundArgs::narrow admits,
-// where a sum is clamped to +-2^30 once: the Act term that follows is at most 16 lambda_Act < 2^23, and
-// every threshold lies below 2^22, so a clamped sum is decided as the sum itself.
+// Energies in 64 bits, for any parameters; and in 32 bits with weights that RoundArgs::narrow admits, where a sum is
+// clamped to +-2^30 once before the Act term is added.  With lambda_Act < 2^19 that term is at least -16 lambda_Act >
+// -2^23 (the gaining cell's mean over its own Max_act) and at most 16 lambda_Act Max_j / Max_i, so with Max_act 1 and
+// 127 at most 2032 lambda_Act <= 2^30 - 2^23 - 2032: no sum reaches 2^31, one clamped from above stays above 2^30 - 2^23
+// and so above every threshold (below 2^22), and one clamped from below stays below 0, as the sums themselves do.
+static_assert(16ll * 127 * ((1 << 19) - 1) < (1 << 30) - (1 << 23), "the Act term stays clear of a clamped sum");
 struct Wide {
     using E = int64_t;
     __device__ __forceinline__ static E energy(int64_t h) { return h; }
