@@ -96,7 +96,7 @@ __device__ __forceinline__ float gelu_f(float z)
 }
 
 // Two GELUs at a time in packed FP32 (Blackwell's f32x2 instructions, half the issue slots).  The value is that of
-// gelu_f, operation by operation, so that each result has its bits for |z| <= kGelu2Max (checked over all floats of
+// gelu_f, operation by operation, so that each result has its bits for |z| <= kGelu2Max (the tests compare all floats of
 // that range); there exp(-z^2 / 2) is a normal number, so that exp2 and the reciprocal need none of the scaling that
 // a subnormal result or a huge argument would.  The sign enters by two multiplications instead of a comparison and a
 // selection: Phi = b - sigma h with (b, sigma) = (1, 1) for z >= 0 and (0, -1) below, exactly.
