@@ -148,7 +148,13 @@ typedef struct cpm_handle cpm_handle;
 int cpm_create(const cpm_config *cfg, void *cuda_stream, cpm_handle **out);
 
 /* Run n_mcs Monte Carlo steps (n_mcs * P * c^d sub-passes).  Asynchronous on
- * the handle's stream.  n_mcs >= 0. */
+ * the handle's stream.  n_mcs >= 0.
+ * On a large 3D lattice (more than 80 MB of sites, areas of edge 16 or more,
+ * extents that are multiples of 8, no persistence term) the first call of half
+ * an MCS or more allocates a second copy of it (4 bytes per site, 4 GiB at
+ * 1024^3), in which such calls run; the handle keeps it until cpm_destroy.
+ * Where it would take more than a quarter of the device memory then free, or
+ * the stream is under capture, the call runs without. */
 int cpm_step(cpm_handle *h, int64_t n_mcs);
 
 /* Run n schedule units: sub-passes (colour visits) of the global schedule,
