@@ -380,17 +380,17 @@ __device__ __forceinline__ void tc_stage(unsigned char *S, const __nv_bfloat16 *
 }
 
 // As tc_stage for 16-byte aligned rows with K a multiple of 8, issued as
-// cp.async copies (rows past `rows` are zero-filled without reading);
+// cp.async copies (rows past `rows` and columns past K are zero-filled without reading);
 // completion: cp.async.wait_all, then fence.proxy.async before the MMAs read.
-__device__ __forceinline__ void tc_stage_async(unsigned char *S, const __nv_bfloat16 *X, int64_t ld, int rows, int r0,
-                                               int rows_tile, int Kp)
+__device__ __forceinline__ void tc_stage_async(unsigned char *S, const __nv_bfloat16 *X, int64_t ld, int rows, int K,
+                                               int r0, int rows_tile, int Kp)
 {
     const int kc = Kp / 8;
     const int n = rows_tile * kc;
     for (int e = threadIdx.x; e < n; e += blockDim.x) {
         const int rr = e & 7, k8 = (e >> 3) % kc, r8 = (e >> 3) / kc;
         const int gr = r0 + r8 * 8 + rr;
-        const bool in = gr < rows;
+        const bool in = gr < rows && k8 * 8 < K;
         const __nv_bfloat16 *src = X + (in ? (int64_t)gr * ld + k8 * 8 : 0);
         const unsigned dst = (unsigned)__cvta_generic_to_shared(S + (size_t)e * 16);
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst), "l"(src), "r"(in ? 16 : 0)
@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const TcArgs p)
     if (t0 < t1) {
         const int z = t0 / p.mtiles, m0 = (t0 % p.mtiles) * kTcM;
         if (async_a) {
-            tc_stage_async(As, p.A + z * p.sa, p.lda, p.M, m0, kTcM, p.Kp);
+            tc_stage_async(As, p.A + z * p.sa, p.lda, p.M, p.K, m0, kTcM, p.Kp);
             asm volatile("cp.async.wait_all;\n" ::: "memory");
         } else {
             tc_stage(As, p.A + z * p.sa, p.lda, p.M, p.K, m0, kTcM, p.Kp, p.vec_a);
@@ -478,7 +478,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const TcArgs p)
         if (next) {
             z1 = (t + 1) / p.mtiles;
             m1 = ((t + 1) % p.mtiles) * kTcM;
-            if (async_a) tc_stage_async(As, p.A + z1 * p.sa, p.lda, p.M, m1, kTcM, p.Kp);
+            if (async_a) tc_stage_async(As, p.A + z1 * p.sa, p.lda, p.M, p.K, m1, kTcM, p.Kp);
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const int row = m0 + q * 32 + lane;
