@@ -107,18 +107,18 @@ BURN_IN = {"cpm2d_200": 50, "cpm3d_256": 50, "cpm3d_512": 50, "cpm3d_tissue_1024
 DEFAULT_WORKLOAD = "cpm3d_tissue_1024"
 
 # DRAM bytes per round-kernel launch from the last ncu capture, valid only for
-# the kernel source and launch shapes it was taken on (sha1 of csrc/cpm_kernels.cu
-# followed by csrc/cpm_internal.h, first 12 hex).  A single-pass capture
-# (dram__bytes_read/write.sum) of one launch at full size, after the growth
-# burn-in and the warm-up.
+# the sources of the kernel and of what chooses it that it was taken on (kernel_hash).
+# A single-pass capture (dram__bytes_read/write.sum) of one launch at full size, the lattice
+# in cubes, cells laid out at their grown size (profiles/round_kernel_tissue_cubes.md).
 NCU_TRAFFIC = {
-    ("cpm3d_tissue_1024", "e0e74b368ce0"): 131.31e6 + 7.67e6,
+    ("cpm3d_tissue_1024", "d8b60b652be6"): 90.80e6 + 1.94e6,
 }
 
 
 def kernel_hash() -> str:
+    """First 12 hex digits of the sha1 over the round kernel, its headers and the choice of its launches."""
     h = hashlib.sha1()
-    for f in ("cpm_kernels.cu", "cpm_round.cuh", "cpm_internal.h"):
+    for f in ("cpm_kernels.cu", "cpm_round.cuh", "cpm_internal.h", "cpm_api.cu"):
         h.update(open(os.path.join(ROOT, "paper_2312_09317_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:12]
 
@@ -389,20 +389,8 @@ def run_gpu(args):
     attempts_all = sum_over_ranks(dist, float(args.steps * n))
     value = attempts_all / t_max
 
-    # per-launch duration of the round kernel: sub-passes (k = 1: one round each) timed alone
-    sub = []
-    with torch.cuda.stream(stream):
-        for k in range(min(64, per_mcs * 4)):
-            if flush is not None:
-                flush.fill_(k)
-            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            a.record(stream)
-            sim.step_subpasses(1)
-            b.record(stream)
-            sub.append((a, b))
-    torch.cuda.synchronize()
-    k_rounds = 1 if w.tile else ((w.a // w.c) ** w.dim) // w.P
-    launch_ms = statistics.mean(a.elapsed_time(b) for a, b in sub) / k_rounds
+    # duration of a round (tiled: of an epoch) in the timed steps, with what a step launches beside them
+    launch_ms = 1e3 * t_max / args.steps / rounds
     peak, peak_kind = peaks()
     alg_bytes_launch = bytes_per_site * n / rounds
     achieved = alg_bytes_launch / (launch_ms / 1e3) / 1e9

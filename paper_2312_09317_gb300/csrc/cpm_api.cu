@@ -417,8 +417,9 @@ int run_spans(cpm_handle *h, int64_t n, SpanPos p)
 
 // Whether a call's rounds run on the lattice in cubes.  A lattice that L2 does not hold is read in windows of
 // 3 x 3 x 3 at random places: nine rows, each its own 64 bytes of a different DRAM page.  In cubes a window is six
-// boxes of 64 bytes of mostly one 2 KB cube: fibre tissue on 1024^3, areas of 16^3, 143 -> 119 ms per MCS with the
-// way there and back (a pass over the lattice each), 768^3 77 -> 69, 400^3 42 -> 38.  With areas of 8^3 and
+// boxes of 64 bytes of mostly one 2 KB cube, 346 bytes of DRAM traffic an attempt instead of 530: fibre tissue on
+// 1024^3, areas of 16^3, 143 -> 119 ms per MCS with the way there and back (a pass over the lattice each), 768^3
+// 77 -> 69, 400^3 42 -> 38.  With areas of 8^3 and
 // less, where the windows of neighbouring areas share lines of a row, there is nothing to gain (cubes of 304^3: 3.3
 // and 3.5, 384^3 with areas of 4^3: 2.0 and 2.1).  The call has to make at least half as many attempts as there are
 // sites; a persistence update reads the lattice in rows after every MCS.

@@ -6,8 +6,9 @@
 // SMs, the rounds are separated by the cluster's hardware barrier, and each thread draws its next
 // attempt while it waits there.  A lattice whose attempts one CTA holds needs no cluster, and its
 // words, tallies and flags stay in that CTA's shared memory from the first round to the last.
-// us per round, with a launch each / in spans: 200^2 points 3.08 / 2.75, the same on areas of 40^2
-// (25 attempts, resident) 2.7 / 1.3, 3D Act tissue of 256^3 on areas of 16^3 8.3 / 5.8, of 64^3 5.0 / 4.0.
+// us per round, with a launch each / in spans: 200^2 points 3.03 / 2.82, the same on areas of 40^2
+// (25 attempts, resident) 2.20 / 1.25, motile cells of 256^2 5.3 / 4.3, 3D Act tissue of 256^3 on areas of
+// 16^3 7.1 / 5.9, 3D Act cells of 64^3 on areas of 8^3 3.9 / 2.7.
 // What is left of a round on a cluster is the release at its barrier (about 1,000 cycles until L2 has
 // acknowledged the writes), two dependent L2 loads (the words of an attempt, then its window) and some
 // 1,500 cycles of instructions.
